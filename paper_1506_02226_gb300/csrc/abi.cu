@@ -85,21 +85,26 @@ size_t layout(DbWork &w, const dbscan_opts &o, char *base) {
         w.occ_cap = 0;
     }
     if (o.max_d >= 16) {
-        // one more 256-row tile than n needs: the FP16 count's column list leaves
-        // a gap of up to 255 rows between its even-norm and odd-norm points
-        const int64_t np = (n + 255) / 256 * 256 + 256;
+        const int64_t np = (n + 255) / 256 * 256 + 256, nt = np / 256;
         w.tc_cap_pad = np;
         w.v16 = c.take<int16_t>((size_t)n * 64);
-        w.inorm = c.take<int32_t>(n);
         w.opAll = c.take<uint16_t>((size_t)np * 128);
-        w.opCore = c.take<uint16_t>((size_t)np * 128);
-        w.opNon = c.take<uint16_t>((size_t)np * 128);
+        w.opCore = c.take<uint16_t>((size_t)np * 64);
+        w.opNon = c.take<uint16_t>((size_t)np * 64);
         w.metaAll = c.take<char>((size_t)np * 16);
         w.metaCore = c.take<char>((size_t)np * 16);
         w.metaNon = c.take<char>((size_t)np * 16);
         w.list_a = c.take<int32_t>(np);
         w.list_b = c.take<int32_t>(n);
         w.tc_lens = c.take<int32_t>(8);
+        w.tc_hist = c.take<int32_t>(8192);
+        w.tc_tag = c.take<int32_t>(nt);
+        w.tc_rowneed = c.take<int32_t>(nt);
+        w.tc_udone = c.take<int32_t>(2 * nt);
+        w.tc_cbeta = c.take<float>(2 * nt);
+        w.tc_crad = c.take<float>(2 * nt);
+        const int64_t ntp = std::min<int64_t>(nt, (int64_t(1) << 17) + 1);  // all-pairs runs take up to 2^25 points
+        w.tc_pairs = c.take<uint32_t>((size_t)ntp * ((ntp + 31) / 32));
     } else {
         w.tc_cap_pad = 0;
     }
@@ -201,16 +206,16 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
             path = DBSCAN_PATH_ALLPAIRS_TC;
             const bool stall = plan->test_hook == DBSCAN_HOOK_TC_STALL;
             plan->test_hook = DBSCAN_HOOK_NONE;  // consumed by this run
-            err = launch_allpairs_tc(plan->w, points, n, d, Tc, min_pts, o.precision == DBSCAN_PREC_BF16_GRAM, stall,
-                                     st);
+            err = launch_allpairs_tc(plan->w, points, n, d, Tc, min_pts, exact, o.precision == DBSCAN_PREC_BF16_GRAM,
+                                     stall, labels, counts_out, core_out, st);
         } else {
             const int dp = dp_for(d);
             if (dp < 0) return DBSCAN_ERR_UNSUPPORTED;
             path = DBSCAN_PATH_ALLPAIRS_SIMT;
             err = launch_prep_dense(plan->w, points, n, d, dp, st);
             if (!err) err = launch_allpairs_simt(plan->w, n, d, dp, Tc, min_pts, exact, st);
+            if (!err) err = launch_labels_allpairs(plan->w, n, labels, counts_out, core_out, st);
         }
-        if (!err) err = launch_labels_allpairs(plan->w, n, labels, counts_out, core_out, st);
     }
     if (!err && o.label_mode == DBSCAN_LABEL_COMPACT) err = launch_compact(plan->w, n, labels, st);
     if (!err && stats && (path == DBSCAN_PATH_GRID || path == DBSCAN_PATH_GRID_PROJECTED))

@@ -153,18 +153,23 @@ __device__ __forceinline__ unsigned lanemask_lt() {
 // Starts kern on st as a programmatic dependent of the previous kernel in st
 // (kern must call db::wait_prior_grid() before its first memory access).
 template <typename... P, typename... A>
-inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A &&...args) {
+inline cudaError_t launch_dependent_smem(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                         A &&...args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, A &&...args) {
+    return launch_dependent_smem(kern, grid, block, 0, st, std::forward<A>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -235,14 +240,16 @@ struct DbWork {
     int32_t noff_cap;
     // tensor-core path (max_d >= 16)
     int64_t tc_cap_pad;     // rows of each packed operand (cap_n rounded up to 256, plus 256)
-    int16_t *v16;           // centred units v = u - 512 by point index, row stride 64
-    int32_t *inorm;         // exact |v|^2 [cap_n]
-    uint16_t *opAll, *opCore, *opNon;  // packed FP16 or two-term BF16 operand tiles [tc_cap_pad * 128]
-    void *metaAll, *metaCore, *metaNon;  // per-point metadata blocks (16 B per row)
-    int32_t *list_a, *list_b;  // core / non-core index lists [tc_cap_pad], [cap_n]
-    // [0] cores, [1] non-cores, [2] all, [3] largest |v|^2, [4] even-norm points,
-    // [5] length of the FP16 count's column list (even points, gap, odd points)
-    int32_t *tc_lens;
+    int16_t *v16;           // centred units by position, row stride K (BF16 recheck, verification) [cap_n * 64]
+    uint16_t *opAll;        // packed operand tiles: FP16 with the folded chunk, or two BF16 terms [tc_cap_pad * 128]
+    uint16_t *opCore, *opNon;  // FP16 tiles of the points before ordering; pivots, then ball centres [tc_cap_pad * 64]
+    void *metaAll, *metaCore, *metaNon;  // per-tile metadata: all, core points only, border rows only (16 B per point)
+    int32_t *list_a, *list_b;  // point of each position [tc_cap_pad], position of each point [cap_n]
+    int32_t *tc_lens;       // [0] largest |v|^2
+    int32_t *tc_hist;       // buckets of the order [8192]
+    int32_t *tc_tag, *tc_rowneed, *tc_udone;  // per tile: common root of its core points, border rows; per unit
+    float *tc_cbeta, *tc_crad;  // per ball (two a tile): |c|^2 of its centre, largest squared distance to it
+    uint32_t *tc_pairs;     // tile pairs that may hold neighbours (bits) [tiles][ceil(tiles / 32)]
     PhaseMarks *marks;      // host-side timing marks of the owning plan
     // second stream of the grid path: independent kernels run beside each
     // other (fork/join by events); unused while per-kernel marks are taken
@@ -263,9 +270,9 @@ struct GridGeom {
 cudaError_t launch_prep_dense(const DbWork &w, const float *x, int64_t n, int32_t d, int32_t dp, cudaStream_t st);
 cudaError_t launch_allpairs_simt(const DbWork &w, int64_t n, int32_t d, int32_t dp, int64_t Tc, int32_t min_pts,
                                  bool exact_counts, cudaStream_t st);
-cudaError_t launch_core_init(const DbWork &w, int64_t n, int32_t min_pts, cudaStream_t st);
 cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n, int32_t d, int64_t Tc, int32_t min_pts,
-                               bool bf16, bool stall, cudaStream_t st);
+                               bool exact, bool bf16, bool stall, int32_t *labels, int32_t *counts_out,
+                               uint8_t *core_out, cudaStream_t st);
 cudaError_t launch_tc_verify(const DbWork &w, const float *x, int64_t n, int32_t d, int64_t Tc, bool bf16,
                              cudaStream_t st);
 cudaError_t launch_labels_allpairs(const DbWork &w, int64_t n, int32_t *labels, int32_t *counts_out,
