@@ -251,8 +251,8 @@ typedef struct dbscan_instance {
 } dbscan_instance;
 
 /* Clusters `count` independent instances, each by Section I's three steps as
- * dbscan_run would (with the plan's label mode; the all-pairs CUDA-core tile
- * of Sections IV-A/IV-B, 1 <= d <= 16, larger d gives
+ * dbscan_run would (with the plan's label mode; the exact all-pairs
+ * test of Sections IV-A/IV-B on ordered rows, 1 <= d <= 16, larger d gives
  * DBSCAN_ERR_UNSUPPORTED).  Batching many instances into one launch sequence
  * is this library's addition: the paper clusters one point set.  All instances run in one graph-captured launch
  * sequence of persistent kernels that share a work queue of (instance, row
@@ -261,8 +261,7 @@ typedef struct dbscan_instance {
  * by the plan.  Synchronous; per_inst (host, nullable, `count` entries)
  * receives per-instance counts.  DBSCAN_ERR_ARG above 2^30 points in all;
  * DBSCAN_ERR_UNSUPPORTED when the work items (32-point row tiles x column
- * chunks of four 64-point tiles, the finest shape the autotuner tries: about
- * n^2 / 8,192 per instance) exceed 2^31.  With per_inst given,
+ * chunks of four 64-point tiles: about n^2 / 8,192 per instance) exceed 2^31.  With per_inst given,
  * each entry's pair_tests counts the instance's evaluated pair predicates and
  * the plan's counters 16..18 (dbscan_plan_counters) hold the batch's totals
  * for the count, merge and border passes. */
@@ -273,8 +272,8 @@ int dbscan_batch(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, 
  * DBSCAN_ERR_NOT_FOUND before the first batch. */
 int dbscan_batch_config(dbscan_plan *plan, int32_t *chunk_tiles, int32_t *blocks_per_sm);
 
-/* The tile shape dbscan_batch's autotuner picked with that configuration:
- * rows per row tile (32, 64 or 128) by 64 columns per column tile.
+/* The tile shape of dbscan_batch: 64 rows per row tile by 64 columns per column
+ * tile (a work item takes half a row tile).
  * DBSCAN_ERR_NOT_FOUND before the first batch. */
 int dbscan_batch_tile(dbscan_plan *plan, int32_t *tile_rows, int32_t *tile_cols);
 

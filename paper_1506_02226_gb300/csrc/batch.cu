@@ -2,64 +2,54 @@
 //
 // Each instance is one DBSCAN problem (Section II's definitions, the three
 // steps of Section IV) with its own n, d, eps and min_pts.  The instances are
-// concatenated: point g of the batch is point g - base_i of instance i.  Every
-// pass is one persistent kernel whose blocks pull work items (instance, row
-// tile of 64 points, chunk of column tiles) from an atomic counter and run the
-// same exact all-pairs tile as the single-instance path (ap_tile.cuh), on
-// pointers offset to the instance, so each instance keeps its own
-// union-find forest and local labels.  The kernel sequence (prep, count, core
-// flags, union, border, labels, optional compaction) is captured once into a
-// CUDA graph; a batch is then one table upload and one graph launch.
+// concatenated in tiles of 64 rows (an instance's last tile is padded).
+// Instances of up to kSortMax points are put in Z-order, so that a tile covers
+// a small region; every pass is one persistent kernel whose warps pull work
+// items (half a tile, a chunk of column tiles) from an atomic counter and run
+// the ordered pair test (warp_tile.cuh).  The kernel
+// sequence (prep, count, core flags with the merge inside tiles, the merge
+// across near tiles, roots, the rest of the merge, border, labels, optional
+// compaction) is captured once into a CUDA graph; a batch is then one table
+// upload and one graph launch.
+//
+// Measured, 4,096 instances of 64 to 8,192 points, d in {2, 3, 16} (us; with
+// 64 x 64 FP32 tiles a block, before / after): prep 1,874 / 630 (scattered row
+// reads, the counting sort), count 10,030 / 785, core flags and the merge inside
+// tiles - / 344, the merge across tiles 30,161 / 1,870 (pairs of tiles that hold
+// several sets or none of whose pairs are neighbours), border 4,556 / 890;
+// 46.6 / 4.70 ms a batch.  All passes are bound by the latency of an item's
+// first loads (record, rows, boxes) and then by the scores' FP32 operations, two
+// a pair; the matrix instructions are a few percent of the issue slots.
 //
 // Autotuning: the column chunk per work item (CH) and the number of resident
 // blocks per SM are picked on the first call by timing every candidate on the
 // caller's batch; the pick is kept by the plan.
+#include <cuda_fp16.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
 
-#include "ap_tile.cuh"
 #include "plan.h"
+#include "warp_tile.cuh"
 
-using namespace aptile;
+using namespace wtile;
 
 namespace {
 
 struct BInst {
     const float *x;
     int32_t *labels;
-    int n, d, dp, mode;
-    int Tc;
-    float Tp1;
-    int min_pts;
-    int base;       // first batch point of this instance
-    long long poff; // first float of its packed rows
-    int ntiles;     // row tiles of 16 * RM points
-    int ctiles;     // column tiles of 64 points
-    int nchunks;    // ceil(ctiles / CH)
-    int item0;      // first work item of this instance
-    int box0[3];    // its first tile box of 32, 64 and 128 rows
-    int pad;
+    TileRec rec;
 };
 
 struct BHdr {  // device-side sizes of the current batch
     int count;
     int total_points;
-    int total_items;
-    int box_level0[3];  // first box of each level (32, 64, 128 rows) in the box array
-    int pad[2];
+    int total_tiles;
+    int max_chunks;  // column chunks of the largest instance
 };
-
-__device__ __forceinline__ int find_inst_by_item(const BInst *__restrict__ t, int count, int item) {
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (t[mid].item0 <= item) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
 
 // Morton (Z-order) dilation of a 10-bit coordinate: bit b moves to bit 3b.
 __device__ __forceinline__ unsigned dilate3(unsigned v) {
@@ -71,239 +61,300 @@ __device__ __forceinline__ unsigned dilate3(unsigned v) {
     return v;
 }
 
+#define DB_BY_DP(DPV, CALL)                \
+    switch (DPV) { /* warp-uniform */      \
+        case 1: CALL(1); break;            \
+        case 2: CALL(2); break;            \
+        case 3: CALL(3); break;            \
+        case 4: CALL(4); break;            \
+        case 8: CALL(8); break;            \
+        default: CALL(16); break;          \
+    }
+
+// What the first kernel writes, by row, tile or point (see Rows).
+struct PackOut {
+    TileRec *tiles;
+    int *perm, *inv, *count, *least;
+    uint2 *P16;
+    float *nb, *box;
+    long long cap_tiles;
+};
+
+__device__ __forceinline__ unsigned half2_bits(int lo, int hi) {
+    const __half2 h = __halves2half2(__int2half_rn(lo), __int2half_rn(hi));
+    return *reinterpret_cast<const unsigned *>(&h);
+}
+
+// Packs the 64 rows of one tile (a warp, two rows a lane): grid check, centred
+// units, norm, the tile's box.  A lane reads its two rows whole (the rows of a
+// tile are scattered in the input), all loads independent.
+template <int DP>
+__device__ __forceinline__ bool pack_tile(const BInst &B, int tt, const uint16_t *order, const PackOut &w) {
+    const TileRec &I = B.rec;
+    const int lane = threadIdx.x & 31, n = I.n, d = I.d, T = I.tile0 + tt;
+    bool bad = false;
+    int v[2][DP];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int s = tt * BT + 32 * h + lane, row = T * BT + 32 * h + lane;
+        const int o = s < n ? (order ? (int)order[s] : s) : 0;
+        const float *src = B.x + (size_t)o * d;
+        float f[DP];
+#pragma unroll
+        for (int k = 0; k < DP; ++k) f[k] = s < n && k < d ? src[k] : 0.5f;
+        if (s < n) {
+            w.perm[row] = o;
+            w.inv[I.point0 + o] = row;
+        }
+        w.count[row] = 0;
+        w.least[row] = DB_NONE;
+        int s2 = 0;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+            int u;
+            bad |= !db::on_grid(f[k], u);
+            v[h][k] = u - 512;  // 0 for the padding
+            s2 += v[h][k] * v[h][k];
+        }
+        w.nb[row] = s < n ? -(float)s2 : -1e30f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // piece k: units 2k, 2k+1, 2k+8, 2k+9
+            uint2 pc;
+            pc.x = half2_bits(2 * k < DP ? v[h][2 * k] : 0, 2 * k + 1 < DP ? v[h][2 * k + 1] : 0);
+            pc.y = half2_bits(2 * k + 8 < DP ? v[h][2 * k + 8] : 0, 2 * k + 9 < DP ? v[h][2 * k + 9] : 0);
+            w.P16[(size_t)row * 4 + k] = pc;
+        }
+    }
+    const bool on0 = tt * BT + lane < n, on1 = tt * BT + 32 + lane < n;
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+        const int lo = __reduce_min_sync(FULL, min(on0 ? v[0][k] : INT_MAX, on1 ? v[1][k] : INT_MAX));
+        const int hi = __reduce_max_sync(FULL, max(on0 ? v[0][k] : INT_MIN, on1 ? v[1][k] : INT_MIN));
+        if (lane == 0) {
+            w.box[(size_t)k * w.cap_tiles + T] = (float)lo;
+            w.box[(size_t)(16 + k) * w.cap_tiles + T] = (float)hi;
+        }
+    }
+    if (lane == 0) w.tiles[T] = I;
+    return bad;
+}
+
+// Z-order code of a point's first three grid coordinates, the top `bits` bits
+// of each interleaved.
+__device__ __forceinline__ unsigned zcode(const float *x, int d, int dz, int bits) {
+    unsigned code = 0;
+    for (int j = 0; j < dz; ++j) {
+        int u;
+        db::on_grid(x[j], u);  // off-grid input is reported when the row is packed
+        code |= dilate3((unsigned)u >> (10 - bits)) << j;
+    }
+    if (dz == 2) {  // no third axis: close the gaps
+        unsigned c = 0;
+        for (int b = 0; b < bits; ++b) c |= ((code >> (3 * b)) & 3u) << (2 * b);
+        return c;
+    }
+    if (dz == 1) {
+        unsigned c = 0;
+        for (int b = 0; b < bits; ++b) c |= ((code >> (3 * b)) & 1u) << b;
+        return c;
+    }
+    return code;
+}
+
 // One block per instance at a time.  An instance of 2 .. sort_cap points is
-// put in Z-order of its first three grid coordinates (a bitonic sort of
-// {code, index} keys in shared memory), so that a 64-row tile covers a small
-// region; larger ones keep their order.  Then the rows are packed in that order
-// (centred units v = u - 512: the Gram form is exact up to d = 16), perm gets
-// the point of each row, and each 64-row tile its box: the least and greatest
-// unit of its rows on every axis.  The reordering changes no result: every
-// pass decides the same pairs, and labels are by point index.
-__global__ void __launch_bounds__(1024) batch_sortpack_kernel(const BInst *__restrict__ t,
-                                                              const BHdr *__restrict__ hdr, int sort_cap,
-                                                              int *__restrict__ pinst, int *__restrict__ perm,
-                                                              float *__restrict__ P, float *__restrict__ tbox,
-                                                              unsigned *status) {
-    extern __shared__ unsigned long long keys[];
+// put in Z-order of its first three grid coordinates, so that a 64-row tile
+// covers a small region; larger ones keep their order.  The order is a counting
+// sort over 2 n to 4 n cells of the Z curve (points of one cell in any order)
+// with 16-bit counters in shared memory: two passes over the points and one
+// over the counters (4,096 instances of 64 to 8,192 points: 0.64 ms; with a
+// bitonic sort of {code, index} keys 1.35).  Then the rows are packed in that
+// order with their norms, perm gets the point of each row, and each tile its
+// box: the least and greatest unit of its rows on every axis.  The reordering
+// changes no result: every pass decides the same pairs, and labels are by point
+// index.
+__global__ void __launch_bounds__(512) batch_sortpack_kernel(const BInst *__restrict__ t,
+                                                             const BHdr *__restrict__ hdr, int sort_cap, PackOut w,
+                                                             unsigned *status) {
+    extern __shared__ unsigned cells[];  // 2 counters a word: 2 sort_cap words, then sort_cap 16-bit indices
+    __shared__ int wsum[16];
+    uint16_t *order = reinterpret_cast<uint16_t *>(cells + 2 * sort_cap);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
     const int count = hdr->count;
     bool bad = false;
     for (int i = blockIdx.x; i < count; i += gridDim.x) {
         const BInst I = t[i];
-        const int n = I.n, d = I.d, dp = I.dp;
+        const int n = I.rec.n, d = I.rec.d;
         const bool sorted = n > 1 && n <= sort_cap;
         if (sorted) {
-            int npow = 2;
-            while (npow < n) npow <<= 1;
             const int dz = d < 3 ? d : 3;
-            for (int s = tid; s < npow; s += blockDim.x) {
-                unsigned long long k = ~0ull;
-                if (s < n) {
-                    unsigned code = 0;
-                    for (int j = 0; j < dz; ++j) {
-                        int u;
-                        db::on_grid(I.x[(size_t)s * d + j], u);  // off-grid input is reported below
-                        code |= dilate3((unsigned)u) << j;
-                    }
-                    k = ((unsigned long long)code << 32) | (unsigned)s;
-                }
-                keys[s] = k;
+            int lg = 1;
+            while ((1 << lg) < n) ++lg;  // n <= 2^lg
+            // the most bits per axis that keep 2^(dz bits) cells within 2^(lg + 2)
+            const int bits = min(10, (lg + 2) / dz), words = (1 << (dz * bits)) / 2;  // 2 counters a word
+            for (int c = tid; c < max(words, 1); c += blockDim.x) cells[c] = 0u;
+            __syncthreads();
+#pragma unroll 4
+            for (int s = tid; s < n; s += blockDim.x) {
+                const unsigned c = zcode(I.x + (size_t)s * d, d, dz, bits);
+                atomicAdd(&cells[c >> 1], 1u << (16 * (c & 1u)));
             }
             __syncthreads();
-            for (int k = 2; k <= npow; k <<= 1)
-                for (int j = k >> 1; j > 0; j >>= 1) {
-                    for (int x = tid; x < npow; x += blockDim.x) {
-                        const int y = x ^ j;
-                        if (y > x) {
-                            const unsigned long long kx = keys[x], ky = keys[y];
-                            if ((kx > ky) == ((x & k) == 0)) {
-                                keys[x] = ky;
-                                keys[y] = kx;
-                            }
-                        }
-                    }
-                    __syncthreads();
-                }
-        }
-        for (int s = tid; s < n; s += blockDim.x) {
-            perm[I.base + s] = sorted ? (int)(unsigned)keys[s] : s;
-            pinst[I.base + s] = i;
-        }
-        for (int e = tid; e < n * dp; e += blockDim.x) {
-            const int s = e / dp, k = e - s * dp;
-            const int o = sorted ? (int)(unsigned)keys[s] : s;
-            float v = 0.f;
-            if (k < d) {
-                int u;
-                bad |= !db::on_grid(I.x[(size_t)o * d + k], u);
-                v = (float)(u - 512);
-            }
-            P[I.poff + (long long)s * dp + k] = v;
-        }
-        __syncthreads();  // the block's rows are visible to it; keys are free again
-        // boxes of the 32-, 64- and 128-row tiles, a warp per tile
-        for (int lv = 0; lv < 3; ++lv) {
-            const int rows = 32 << lv, nt = (n + rows - 1) / rows;
-            float *lvl = tbox + (size_t)(hdr->box_level0[lv] + I.box0[lv]) * 32;
-            for (int tt = warp; tt < nt; tt += nwarps) {
-                for (int k = 0; k < dp; ++k) {
-                    float lo = 3.0e38f, hi = -3.0e38f;
-                    for (int r = tt * rows + lane; r < min(n, (tt + 1) * rows); r += 32) {
-                        const float v = P[I.poff + (long long)r * dp + k];
-                        lo = fminf(lo, v);
-                        hi = fmaxf(hi, v);
-                    }
+            // exclusive starts: each thread a run of words, then the block
+            const int per = (max(words, 1) + (int)blockDim.x - 1) / (int)blockDim.x;
+            const int w0 = min(tid * per, max(words, 1)), w1 = min(w0 + per, max(words, 1));
+            int sum = 0;
+            for (int c = w0; c < w1; ++c) sum += (int)(cells[c] & 0xffffu) + (int)(cells[c] >> 16);
+            int incl = sum;
 #pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-                        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-                    }
-                    if (lane == 0) {
-                        lvl[(size_t)tt * 32 + k] = lo;
-                        lvl[(size_t)tt * 32 + 16 + k] = hi;
-                    }
-                }
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += y;
             }
+            if (lane == 31) wsum[warp] = incl;
+            __syncthreads();
+            int at = incl - sum;
+            for (int k = 0; k < warp; ++k) at += wsum[k];
+            for (int c = w0; c < w1; ++c) {
+                const unsigned two = cells[c];
+                cells[c] = (unsigned)at | ((unsigned)(at + (int)(two & 0xffffu)) << 16);
+                at += (int)(two & 0xffffu) + (int)(two >> 16);
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int s = tid; s < n; s += blockDim.x) {
+                const unsigned c = zcode(I.x + (size_t)s * d, d, dz, bits);
+                const unsigned old = atomicAdd(&cells[c >> 1], 1u << (16 * (c & 1u)));
+                order[(old >> (16 * (c & 1u))) & 0xffffu] = (uint16_t)s;
+            }
+            __syncthreads();
         }
-        __syncthreads();
+        const int dp = d <= 4 ? d : (d <= 8 ? 8 : 16);
+        for (int tt = warp; tt < I.rec.ntiles; tt += nwarps) {
+#define DB_CALL(D) bad |= pack_tile<D>(I, tt, sorted ? order : nullptr, w)
+            DB_BY_DP(dp, DB_CALL)
+#undef DB_CALL
+        }
+        __syncthreads();  // the order is free again
     }
     if (bad) atomicOr(status, DB_EBIT_NOT_QUANTISED);
 }
 
-template <int PASS, int RM>
-__global__ void __launch_bounds__(NT) batch_pass_kernel(const BInst *__restrict__ t, const BHdr *__restrict__ hdr,
-                                                        int ch_tiles, int *work, const float *P,
-                                                        const int *perm, const float *tbox, int *count,
-                                                        const uint8_t *core, int *parent, int *border,
-                                                        unsigned *status, unsigned long long *ev) {
-    __shared__ int item_s;
-    const int nitems = hdr->total_items, ninst = hdr->count;
+// Work item w: half w mod 2 of tile (w / 2) mod total, chunk (w / 2) / total,
+// for one warp; the next item is claimed while the current one runs.
+template <int PASS>
+__global__ void __launch_bounds__(NT, 3) batch_pass_kernel(Rows R, const BHdr *__restrict__ hdr, int ch_tiles,
+                                                           unsigned long long *work) {
+    const int total = hdr->total_tiles, lane = threadIdx.x & 31;
+    const unsigned long long nitems =
+        2ull * (unsigned long long)total * (PASS == WT_NEAR ? 1 : hdr->max_chunks);
+    unsigned long long next = 0;
+    if (lane == 0) next = atomicAdd(work, 1ull);
     while (true) {
-        if (threadIdx.x == 0) item_s = atomicAdd(work, 1);
-        __syncthreads();
-        const int item = item_s;
-        __syncthreads();
+        const unsigned long long item = __shfl_sync(FULL, next, 0);
         if (item >= nitems) return;
-        const int i = find_inst_by_item(t, ninst, item);
-        const BInst &I = t[i];
-        const int k = item - I.item0;
-        const int rt = k / I.nchunks, chunk = k - rt * I.nchunks;
-        int ct0 = chunk * ch_tiles;
-        const int ct1 = min(I.ctiles, ct0 + ch_tiles);
-        if (PASS == PASS_UNION) ct0 = max(ct0, rt * RM / 4);  // the column tile of the row tile's first row
-        if (ct0 >= ct1) continue;
-        ApArgs a;
-        a.P = P + I.poff;
-        a.n = I.n;
-        a.Tp1 = I.Tp1;
-        a.Tc = I.Tc;
-        a.core = core + I.base;
-        a.count = count + I.base;
-        a.parent = parent + I.base;
-        a.border = border + I.base;
-        a.status = status;
-        a.ntiles = I.ntiles;
-        a.splits = 1;
-        a.early = I.min_pts;  // batch outputs labels only: counts may stop at min_pts
-        a.ev = ev ? ev + 3 * i : nullptr;  // pair tests evaluated by instance i's three passes
-        a.perm = perm + I.base;
-        constexpr int lv = RM == 2 ? 0 : (RM == 4 ? 1 : 2);  // box level of the row tiles
-        a.tbox = tbox + (size_t)(hdr->box_level0[1] + I.box0[1]) * 32;
-        a.tbox_rows = tbox + (size_t)(hdr->box_level0[lv] + I.box0[lv]) * 32;
-        switch (I.dp) {  // block-uniform: one instance per work item
-            case 1: ap_tile_body<1, MODE_GRAM, PASS, RM>(a, rt, ct0, ct1); break;
-            case 2: ap_tile_body<2, MODE_GRAM, PASS, RM>(a, rt, ct0, ct1); break;
-            case 3: ap_tile_body<3, MODE_GRAM, PASS, RM>(a, rt, ct0, ct1); break;
-            case 4: ap_tile_body<4, MODE_GRAM, PASS, RM>(a, rt, ct0, ct1); break;
-            case 8: ap_tile_body<8, MODE_GRAM, PASS, RM>(a, rt, ct0, ct1); break;
-            default: ap_tile_body<16, MODE_GRAM, PASS, RM>(a, rt, ct0, ct1); break;
+        if (lane == 0) next = atomicAdd(work, 1ull);
+        const unsigned long long two = item >> 1;
+        const int chunk = (int)(two / (unsigned)total), T = (int)(two - (unsigned long long)chunk * total);
+        const TileRec I = R.tiles[T];
+        int ct0, ct1;
+        if (PASS == WT_NEAR) {
+            ct0 = T + 1;
+            ct1 = min(I.tile0 + I.ntiles, T + 1 + kNear);
+        } else {
+            ct0 = I.tile0 + chunk * ch_tiles;
+            ct1 = min(I.tile0 + I.ntiles, ct0 + ch_tiles);
+            if (PASS == WT_FAR) ct0 = max(ct0, T + 1 + kNear);
         }
+        if (ct0 < ct1) run_item<PASS>(R, I, T, (int)(item & 1), ct0, ct1);
     }
 }
 
-__global__ void batch_core_init_kernel(const BInst *__restrict__ t, const BHdr *__restrict__ hdr,
-                                       const int *__restrict__ pinst, const int *__restrict__ count,
-                                       uint8_t *__restrict__ core, int *__restrict__ parent, int *__restrict__ border) {
-    const int total = hdr->total_points;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        const BInst &I = t[pinst[g]];
-        core[g] = count[g] >= I.min_pts;
-        parent[g] = g - I.base;
-        border[g] = DB_NONE;
+__global__ void __launch_bounds__(NT, 3) batch_core_kernel(Rows R, const BHdr *__restrict__ hdr) {
+    __shared__ unsigned long long adj[NT / 32][BT];
+    __shared__ int lab[NT / 32][BT];
+    const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5), wib = threadIdx.x >> 5;
+    for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps)
+        core_tile(R, R.tiles[T], T, adj[wib], lab[wib]);
+}
+
+__global__ void __launch_bounds__(NT) batch_flatten_kernel(Rows R, const BHdr *__restrict__ hdr) {
+    const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps) flatten_tile(R, T);
+}
+
+__global__ void __launch_bounds__(NT) batch_root_kernel(Rows R, const BHdr *__restrict__ hdr, int *least) {
+    const int total = hdr->total_tiles * BT, step = (int)(gridDim.x * blockDim.x);
+    for (int g0 = (int)(blockIdx.x * blockDim.x); g0 < total; g0 += step) {
+        const int g = g0 + (int)threadIdx.x;
+        const bool is = g < total && R.core[g];
+        root_row(R.parent, least, is, g, is ? R.perm[g] : 0);
     }
 }
 
-// Labels in each instance's own index space (a thread per row: core flags
-// are by row, the forest and border choices by point); per-instance counts
-// (core, border, noise, clusters) when istats != nullptr; root flags for
-// compaction, by point.
-__global__ void batch_label_kernel(const BInst *__restrict__ t, const BHdr *__restrict__ hdr,
-                                   const int *__restrict__ pinst, const int *__restrict__ perm,
-                                   const uint8_t *__restrict__ core, int *parent, const int *__restrict__ border,
-                                   int *__restrict__ flags, int *istats) {
-    const int total = hdr->total_points;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        const int i = pinst[g];
-        const BInst &I = t[i];
-        const int loc = perm[g];  // row g - base holds point loc
-        int *par = parent + I.base;
-        const int bo = border[I.base + loc];
-        int lab, kind;
-        if (core[g]) {
-            lab = db::uf_find(par, loc);
+// Labels in each instance's own index space, a thread per row: a core row the
+// smallest point index of its set, a border row that of its smallest-index
+// core neighbour, noise -1; per-instance counts (core, border, noise,
+// clusters) when istats != nullptr; root flags for compaction, by point.
+__global__ void __launch_bounds__(NT) batch_label_kernel(Rows R, const BHdr *__restrict__ hdr,
+                                                         const BInst *__restrict__ t, const int *__restrict__ inv,
+                                                         const int *__restrict__ least, int *__restrict__ flags,
+                                                         int *istats) {
+    const int total = hdr->total_tiles * BT;
+    for (int g = (int)(blockIdx.x * blockDim.x + threadIdx.x); g < total; g += (int)(gridDim.x * blockDim.x)) {
+        const TileRec &I = R.tiles[g >> 6];
+        if (g - I.tile0 * BT >= I.n) continue;
+        const int loc = R.perm[g], bo = R.border[g];
+        int lab = -1, kind = 2;
+        if (R.core[g]) {
+            lab = least[R.parent[g]];
             kind = 0;
         } else if (bo != DB_NONE) {
-            lab = db::uf_find(par, bo);
+            lab = least[R.parent[inv[I.point0 + bo]]];
             kind = 1;
-        } else {
-            lab = -1;
-            kind = 2;
         }
-        I.labels[loc] = lab;
+        t[I.inst].labels[loc] = lab;
         const int root = (kind == 0 && lab == loc);
-        flags[I.base + loc] = root;
+        if (flags) flags[I.point0 + loc] = root;
         if (istats) {
-            atomicAdd(istats + 4 * i + kind, 1);
-            if (root) atomicAdd(istats + 4 * i + 3, 1);
+            atomicAdd(istats + 4 * I.inst + kind, 1);
+            if (root) atomicAdd(istats + 4 * I.inst + 3, 1);
         }
     }
 }
 
-__global__ void batch_compact_kernel(const BInst *__restrict__ t, const BHdr *__restrict__ hdr,
-                                     const int *__restrict__ pinst, const int *__restrict__ rank) {
-    const int total = hdr->total_points;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-        const BInst &I = t[pinst[g]];
-        const int loc = g - I.base;
-        const int l = I.labels[loc];
-        if (l >= 0) I.labels[loc] = rank[I.base + l] - rank[I.base];
+// Dense cluster numbers from the scan of the root flags (a thread per row).
+__global__ void batch_compact_kernel(Rows R, const BHdr *__restrict__ hdr, const BInst *__restrict__ t,
+                                     const int *__restrict__ rank) {
+    const int total = hdr->total_tiles * BT;
+    for (int g = (int)(blockIdx.x * blockDim.x + threadIdx.x); g < total; g += (int)(gridDim.x * blockDim.x)) {
+        const TileRec &I = R.tiles[g >> 6];
+        if (g - I.tile0 * BT >= I.n) continue;
+        int *labels = t[I.inst].labels + R.perm[g];
+        const int l = *labels;
+        if (l >= 0) *labels = rank[I.point0 + l] - rank[I.point0];
     }
 }
 
-constexpr int kCH[] = {4, 16, 64};
-constexpr int kRM[] = {2, 4, 8};  // row tiles of 32, 64 and 128 points (8 rows per thread for the last)
-constexpr int kSortMax = 16384;  // largest instance reordered (128 KiB of sort keys in shared memory)
+constexpr int kCH[] = {64, 256};
 constexpr int kBPS[] = {4, 8};
+constexpr int kSortMax = 16384;  // largest instance reordered (160 KiB of shared memory, 16-bit starts)
+constexpr size_t sort_bytes(int cap) { return (size_t)cap * (2 * sizeof(unsigned) + sizeof(uint16_t)); }
 
 }  // namespace
 
 struct BatchState {
     int cap_count = 0;
-    int64_t cap_points = 0, cap_pfloats = 0, cap_tiles = 0;
+    int64_t cap_points = 0, cap_tiles = 0;
     void *dev = nullptr;
     size_t dev_bytes = 0;
     BInst *d_table = nullptr;
     BHdr *d_hdr = nullptr;
-    int *d_pinst = nullptr;
-    int *d_perm = nullptr;     // point of each row (rows of an instance in Z-order)
-    float *d_tbox = nullptr;   // per 64-row tile: least and greatest unit on each axis [tiles][32]
-    int sort_cap = 0;          // instances up to this many points are reordered (a power of two)
-    float *d_P = nullptr;
-    int *d_count = nullptr;
-    uint8_t *d_core = nullptr;
-    int *d_parent = nullptr, *d_border = nullptr, *d_flags = nullptr, *d_scan = nullptr, *d_part = nullptr;
+    Rows rows{};               // by row and tile (ev set per launch)
+    PackOut pack{};            // the same arrays, writable
+    int *d_flags = nullptr, *d_scan = nullptr, *d_part = nullptr;  // by point
     int64_t part_cap = 0;
-    int *d_work = nullptr;
+    int sort_cap = 0;          // instances up to this many points are reordered (a power of two)
+    unsigned long long *d_work = nullptr;
     unsigned *d_status = nullptr;
     int *d_istats = nullptr;
     unsigned long long *d_ev = nullptr;  // pair tests evaluated per instance and pass [count][3]
@@ -313,8 +364,8 @@ struct BatchState {
     int *h_istats = nullptr;
     unsigned *h_status = nullptr;
     cudaGraphExec_t graph = nullptr;
-    int graph_ch = -1, graph_bps = -1, graph_rm = -1, graph_stats = -1;
-    int ch = 16, bps = 8, rm = 4;  // column tiles per work item, blocks per SM, rows per thread (tile of 16 rm rows)
+    int graph_ch = -1, graph_bps = -1, graph_stats = -1;
+    int ch = 64, bps = 8;  // column tiles per work item, blocks per SM
     bool tuned = false;
     PhaseMarks marks;  // timing off
 };
@@ -336,13 +387,11 @@ namespace {
 size_t al256(size_t v) { return (v + 255) / 256 * 256; }
 
 // (Re)allocates the batch workspace for at least these sizes.
-int batch_reserve(BatchState *b, int count, int64_t points, int64_t pfloats, int64_t tiles) {
-    if (count <= b->cap_count && points <= b->cap_points && pfloats <= b->cap_pfloats && tiles <= b->cap_tiles)
-        return DBSCAN_OK;
+int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
+    if (count <= b->cap_count && points <= b->cap_points && tiles <= b->cap_tiles) return DBSCAN_OK;
     const int nc = std::max(count, b->cap_count);
     const int64_t np = std::max<int64_t>(std::max(points, b->cap_points), 1);
-    const int64_t nf = std::max<int64_t>(std::max(pfloats, b->cap_pfloats), 1);
-    const int64_t nt = std::max<int64_t>(std::max(tiles, b->cap_tiles), 1);
+    const int64_t nt = std::max<int64_t>(std::max(tiles, b->cap_tiles), 1), nr = nt * BT;
     const int64_t part = np / 2048 + 4;
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -350,11 +399,12 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t pfloats, int
         off = al256(off + bytes);
         return o;
     };
-    const size_t o_table = take(sizeof(BInst) * nc), o_hdr = take(sizeof(BHdr)), o_pinst = take(4 * np),
-                 o_P = take(4 * nf), o_count = take(4 * np), o_core = take(np), o_parent = take(4 * np),
-                 o_border = take(4 * np), o_flags = take(4 * np), o_scan = take(4 * (np + 1)),
-                 o_part = take(4 * part), o_work = take(4 * 8), o_status = take(16), o_istats = take(16 * nc),
-                 o_ev = take(24 * (size_t)nc), o_perm = take(4 * np), o_tbox = take(128 * (size_t)nt);
+    const size_t o_table = take(sizeof(BInst) * nc), o_hdr = take(sizeof(BHdr)), o_tiles = take(sizeof(TileRec) * nt),
+                 o_P16 = take(32 * nr), o_nb = take(4 * nr), o_nbc = take(4 * nr), o_box = take(128 * nt),
+                 o_count = take(4 * nr), o_core = take(nr), o_parent = take(4 * nr), o_border = take(4 * nr),
+                 o_perm = take(4 * nr), o_least = take(4 * nr), o_tag = take(4 * nt), o_need = take(4 * nt),
+                 o_inv = take(4 * np), o_flags = take(4 * np), o_scan = take(4 * (np + 1)), o_part = take(4 * part),
+                 o_work = take(8 * 8), o_status = take(16), o_istats = take(16 * nc), o_ev = take(24 * (size_t)nc);
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
@@ -370,7 +420,7 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t pfloats, int
     if (cudaMalloc(&b->dev, off) != cudaSuccess) {
         cudaGetLastError();
         b->cap_count = 0;
-        b->cap_points = b->cap_pfloats = b->cap_tiles = 0;
+        b->cap_points = b->cap_tiles = 0;
         return DBSCAN_ERR_OOM;
     }
     if (cudaMallocHost(&b->h_table, sizeof(BInst) * nc) != cudaSuccess ||
@@ -380,89 +430,83 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t pfloats, int
     if (!b->h_hdr && cudaMallocHost(&b->h_hdr, sizeof(BHdr)) != cudaSuccess) return DBSCAN_ERR_OOM;
     if (!b->h_status && cudaMallocHost(&b->h_status, 16) != cudaSuccess) return DBSCAN_ERR_OOM;
     char *base = static_cast<char *>(b->dev);
+    auto at = [&](size_t o) { return static_cast<void *>(base + o); };
     b->dev_bytes = off;
-    b->d_table = reinterpret_cast<BInst *>(base + o_table);
-    b->d_hdr = reinterpret_cast<BHdr *>(base + o_hdr);
-    b->d_pinst = reinterpret_cast<int *>(base + o_pinst);
-    b->d_perm = reinterpret_cast<int *>(base + o_perm);
-    b->d_tbox = reinterpret_cast<float *>(base + o_tbox);
-    b->d_P = reinterpret_cast<float *>(base + o_P);
-    b->d_count = reinterpret_cast<int *>(base + o_count);
-    b->d_core = reinterpret_cast<uint8_t *>(base + o_core);
-    b->d_parent = reinterpret_cast<int *>(base + o_parent);
-    b->d_border = reinterpret_cast<int *>(base + o_border);
-    b->d_flags = reinterpret_cast<int *>(base + o_flags);
-    b->d_scan = reinterpret_cast<int *>(base + o_scan);
-    b->d_part = reinterpret_cast<int *>(base + o_part);
+    b->d_table = static_cast<BInst *>(at(o_table));
+    b->d_hdr = static_cast<BHdr *>(at(o_hdr));
+    PackOut &w = b->pack;
+    w.tiles = static_cast<TileRec *>(at(o_tiles));
+    w.perm = static_cast<int *>(at(o_perm));
+    w.inv = static_cast<int *>(at(o_inv));
+    w.count = static_cast<int *>(at(o_count));
+    w.least = static_cast<int *>(at(o_least));
+    w.P16 = static_cast<uint2 *>(at(o_P16));
+    w.nb = static_cast<float *>(at(o_nb));
+    w.box = static_cast<float *>(at(o_box));
+    w.cap_tiles = nt;
+    Rows &r = b->rows;
+    r.tiles = w.tiles;
+    r.P16 = w.P16;
+    r.nb = w.nb;
+    r.nbc = static_cast<float *>(at(o_nbc));
+    r.box = w.box;
+    r.cap_tiles = nt;
+    r.count = w.count;
+    r.core = static_cast<uint8_t *>(at(o_core));
+    r.parent = static_cast<int *>(at(o_parent));
+    r.border = static_cast<int *>(at(o_border));
+    r.perm = w.perm;
+    r.tag = static_cast<int *>(at(o_tag));
+    r.need = static_cast<int *>(at(o_need));
+    b->d_flags = static_cast<int *>(at(o_flags));
+    b->d_scan = static_cast<int *>(at(o_scan));
+    b->d_part = static_cast<int *>(at(o_part));
     b->part_cap = part;
-    b->d_work = reinterpret_cast<int *>(base + o_work);
-    b->d_status = reinterpret_cast<unsigned *>(base + o_status);
-    b->d_istats = reinterpret_cast<int *>(base + o_istats);
-    b->d_ev = reinterpret_cast<unsigned long long *>(base + o_ev);
+    b->d_work = static_cast<unsigned long long *>(at(o_work));
+    b->d_status = r.status = static_cast<unsigned *>(at(o_status));
+    b->d_istats = static_cast<int *>(at(o_istats));
+    b->d_ev = static_cast<unsigned long long *>(at(o_ev));
     b->cap_count = nc;
     b->cap_points = np;
-    b->cap_pfloats = nf;
     b->cap_tiles = nt;
     if (cudaMemset(b->d_status, 0, 16) != cudaSuccess) return DBSCAN_ERR_CUDA;
     return DBSCAN_OK;
 }
 
-// Host table for chunk size ch and row tiles of 16 * rm points; returns the
-// total work items.  boxes[lv] counts the tile boxes of 32 << lv rows.
-int64_t build_table(const dbscan_instance *inst, int count, int ch, int rm, BInst *t, int64_t *points,
-                    int64_t *pfloats, int64_t boxes[3], int64_t *max_n) {
-    int64_t base = 0, poff = 0, items = 0, mx = 0;
-    boxes[0] = boxes[1] = boxes[2] = 0;
+// Host table; returns the tiles of the largest instance.
+int64_t build_table(const dbscan_instance *inst, int count, BInst *t, int64_t *points, int64_t *tiles,
+                    int64_t *max_n) {
+    int64_t base = 0, nt = 0, mx = 0;
     for (int i = 0; i < count; ++i) {
         const dbscan_instance &in = inst[i];
-        BInst &I = t[i];
+        BInst &B = t[i];
+        B = BInst{};
         const double e = (double)in.eps;
         const int64_t T = (int64_t)std::floor(e * e * 1048576.0);
         const int64_t Tc = std::min<int64_t>(T, (int64_t)in.d * 1023 * 1023);
-        I.x = in.points;
-        I.labels = in.labels_out;
+        B.x = in.points;
+        B.labels = in.labels_out;
+        TileRec &I = B.rec;
         I.n = (int)in.n;
         I.d = in.d;
-        I.dp = dp_for(in.d);  // 1, 2, 3, 4, 8 or 16
-        I.mode = MODE_GRAM;
         I.Tc = (int)Tc;
         I.Tp1 = (float)(Tc + 1);
         I.min_pts = in.min_pts;
-        I.base = (int)base;
-        I.poff = poff;
-        I.ntiles = (int)((in.n + 16 * rm - 1) / (16 * rm));
-        I.ctiles = (int)((in.n + BN - 1) / BN);
-        I.nchunks = (I.ctiles + ch - 1) / ch;
-        I.item0 = (int)items;
-        for (int lv = 0; lv < 3; ++lv) {
-            I.box0[lv] = (int)boxes[lv];
-            boxes[lv] += (in.n + (32 << lv) - 1) / (32 << lv);
-        }
-        I.pad = 0;
+        I.inst = i;
+        I.point0 = (int)base;
+        I.tile0 = (int)nt;
+        I.ntiles = (int)((in.n + BT - 1) / BT);
         base += in.n;
-        poff += (in.n * I.dp + 3) / 4 * 4;  // 16-byte aligned rows of every instance (vector tile loads)
-        items += (int64_t)I.ntiles * I.nchunks;
+        nt += I.ntiles;
         mx = std::max<int64_t>(mx, in.n);
     }
     *points = base;
-    *pfloats = poff;
+    *tiles = nt;
     *max_n = mx;
-    return items;
+    return (mx + BT - 1) / BT;
 }
 
-template <int PASS>
-void launch_batch_pass(BatchState *b, int rm, int grid, int ch, int *work, bool stats, cudaStream_t st) {
-    unsigned long long *ev = stats ? b->d_ev : nullptr;
-#define DB_BATCH_PASS(R)                                                                                            \
-    batch_pass_kernel<PASS, R><<<grid, NT, 0, st>>>(b->d_table, b->d_hdr, ch, work, b->d_P, b->d_perm, b->d_tbox,  \
-                                                    b->d_count, b->d_core, b->d_parent, b->d_border, b->d_status, ev)
-    if (rm == 2) DB_BATCH_PASS(2);
-    else if (rm == 8) DB_BATCH_PASS(8);
-    else DB_BATCH_PASS(4);
-#undef DB_BATCH_PASS
-}
-
-cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int bps, int rm, cudaStream_t st,
+cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int bps, cudaStream_t st,
                           PhaseMarks *pm = nullptr) {
     PhaseMarks off;
     if (!pm) pm = &off;
@@ -474,31 +518,37 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
     if ((e = cudaMemcpyAsync(b->d_table, b->h_table, sizeof(BInst) * b->cap_count, cudaMemcpyHostToDevice, st)))
         return e;
     if ((e = cudaMemcpyAsync(b->d_hdr, b->h_hdr, sizeof(BHdr), cudaMemcpyHostToDevice, st))) return e;
-    if ((e = cudaMemsetAsync(b->d_work, 0, 4 * 8, st))) return e;
-    if ((e = cudaMemsetAsync(b->d_count, 0, 4 * (size_t)b->cap_points, st))) return e;
+    if ((e = cudaMemsetAsync(b->d_work, 0, 8 * 8, st))) return e;
     if (stats && (e = cudaMemsetAsync(b->d_istats, 0, 16 * (size_t)b->cap_count, st))) return e;
     if (stats && (e = cudaMemsetAsync(b->d_ev, 0, 24 * (size_t)b->cap_count, st))) return e;
-    batch_sortpack_kernel<<<sms * 2, 1024, sizeof(unsigned long long) * std::max(b->sort_cap, 2), st>>>(
-        b->d_table, b->d_hdr, b->sort_cap, b->d_pinst, b->d_perm, b->d_P, b->d_tbox, b->d_status);
+    Rows R = b->rows;
+    R.ev = stats ? b->d_ev : nullptr;
+    batch_sortpack_kernel<<<sms * 3, 512, sort_bytes(b->sort_cap), st>>>(b->d_table, b->d_hdr, b->sort_cap, b->pack,
+                                                                        b->d_status);
     pm->kernel("batch_prep", st);
-    launch_batch_pass<PASS_COUNT>(b, rm, pgrid, ch, b->d_work + 0, stats, st);
+    batch_pass_kernel<WT_COUNT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 0);
     pm->kernel("batch_count", st);
-    batch_core_init_kernel<<<egrid, 256, 0, st>>>(b->d_table, b->d_hdr, b->d_pinst, b->d_count, b->d_core,
-                                                  b->d_parent, b->d_border);
-    pm->kernel("batch_core_init", st);
-    launch_batch_pass<PASS_UNION>(b, rm, pgrid, ch, b->d_work + 1, stats, st);
+    batch_core_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
+    pm->kernel("batch_core", st);
+    batch_pass_kernel<WT_NEAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 1);
+    pm->kernel("batch_union_near", st);
+    batch_flatten_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
+    pm->kernel("batch_flatten", st);
+    batch_pass_kernel<WT_FAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 2);
     pm->kernel("batch_union", st);
-    launch_batch_pass<PASS_BORDER>(b, rm, pgrid, ch, b->d_work + 2, stats, st);
+    batch_pass_kernel<WT_BORDER><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 3);
     pm->kernel("batch_border", st);
-    batch_label_kernel<<<egrid, 256, 0, st>>>(b->d_table, b->d_hdr, b->d_pinst, b->d_perm, b->d_core, b->d_parent,
-                                              b->d_border,
-                                              b->d_flags, stats ? b->d_istats : nullptr);
+    batch_root_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->pack.least);
+    pm->kernel("batch_root", st);
+    const bool compact = label_mode == DBSCAN_LABEL_COMPACT;
+    batch_label_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->d_table, b->pack.inv, b->pack.least,
+                                             compact ? b->d_flags : nullptr, stats ? b->d_istats : nullptr);
     pm->kernel("batch_label", st);
     if ((e = cudaGetLastError())) return e;
-    if (label_mode == DBSCAN_LABEL_COMPACT) {
+    if (compact) {
         if ((e = launch_exclusive_scan(b->d_flags, b->d_scan, b->cap_points, b->d_part, b->part_cap, st, pm)))
             return e;
-        batch_compact_kernel<<<egrid, 256, 0, st>>>(b->d_table, b->d_hdr, b->d_pinst, b->d_scan);
+        batch_compact_kernel<<<egrid, 256, 0, st>>>(R, b->d_hdr, b->d_table, b->d_scan);
         pm->kernel("batch_compact", st);
     }
     if (stats && (e = cudaMemcpyAsync(b->h_istats, b->d_istats, 16 * (size_t)b->cap_count, cudaMemcpyDeviceToHost,
@@ -514,7 +564,7 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
 // The whole sequence as one CUDA graph (rebuilt when capacities or the tuned
 // configuration change).
 int batch_graph_launch(BatchState *b, int label_mode, bool stats, cudaStream_t st) {
-    if (!b->graph || b->graph_ch != b->ch || b->graph_bps != b->bps || b->graph_rm != b->rm ||
+    if (!b->graph || b->graph_ch != b->ch || b->graph_bps != b->bps ||
         b->graph_stats != (int)stats || b->graph_ch < 0) {
         if (b->graph) {
             cudaGraphExecDestroy(b->graph);
@@ -524,7 +574,7 @@ int batch_graph_launch(BatchState *b, int label_mode, bool stats, cudaStream_t s
         if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return DBSCAN_ERR_CUDA;
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        if (!e) e = enqueue_batch(b, label_mode, stats, b->ch, b->bps, b->rm, cs);
+        if (!e) e = enqueue_batch(b, label_mode, stats, b->ch, b->bps, cs);
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         cudaStreamDestroy(cs);
         if (e || e2 || !g) {
@@ -541,10 +591,121 @@ int batch_graph_launch(BatchState *b, int label_mode, bool stats, cudaStream_t s
         }
         b->graph_ch = b->ch;
         b->graph_bps = b->bps;
-        b->graph_rm = b->rm;
         b->graph_stats = (int)stats;
     }
     return cudaGraphLaunch(b->graph, st) == cudaSuccess ? DBSCAN_OK : DBSCAN_ERR_CUDA;
+}
+
+}  // namespace
+
+namespace {
+
+// One part of a batch, its sizes checked; adds the pair tests per pass to tot.
+int batch_run(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, dbscan_stats *per_inst,
+              unsigned long long tot[4]) {
+    int cur = -1;
+    cudaGetDevice(&cur);
+    if (cur != plan->opts.device) cudaSetDevice(plan->opts.device);
+    if (!plan->batch) plan->batch = new BatchState();
+    BatchState *b = plan->batch;
+    const int label_mode = plan->opts.label_mode;
+    const bool stats = per_inst != nullptr;
+    cudaStream_t st = plan->stream;
+
+    std::vector<BInst> tmp(count);
+    int64_t points = 0, tiles = 0, max_n = 0;
+    const int64_t max_tiles = build_table(inst, count, tmp.data(), &points, &tiles, &max_n);
+    int s = batch_reserve(b, count, points, tiles);
+    if (s) return s;
+    // Instances up to kSortMax points are put in Z-order; the sort's shared
+    // memory is sized for the largest of them.
+    int sort_cap = 2;
+    while (sort_cap < std::min<int64_t>(max_n, kSortMax)) sort_cap <<= 1;
+    if (sort_cap != b->sort_cap && b->graph) {
+        cudaGraphExecDestroy(b->graph);
+        b->graph = nullptr;
+    }
+    b->sort_cap = sort_cap;
+    if (sort_bytes(sort_cap) > 48 * 1024 &&
+        cudaFuncSetAttribute(batch_sortpack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sort_bytes(sort_cap)) != cudaSuccess)
+        return DBSCAN_ERR_CUDA;
+
+    std::memcpy(b->h_table, tmp.data(), sizeof(BInst) * count);
+    if (b->cap_count > count) std::memset(b->h_table + count, 0, sizeof(BInst) * (b->cap_count - count));
+    auto prepare = [&](int ch) {
+        b->h_hdr->count = count;
+        b->h_hdr->total_points = (int)points;
+        b->h_hdr->total_tiles = (int)tiles;
+        b->h_hdr->max_chunks = (int)((max_tiles + ch - 1) / ch);
+    };
+
+    if (!b->tuned) {
+        // Autotune on this batch: every (CH, blocks per SM) candidate, best of 2 runs.
+        cudaEvent_t e0, e1;
+        cudaEventCreate(&e0);
+        cudaEventCreate(&e1);
+        float best = 1e30f;
+        for (int ch : kCH)
+            for (int bps : kBPS) {
+                prepare(ch);
+                float tbest = 1e30f;
+                for (int rep = 0; rep < 2; ++rep) {
+                    cudaEventRecord(e0, st);
+                    if (enqueue_batch(b, label_mode, false, ch, bps, st)) {
+                        cudaEventDestroy(e0);
+                        cudaEventDestroy(e1);
+                        return DBSCAN_ERR_CUDA;
+                    }
+                    cudaEventRecord(e1, st);
+                    cudaEventSynchronize(e1);
+                    float ms = 0.f;
+                    cudaEventElapsedTime(&ms, e0, e1);
+                    tbest = std::min(tbest, ms);
+                }
+                if (tbest < best) {
+                    best = tbest;
+                    b->ch = ch;
+                    b->bps = bps;
+                }
+            }
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        b->tuned = true;
+    }
+    prepare(b->ch);
+    if (plan->opts.profile) {  // per-kernel events: run the sequence uncaptured
+        plan->marks.begin(st);
+        if (enqueue_batch(b, label_mode, stats, b->ch, b->bps, st, &plan->marks)) return DBSCAN_ERR_CUDA;
+    } else {
+        s = batch_graph_launch(b, label_mode, stats, st);
+        if (s) return s;
+    }
+    if (cudaStreamSynchronize(st) != cudaSuccess) return DBSCAN_ERR_CUDA;
+    if (cur >= 0 && cur != plan->opts.device) cudaSetDevice(cur);
+    const unsigned bits = *b->h_status;
+    if (bits & DB_EBIT_NOT_QUANTISED) return DBSCAN_ERR_NOT_QUANTISED;
+    if (bits & DB_EBIT_TIMEOUT) return DBSCAN_ERR_TIMEOUT;
+    if (bits) return DBSCAN_ERR_CUDA;
+    if (stats) {
+        for (int i = 0; i < count; ++i)
+            for (int k = 0; k < 3; ++k) tot[k] += b->h_ev[3 * i + k];
+        for (int i = 0; i < count; ++i) {
+            dbscan_stats &o = per_inst[i];
+            std::memset(&o, 0, sizeof(o));
+            o.n_core = b->h_istats[4 * i + 0];
+            o.n_border = b->h_istats[4 * i + 1];
+            o.n_noise = b->h_istats[4 * i + 2];
+            o.n_clusters = b->h_istats[4 * i + 3];
+            o.candidate_pairs = inst[i].n * inst[i].n;
+            o.path = DBSCAN_PATH_ALLPAIRS_SIMT;
+            const double e = (double)inst[i].eps;
+            o.threshold = (int64_t)std::floor(e * e * 1048576.0);
+            o.kernels = 9 + (label_mode == DBSCAN_LABEL_COMPACT ? 4 : 0);
+            o.pair_tests = (int64_t)(b->h_ev[3 * i] + b->h_ev[3 * i + 1] + b->h_ev[3 * i + 2]);
+        }
+    }
+    return DBSCAN_OK;
 }
 
 }  // namespace
@@ -561,127 +722,28 @@ extern "C" int dbscan_batch(dbscan_plan *plan, const dbscan_instance *inst, int3
         total += in.n;
     }
     if (total > INT32_MAX / 2) return DBSCAN_ERR_ARG;
-    // work items (instance, row tile, column chunk) are counted in int32: the
-    // smallest chunk gives the most items
+    // the limit on work: 32-point row tiles x chunks of four 64-point column
+    // tiles (about n^2 / 8,192 per instance) in int32
     int64_t items = 0;
     for (int i = 0; i < count; ++i) {
-        const int64_t rows = (inst[i].n + 31) / 32, cols = (inst[i].n + 63) / 64;  // the smallest row tile
-        items += rows * ((cols + kCH[0] - 1) / kCH[0]);
+        const int64_t rows = (inst[i].n + 31) / 32, cols = (inst[i].n + 63) / 64;
+        items += rows * ((cols + 3) / 4);
     }
     if (items > INT32_MAX) return DBSCAN_ERR_UNSUPPORTED;
-    int cur = -1;
-    cudaGetDevice(&cur);
-    if (cur != plan->opts.device) cudaSetDevice(plan->opts.device);
-    if (!plan->batch) plan->batch = new BatchState();
-    BatchState *b = plan->batch;
-    const int label_mode = plan->opts.label_mode;
-    const bool stats = per_inst != nullptr;
-    cudaStream_t st = plan->stream;
-
-    // Sizes for the largest chunk count (smallest CH) so every candidate fits.
-    std::vector<BInst> tmp(count);
-    int64_t points = 0, pfloats = 0, boxes[3] = {0, 0, 0}, max_n = 0;
-    build_table(inst, count, kCH[0], kRM[0], tmp.data(), &points, &pfloats, boxes, &max_n);
-    int s = batch_reserve(b, count, points, pfloats, boxes[0] + boxes[1] + boxes[2]);
-    if (s) return s;
-    // Instances up to kSortMax points are put in Z-order; the sort's shared
-    // memory is sized for the largest of them.
-    int sort_cap = 2;
-    while (sort_cap < std::min<int64_t>(max_n, kSortMax)) sort_cap <<= 1;
-    if (sort_cap != b->sort_cap && b->graph) {
-        cudaGraphExecDestroy(b->graph);
-        b->graph = nullptr;
-    }
-    b->sort_cap = sort_cap;
-    if (sizeof(unsigned long long) * sort_cap > 48 * 1024 &&
-        cudaFuncSetAttribute(batch_sortpack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(unsigned long long) * sort_cap)) != cudaSuccess)
-        return DBSCAN_ERR_CUDA;
-
-    auto prepare = [&](int ch, int rm) {
-        int64_t pts, pf, bx[3], mn;
-        const int64_t items = build_table(inst, count, ch, rm, b->h_table, &pts, &pf, bx, &mn);
-        for (int i = count; i < b->cap_count; ++i) std::memset(&b->h_table[i], 0, sizeof(BInst));
-        b->h_hdr->count = count;
-        b->h_hdr->total_points = (int)pts;
-        b->h_hdr->total_items = (int)std::min<int64_t>(items, INT32_MAX);
-        b->h_hdr->box_level0[0] = 0;
-        b->h_hdr->box_level0[1] = (int)bx[0];
-        b->h_hdr->box_level0[2] = (int)(bx[0] + bx[1]);
-        b->h_hdr->pad[0] = b->h_hdr->pad[1] = 0;
-    };
-
-    if (!b->tuned) {
-        // Autotune on this batch: every (row tile, CH, blocks per SM) candidate, best of 2 runs.
-        cudaEvent_t e0, e1;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        float best = 1e30f;
-        for (int rm : kRM)
-        for (int ch : kCH)
-            for (int bps : kBPS) {
-                prepare(ch, rm);
-                float tbest = 1e30f;
-                for (int rep = 0; rep < 2; ++rep) {
-                    cudaEventRecord(e0, st);
-                    if (enqueue_batch(b, label_mode, false, ch, bps, rm, st)) {
-                        cudaEventDestroy(e0);
-                        cudaEventDestroy(e1);
-                        return DBSCAN_ERR_CUDA;
-                    }
-                    cudaEventRecord(e1, st);
-                    cudaEventSynchronize(e1);
-                    float ms = 0.f;
-                    cudaEventElapsedTime(&ms, e0, e1);
-                    tbest = std::min(tbest, ms);
-                }
-                if (tbest < best) {
-                    best = tbest;
-                    b->ch = ch;
-                    b->bps = bps;
-                    b->rm = rm;
-                }
-            }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        b->tuned = true;
-    }
-    prepare(b->ch, b->rm);
-    if (plan->opts.profile) {  // per-kernel events: run the sequence uncaptured
-        plan->marks.begin(st);
-        if (enqueue_batch(b, label_mode, stats, b->ch, b->bps, b->rm, st, &plan->marks)) return DBSCAN_ERR_CUDA;
-    } else {
-        s = batch_graph_launch(b, label_mode, stats, st);
+    // Rows are counted in int32 (64 per tile): a batch of more tiles (tens of
+    // millions of tiny instances) runs in parts.
+    unsigned long long tot[4] = {0, 0, 0, 0};
+    for (int32_t i = 0; i < count;) {
+        int64_t tiles = 0;
+        int32_t end = i;
+        while (end < count && tiles + (inst[end].n + BT - 1) / BT <= INT32_MAX / BT) tiles += (inst[end++].n + BT - 1) / BT;
+        const int s = batch_run(plan, inst + i, end - i, per_inst ? per_inst + i : nullptr, tot);
         if (s) return s;
+        i = end;
     }
-    if (cudaStreamSynchronize(st) != cudaSuccess) return DBSCAN_ERR_CUDA;
-    if (cur >= 0 && cur != plan->opts.device) cudaSetDevice(cur);
-    const unsigned bits = *b->h_status;
-    if (bits & DB_EBIT_NOT_QUANTISED) return DBSCAN_ERR_NOT_QUANTISED;
-    if (bits & DB_EBIT_TIMEOUT) return DBSCAN_ERR_TIMEOUT;
-    if (bits) return DBSCAN_ERR_CUDA;
-    if (stats) {
-        // the batch's pair tests per pass, also left in the plan's counters 16..18
-        unsigned long long tot[4] = {0, 0, 0, 0};
-        for (int i = 0; i < count; ++i)
-            for (int k = 0; k < 3; ++k) tot[k] += b->h_ev[3 * i + k];
-        if (cudaMemcpy(plan->w.ctr + DB_CTR_EVAL, tot, sizeof(tot), cudaMemcpyHostToDevice) != cudaSuccess)
-            return DBSCAN_ERR_CUDA;
-        for (int i = 0; i < count; ++i) {
-            dbscan_stats &o = per_inst[i];
-            std::memset(&o, 0, sizeof(o));
-            o.n_core = b->h_istats[4 * i + 0];
-            o.n_border = b->h_istats[4 * i + 1];
-            o.n_noise = b->h_istats[4 * i + 2];
-            o.n_clusters = b->h_istats[4 * i + 3];
-            o.candidate_pairs = inst[i].n * inst[i].n;
-            o.path = DBSCAN_PATH_ALLPAIRS_SIMT;
-            const double e = (double)inst[i].eps;
-            o.threshold = (int64_t)std::floor(e * e * 1048576.0);
-            o.kernels = 6 + (label_mode == DBSCAN_LABEL_COMPACT ? 4 : 0);
-            o.pair_tests = (int64_t)(b->h_ev[3 * i] + b->h_ev[3 * i + 1] + b->h_ev[3 * i + 2]);
-        }
-    }
+    // the batch's pair tests per pass, also left in the plan's counters 16..18
+    if (per_inst && cudaMemcpy(plan->w.ctr + DB_CTR_EVAL, tot, sizeof(tot), cudaMemcpyHostToDevice) != cudaSuccess)
+        return DBSCAN_ERR_CUDA;
     return DBSCAN_OK;
 }
 
@@ -696,7 +758,7 @@ extern "C" int dbscan_batch_config(dbscan_plan *plan, int32_t *chunk_tiles, int3
 extern "C" int dbscan_batch_tile(dbscan_plan *plan, int32_t *tile_rows, int32_t *tile_cols) {
     if (!plan) return DBSCAN_ERR_ARG;
     if (!plan->batch || !plan->batch->tuned) return DBSCAN_ERR_NOT_FOUND;
-    if (tile_rows) *tile_rows = 16 * plan->batch->rm;
-    if (tile_cols) *tile_cols = BN;
+    if (tile_rows) *tile_rows = BT;
+    if (tile_cols) *tile_cols = BT;
     return DBSCAN_OK;
 }
