@@ -64,7 +64,8 @@ extern "C" {
 #define DBSCAN_ERR_NOT_FOUND 8     /* unknown serve job id */
 
 /* Pair-test arithmetic. */
-#define DBSCAN_PREC_AUTO 0       /* tensor-core FP16 Gram for d >= 16 all-pairs, SIMT otherwise */
+#define DBSCAN_PREC_AUTO 0       /* all pairs: tensor-core FP16 Gram for d >= 16 (from 4,096 points), below that the
+                                    SIMT path, for d <= 16 on ordered rows with exact FP16 dot products */
 #define DBSCAN_PREC_EXACT_SIMT 1 /* FP32/INT32 CUDA-core pair test, exact by construction */
 #define DBSCAN_PREC_FP16_GRAM 2  /* tcgen05 FP16 Gram product, exact by proof (band 0) */
 #define DBSCAN_PREC_BF16_GRAM 3  /* tcgen05 BF16 Gram product (two-term split) + exact recheck of the band */
@@ -82,7 +83,7 @@ extern "C" {
 /* Which path a run took (dbscan_stats.path). */
 #define DBSCAN_PATH_NONE 0
 #define DBSCAN_PATH_GRID 1
-#define DBSCAN_PATH_ALLPAIRS_SIMT 2
+#define DBSCAN_PATH_ALLPAIRS_SIMT 2 /* per-warp pair tests: CUDA cores, or (PREC_AUTO, d <= 16) mma.sync */
 #define DBSCAN_PATH_ALLPAIRS_TC 3
 #define DBSCAN_PATH_GRID_PROJECTED 4 /* 4 <= d <= 8: cells of the first three coordinates, full-d test */
 #define DBSCAN_PATH_PAPER 5          /* dbscan_run_paper: the paper's materialised matrices */

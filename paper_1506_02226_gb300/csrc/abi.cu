@@ -34,8 +34,9 @@ struct Carver {
     }
 };
 
-// Lays the workspace out (base == nullptr: just measures it).
-size_t layout(DbWork &w, const dbscan_opts &o, char *base) {
+// Lays the workspace out (base == nullptr: just measures it).  exact_d: o.max_d
+// is the only dimension served (a plan's is an upper bound).
+size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
     Carver c{base};
     const int64_t n = std::max<int64_t>(o.max_n, 1);
     w.cap_n = n;
@@ -108,6 +109,9 @@ size_t layout(DbWork &w, const dbscan_opts &o, char *base) {
     } else {
         w.tc_cap_pad = 0;
     }
+    // warp tiles: all-pairs runs of d <= 16, none at d <= 3 with a grid (the eps-grid always applies there)
+    const bool wt = o.precision == DBSCAN_PREC_AUTO && (!grid || o.max_d > 3) && !(exact_d && o.max_d > 16);
+    w.wt = wt ? c.take<char>(wt_bytes(n)) : nullptr;
     return align_up(c.off, 256);
 }
 
@@ -208,6 +212,9 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
             plan->test_hook = DBSCAN_HOOK_NONE;  // consumed by this run
             err = launch_allpairs_tc(plan->w, points, n, d, Tc, min_pts, exact, o.precision == DBSCAN_PREC_BF16_GRAM,
                                      stall, labels, counts_out, core_out, st);
+        } else if (d <= 16 && o.precision == DBSCAN_PREC_AUTO && plan->w.wt) {
+            path = DBSCAN_PATH_ALLPAIRS_SIMT;
+            err = launch_allpairs_wt(plan->w, points, n, d, Tc, min_pts, exact, labels, counts_out, core_out, st);
         } else {
             const int dp = dp_for(d);
             if (dp < 0) return DBSCAN_ERR_UNSUPPORTED;
@@ -311,7 +318,7 @@ static dbscan_opts layout_opts(const dbscan_opts &o, int64_t n, int32_t d, bool 
 
 size_t plan_workspace_bytes_for(const dbscan_opts &o, int64_t n, int32_t d, bool exact_d) {
     DbWork w{};
-    return layout(w, layout_opts(o, n, d, exact_d), nullptr);
+    return layout(w, layout_opts(o, n, d, exact_d), exact_d, nullptr);
 }
 
 int plan_bind_workspace(dbscan_plan *p, void *base, size_t bytes, int64_t n, int32_t d, bool exact_d) {
@@ -322,7 +329,7 @@ int plan_bind_workspace(dbscan_plan *p, void *base, size_t bytes, int64_t n, int
     cudaStream_t side = p->w.side;
     cudaEvent_t fj[4] = {p->w.fj[0], p->w.fj[1], p->w.fj[2], p->w.fj[3]};
     DbWork w{};
-    layout(w, q, static_cast<char *>(base));
+    layout(w, q, exact_d, static_cast<char *>(base));
     w.marks = marks;
     w.side = side;
     for (int i = 0; i < 4; ++i) w.fj[i] = fj[i];

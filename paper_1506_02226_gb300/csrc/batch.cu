@@ -24,8 +24,6 @@
 // Autotuning: the column chunk per work item (CH) and the number of resident
 // blocks per SM are picked on the first call by timing every candidate on the
 // caller's batch; the pick is kept by the plan.
-#include <cuda_fp16.h>
-
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -44,123 +42,6 @@ struct BInst {
     TileRec rec;
 };
 
-struct BHdr {  // device-side sizes of the current batch
-    int count;
-    int total_points;
-    int total_tiles;
-    int max_chunks;  // column chunks of the largest instance
-};
-
-// Morton (Z-order) dilation of a 10-bit coordinate: bit b moves to bit 3b.
-__device__ __forceinline__ unsigned dilate3(unsigned v) {
-    v &= 1023u;
-    v = (v | (v << 16)) & 0x030000FFu;
-    v = (v | (v << 8)) & 0x0300F00Fu;
-    v = (v | (v << 4)) & 0x030C30C3u;
-    v = (v | (v << 2)) & 0x09249249u;
-    return v;
-}
-
-#define DB_BY_DP(DPV, CALL)                \
-    switch (DPV) { /* warp-uniform */      \
-        case 1: CALL(1); break;            \
-        case 2: CALL(2); break;            \
-        case 3: CALL(3); break;            \
-        case 4: CALL(4); break;            \
-        case 8: CALL(8); break;            \
-        default: CALL(16); break;          \
-    }
-
-// What the first kernel writes, by row, tile or point (see Rows).
-struct PackOut {
-    TileRec *tiles;
-    int *perm, *inv, *count, *least;
-    uint2 *P16;
-    float *nb, *box;
-    long long cap_tiles;
-};
-
-__device__ __forceinline__ unsigned half2_bits(int lo, int hi) {
-    const __half2 h = __halves2half2(__int2half_rn(lo), __int2half_rn(hi));
-    return *reinterpret_cast<const unsigned *>(&h);
-}
-
-// Packs the 64 rows of one tile (a warp, two rows a lane): grid check, centred
-// units, norm, the tile's box.  A lane reads its two rows whole (the rows of a
-// tile are scattered in the input), all loads independent.
-template <int DP>
-__device__ __forceinline__ bool pack_tile(const BInst &B, int tt, const uint16_t *order, const PackOut &w) {
-    const TileRec &I = B.rec;
-    const int lane = threadIdx.x & 31, n = I.n, d = I.d, T = I.tile0 + tt;
-    bool bad = false;
-    int v[2][DP];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int s = tt * BT + 32 * h + lane, row = T * BT + 32 * h + lane;
-        const int o = s < n ? (order ? (int)order[s] : s) : 0;
-        const float *src = B.x + (size_t)o * d;
-        float f[DP];
-#pragma unroll
-        for (int k = 0; k < DP; ++k) f[k] = s < n && k < d ? src[k] : 0.5f;
-        if (s < n) {
-            w.perm[row] = o;
-            w.inv[I.point0 + o] = row;
-        }
-        w.count[row] = 0;
-        w.least[row] = DB_NONE;
-        int s2 = 0;
-#pragma unroll
-        for (int k = 0; k < DP; ++k) {
-            int u;
-            bad |= !db::on_grid(f[k], u);
-            v[h][k] = u - 512;  // 0 for the padding
-            s2 += v[h][k] * v[h][k];
-        }
-        w.nb[row] = s < n ? -(float)s2 : -1e30f;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {  // piece k: units 2k, 2k+1, 2k+8, 2k+9
-            uint2 pc;
-            pc.x = half2_bits(2 * k < DP ? v[h][2 * k] : 0, 2 * k + 1 < DP ? v[h][2 * k + 1] : 0);
-            pc.y = half2_bits(2 * k + 8 < DP ? v[h][2 * k + 8] : 0, 2 * k + 9 < DP ? v[h][2 * k + 9] : 0);
-            w.P16[(size_t)row * 4 + k] = pc;
-        }
-    }
-    const bool on0 = tt * BT + lane < n, on1 = tt * BT + 32 + lane < n;
-#pragma unroll
-    for (int k = 0; k < DP; ++k) {
-        const int lo = __reduce_min_sync(FULL, min(on0 ? v[0][k] : INT_MAX, on1 ? v[1][k] : INT_MAX));
-        const int hi = __reduce_max_sync(FULL, max(on0 ? v[0][k] : INT_MIN, on1 ? v[1][k] : INT_MIN));
-        if (lane == 0) {
-            w.box[(size_t)k * w.cap_tiles + T] = (float)lo;
-            w.box[(size_t)(16 + k) * w.cap_tiles + T] = (float)hi;
-        }
-    }
-    if (lane == 0) w.tiles[T] = I;
-    return bad;
-}
-
-// Z-order code of a point's first three grid coordinates, the top `bits` bits
-// of each interleaved.
-__device__ __forceinline__ unsigned zcode(const float *x, int d, int dz, int bits) {
-    unsigned code = 0;
-    for (int j = 0; j < dz; ++j) {
-        int u;
-        db::on_grid(x[j], u);  // off-grid input is reported when the row is packed
-        code |= dilate3((unsigned)u >> (10 - bits)) << j;
-    }
-    if (dz == 2) {  // no third axis: close the gaps
-        unsigned c = 0;
-        for (int b = 0; b < bits; ++b) c |= ((code >> (3 * b)) & 3u) << (2 * b);
-        return c;
-    }
-    if (dz == 1) {
-        unsigned c = 0;
-        for (int b = 0; b < bits; ++b) c |= ((code >> (3 * b)) & 1u) << b;
-        return c;
-    }
-    return code;
-}
-
 // One block per instance at a time.  An instance of 2 .. sort_cap points is
 // put in Z-order of its first three grid coordinates, so that a 64-row tile
 // covers a small region; larger ones keep their order.  The order is a counting
@@ -173,7 +54,7 @@ __device__ __forceinline__ unsigned zcode(const float *x, int d, int dz, int bit
 // changes no result: every pass decides the same pairs, and labels are by point
 // index.
 __global__ void __launch_bounds__(512) batch_sortpack_kernel(const BInst *__restrict__ t,
-                                                             const BHdr *__restrict__ hdr, int sort_cap, PackOut w,
+                                                             const Hdr *__restrict__ hdr, int sort_cap, PackOut w,
                                                              unsigned *status) {
     extern __shared__ unsigned cells[];  // 2 counters a word: 2 sort_cap words, then sort_cap 16-bit indices
     __shared__ int wsum[16];
@@ -195,7 +76,7 @@ __global__ void __launch_bounds__(512) batch_sortpack_kernel(const BInst *__rest
             __syncthreads();
 #pragma unroll 4
             for (int s = tid; s < n; s += blockDim.x) {
-                const unsigned c = zcode(I.x + (size_t)s * d, d, dz, bits);
+                const unsigned c = zcode(I.x + (size_t)s * d, dz, bits);
                 atomicAdd(&cells[c >> 1], 1u << (16 * (c & 1u)));
             }
             __syncthreads();
@@ -222,80 +103,24 @@ __global__ void __launch_bounds__(512) batch_sortpack_kernel(const BInst *__rest
             __syncthreads();
 #pragma unroll 4
             for (int s = tid; s < n; s += blockDim.x) {
-                const unsigned c = zcode(I.x + (size_t)s * d, d, dz, bits);
+                const unsigned c = zcode(I.x + (size_t)s * d, dz, bits);
                 const unsigned old = atomicAdd(&cells[c >> 1], 1u << (16 * (c & 1u)));
                 order[(old >> (16 * (c & 1u))) & 0xffffu] = (uint16_t)s;
             }
             __syncthreads();
         }
-        const int dp = d <= 4 ? d : (d <= 8 ? 8 : 16);
-        for (int tt = warp; tt < I.rec.ntiles; tt += nwarps) {
-#define DB_CALL(D) bad |= pack_tile<D>(I, tt, sorted ? order : nullptr, w)
-            DB_BY_DP(dp, DB_CALL)
-#undef DB_CALL
-        }
+        for (int tt = warp; tt < I.rec.ntiles; tt += nwarps)
+            bad |= pack_tile_d(I.x, I.rec, tt, sorted ? order : nullptr, w);
         __syncthreads();  // the order is free again
     }
     if (bad) atomicOr(status, DB_EBIT_NOT_QUANTISED);
-}
-
-// Work item w: half w mod 2 of tile (w / 2) mod total, chunk (w / 2) / total,
-// for one warp; the next item is claimed while the current one runs.
-template <int PASS>
-__global__ void __launch_bounds__(NT, 3) batch_pass_kernel(Rows R, const BHdr *__restrict__ hdr, int ch_tiles,
-                                                           unsigned long long *work) {
-    const int total = hdr->total_tiles, lane = threadIdx.x & 31;
-    const unsigned long long nitems =
-        2ull * (unsigned long long)total * (PASS == WT_NEAR ? 1 : hdr->max_chunks);
-    unsigned long long next = 0;
-    if (lane == 0) next = atomicAdd(work, 1ull);
-    while (true) {
-        const unsigned long long item = __shfl_sync(FULL, next, 0);
-        if (item >= nitems) return;
-        if (lane == 0) next = atomicAdd(work, 1ull);
-        const unsigned long long two = item >> 1;
-        const int chunk = (int)(two / (unsigned)total), T = (int)(two - (unsigned long long)chunk * total);
-        const TileRec I = R.tiles[T];
-        int ct0, ct1;
-        if (PASS == WT_NEAR) {
-            ct0 = T + 1;
-            ct1 = min(I.tile0 + I.ntiles, T + 1 + kNear);
-        } else {
-            ct0 = I.tile0 + chunk * ch_tiles;
-            ct1 = min(I.tile0 + I.ntiles, ct0 + ch_tiles);
-            if (PASS == WT_FAR) ct0 = max(ct0, T + 1 + kNear);
-        }
-        if (ct0 < ct1) run_item<PASS>(R, I, T, (int)(item & 1), ct0, ct1);
-    }
-}
-
-__global__ void __launch_bounds__(NT, 3) batch_core_kernel(Rows R, const BHdr *__restrict__ hdr) {
-    __shared__ unsigned long long adj[NT / 32][BT];
-    __shared__ int lab[NT / 32][BT];
-    const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5), wib = threadIdx.x >> 5;
-    for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps)
-        core_tile(R, R.tiles[T], T, adj[wib], lab[wib]);
-}
-
-__global__ void __launch_bounds__(NT) batch_flatten_kernel(Rows R, const BHdr *__restrict__ hdr) {
-    const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5);
-    for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps) flatten_tile(R, T);
-}
-
-__global__ void __launch_bounds__(NT) batch_root_kernel(Rows R, const BHdr *__restrict__ hdr, int *least) {
-    const int total = hdr->total_tiles * BT, step = (int)(gridDim.x * blockDim.x);
-    for (int g0 = (int)(blockIdx.x * blockDim.x); g0 < total; g0 += step) {
-        const int g = g0 + (int)threadIdx.x;
-        const bool is = g < total && R.core[g];
-        root_row(R.parent, least, is, g, is ? R.perm[g] : 0);
-    }
 }
 
 // Labels in each instance's own index space, a thread per row: a core row the
 // smallest point index of its set, a border row that of its smallest-index
 // core neighbour, noise -1; per-instance counts (core, border, noise,
 // clusters) when istats != nullptr; root flags for compaction, by point.
-__global__ void __launch_bounds__(NT) batch_label_kernel(Rows R, const BHdr *__restrict__ hdr,
+__global__ void __launch_bounds__(NT) batch_label_kernel(Rows R, const Hdr *__restrict__ hdr,
                                                          const BInst *__restrict__ t, const int *__restrict__ inv,
                                                          const int *__restrict__ least, int *__restrict__ flags,
                                                          int *istats) {
@@ -323,7 +148,7 @@ __global__ void __launch_bounds__(NT) batch_label_kernel(Rows R, const BHdr *__r
 }
 
 // Dense cluster numbers from the scan of the root flags (a thread per row).
-__global__ void batch_compact_kernel(Rows R, const BHdr *__restrict__ hdr, const BInst *__restrict__ t,
+__global__ void batch_compact_kernel(Rows R, const Hdr *__restrict__ hdr, const BInst *__restrict__ t,
                                      const int *__restrict__ rank) {
     const int total = hdr->total_tiles * BT;
     for (int g = (int)(blockIdx.x * blockDim.x + threadIdx.x); g < total; g += (int)(gridDim.x * blockDim.x)) {
@@ -348,7 +173,7 @@ struct BatchState {
     void *dev = nullptr;
     size_t dev_bytes = 0;
     BInst *d_table = nullptr;
-    BHdr *d_hdr = nullptr;
+    Hdr *d_hdr = nullptr;
     Rows rows{};               // by row and tile (ev set per launch)
     PackOut pack{};            // the same arrays, writable
     int *d_flags = nullptr, *d_scan = nullptr, *d_part = nullptr;  // by point
@@ -360,7 +185,7 @@ struct BatchState {
     unsigned long long *d_ev = nullptr;  // pair tests evaluated per instance and pass [count][3]
     unsigned long long *h_ev = nullptr;
     BInst *h_table = nullptr;
-    BHdr *h_hdr = nullptr;
+    Hdr *h_hdr = nullptr;
     int *h_istats = nullptr;
     unsigned *h_status = nullptr;
     cudaGraphExec_t graph = nullptr;
@@ -399,7 +224,7 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
         off = al256(off + bytes);
         return o;
     };
-    const size_t o_table = take(sizeof(BInst) * nc), o_hdr = take(sizeof(BHdr)), o_tiles = take(sizeof(TileRec) * nt),
+    const size_t o_table = take(sizeof(BInst) * nc), o_hdr = take(sizeof(Hdr)), o_tiles = take(sizeof(TileRec) * nt),
                  o_P16 = take(32 * nr), o_nb = take(4 * nr), o_nbc = take(4 * nr), o_box = take(128 * nt),
                  o_count = take(4 * nr), o_core = take(nr), o_parent = take(4 * nr), o_border = take(4 * nr),
                  o_perm = take(4 * nr), o_least = take(4 * nr), o_tag = take(4 * nt), o_need = take(4 * nt),
@@ -427,13 +252,13 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
         cudaMallocHost(&b->h_istats, 16 * (size_t)nc) != cudaSuccess ||
         cudaMallocHost(&b->h_ev, 24 * (size_t)nc) != cudaSuccess)
         return DBSCAN_ERR_OOM;
-    if (!b->h_hdr && cudaMallocHost(&b->h_hdr, sizeof(BHdr)) != cudaSuccess) return DBSCAN_ERR_OOM;
+    if (!b->h_hdr && cudaMallocHost(&b->h_hdr, sizeof(Hdr)) != cudaSuccess) return DBSCAN_ERR_OOM;
     if (!b->h_status && cudaMallocHost(&b->h_status, 16) != cudaSuccess) return DBSCAN_ERR_OOM;
     char *base = static_cast<char *>(b->dev);
     auto at = [&](size_t o) { return static_cast<void *>(base + o); };
     b->dev_bytes = off;
     b->d_table = static_cast<BInst *>(at(o_table));
-    b->d_hdr = static_cast<BHdr *>(at(o_hdr));
+    b->d_hdr = static_cast<Hdr *>(at(o_hdr));
     PackOut &w = b->pack;
     w.tiles = static_cast<TileRec *>(at(o_tiles));
     w.perm = static_cast<int *>(at(o_perm));
@@ -492,6 +317,7 @@ int64_t build_table(const dbscan_instance *inst, int count, BInst *t, int64_t *p
         I.Tc = (int)Tc;
         I.Tp1 = (float)(Tc + 1);
         I.min_pts = in.min_pts;
+        I.leave = in.min_pts;  // batch outputs labels only
         I.inst = i;
         I.point0 = (int)base;
         I.tile0 = (int)nt;
@@ -517,7 +343,7 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
     cudaError_t e;
     if ((e = cudaMemcpyAsync(b->d_table, b->h_table, sizeof(BInst) * b->cap_count, cudaMemcpyHostToDevice, st)))
         return e;
-    if ((e = cudaMemcpyAsync(b->d_hdr, b->h_hdr, sizeof(BHdr), cudaMemcpyHostToDevice, st))) return e;
+    if ((e = cudaMemcpyAsync(b->d_hdr, b->h_hdr, sizeof(Hdr), cudaMemcpyHostToDevice, st))) return e;
     if ((e = cudaMemsetAsync(b->d_work, 0, 8 * 8, st))) return e;
     if (stats && (e = cudaMemsetAsync(b->d_istats, 0, 16 * (size_t)b->cap_count, st))) return e;
     if (stats && (e = cudaMemsetAsync(b->d_ev, 0, 24 * (size_t)b->cap_count, st))) return e;
@@ -526,19 +352,19 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
     batch_sortpack_kernel<<<sms * 3, 512, sort_bytes(b->sort_cap), st>>>(b->d_table, b->d_hdr, b->sort_cap, b->pack,
                                                                         b->d_status);
     pm->kernel("batch_prep", st);
-    batch_pass_kernel<WT_COUNT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 0);
+    pass_kernel<WT_COUNT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 0);
     pm->kernel("batch_count", st);
-    batch_core_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
+    core_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
     pm->kernel("batch_core", st);
-    batch_pass_kernel<WT_NEAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 1);
+    pass_kernel<WT_NEAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 1);
     pm->kernel("batch_union_near", st);
-    batch_flatten_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
+    flatten_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
     pm->kernel("batch_flatten", st);
-    batch_pass_kernel<WT_FAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 2);
+    pass_kernel<WT_FAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 2);
     pm->kernel("batch_union", st);
-    batch_pass_kernel<WT_BORDER><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 3);
+    pass_kernel<WT_BORDER><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 3);
     pm->kernel("batch_border", st);
-    batch_root_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->pack.least);
+    root_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->pack.least);
     pm->kernel("batch_root", st);
     const bool compact = label_mode == DBSCAN_LABEL_COMPACT;
     batch_label_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->d_table, b->pack.inv, b->pack.least,

@@ -1510,35 +1510,6 @@ __global__ void __launch_bounds__(1024) tc_pivot_rank_kernel(const int *__restri
     prank[s[t] & 1023u] = t;
 }
 
-// Exclusive scan of the bucket sizes, in place, by one block.
-__global__ void __launch_bounds__(1024) tc_bucket_scan_kernel(int *__restrict__ hist, int nhist) {
-    db::wait_prior_grid();  // started as a programmatic dependent
-    db::allow_next_grid();
-    __shared__ int wt[32];
-    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    int v[8], s = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        v[k] = t * 8 + k < nhist ? hist[t * 8 + k] : 0;
-        s += v[k];
-    }
-    int xs = s;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(FULL, xs, o);
-        if (lane >= o) xs += y;
-    }
-    if (lane == 31) wt[wid] = xs;
-    __syncthreads();
-    int off = xs - s;
-    for (int w = 0; w < wid; ++w) off += wt[w];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        if (t * 8 + k < nhist) hist[t * 8 + k] = off;
-        off += v[k];
-    }
-}
-
 __global__ void tc_bucket_scatter_kernel(int n, const int *__restrict__ key, const int *__restrict__ rank,
                                          const int *__restrict__ start, int *__restrict__ list) {
     db::wait_prior_grid();  // started as a programmatic dependent
@@ -1824,7 +1795,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
         o.hist = hist;
         if ((e = launch_pass_t<TC_ORDER, false>(o, sms, st))) return e;
         w.marks->kernel("tc_order", st);
-        launch_dependent(tc_bucket_scan_kernel, 1, 1024, st, hist, nhist);
+        if ((e = launch_bucket_scan(hist, nhist, st))) return e;
         w.marks->kernel("tc_bucket_scan", st);
         launch_dependent(tc_bucket_scatter_kernel, (n + 255) / 256, 256, st, n, key, rank, hist, perm);
         w.marks->kernel("tc_bucket_scatter", st);

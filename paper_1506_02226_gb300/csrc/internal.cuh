@@ -250,6 +250,7 @@ struct DbWork {
     int32_t *tc_tag, *tc_rowneed, *tc_udone;  // per tile: common root of its core points, border rows; per unit
     float *tc_cbeta, *tc_crad;  // per ball (two a tile): |c|^2 of its centre, largest squared distance to it
     uint32_t *tc_pairs;     // tile pairs that may hold neighbours (bits) [tiles][ceil(tiles / 32)]
+    void *wt;               // warp-tile path (d <= 16 all pairs): its arrays, wt_bytes(cap_n) (null: not served)
     PhaseMarks *marks;      // host-side timing marks of the owning plan
     // second stream of the grid path: independent kernels run beside each
     // other (fork/join by events); unused while per-kernel marks are taken
@@ -275,6 +276,14 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n, int32
                                uint8_t *core_out, cudaStream_t st);
 cudaError_t launch_tc_verify(const DbWork &w, const float *x, int64_t n, int32_t d, int64_t Tc, bool bf16,
                              cudaStream_t st);
+// In-place exclusive scan of n bucket sizes by one block.
+cudaError_t launch_bucket_scan(int32_t *v, int32_t n, cudaStream_t st);
+// All pairs for d <= 16 on ordered rows (pairs_wt.cu): device bytes of its
+// arrays, and the whole run.
+constexpr int kWtMaxCellBits = 18;  // cells of its counting sort
+size_t wt_bytes(int64_t n);
+cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n, int32_t d, int64_t Tc, int32_t min_pts,
+                               bool exact, int32_t *labels, int32_t *counts_out, uint8_t *core_out, cudaStream_t st);
 cudaError_t launch_labels_allpairs(const DbWork &w, int64_t n, int32_t *labels, int32_t *counts_out,
                                    uint8_t *core_out, cudaStream_t st);
 cudaError_t launch_compact(const DbWork &w, int64_t n, int32_t *labels, cudaStream_t st);

@@ -129,6 +129,32 @@ __global__ void scan_tiles(const int *__restrict__ in, int64_t n, const int *__r
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = part[gridDim.x];
 }
 
+// In-place exclusive scan by one block of 1024 threads, 8 values a thread and
+// round: the bucket sizes of a counting sort (some thousands to 2^18).
+__global__ void __launch_bounds__(1024) bucket_scan_kernel(int *__restrict__ v, int n) {
+    db::wait_prior_grid();  // started as a programmatic dependent
+    db::allow_next_grid();
+    __shared__ int wt[32];
+    int carry = 0;
+    for (int base = 0; base < n; base += 8192) {
+        const int i0 = base + (int)threadIdx.x * 8;
+        int x[8], s = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            x[k] = i0 + k < n ? v[i0 + k] : 0;
+            s += x[k];
+        }
+        int total;
+        int at = carry + block_excl_scan(s, wt, total);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (i0 + k < n) v[i0 + k] = at;
+            at += x[k];
+        }
+        carry += total;
+    }
+}
+
 __global__ void root_flags_kernel(int n, const int *__restrict__ labels, int *__restrict__ flags) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         flags[i] = labels[i] == i;
@@ -157,6 +183,10 @@ cudaError_t launch_exclusive_scan(const int32_t *in, int32_t *out, int64_t n, in
     scan_tiles<<<(unsigned)tiles, SCAN_NT, 0, st>>>(in, n, part, out);
     if (pm) pm->kernel("scan_tiles", st);
     return cudaGetLastError();
+}
+
+cudaError_t launch_bucket_scan(int32_t *v, int32_t n, cudaStream_t st) {
+    return launch_dependent(bucket_scan_kernel, 1, 1024, st, v, n);
 }
 
 cudaError_t launch_labels_allpairs(const DbWork &w, int64_t n, int32_t *labels, int32_t *counts_out,

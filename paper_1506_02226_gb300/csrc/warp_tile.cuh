@@ -1,5 +1,6 @@
 // warp_tile.cuh — the exact pair test of ordered rows for d <= 16, a warp at a
-// time on matrix instructions (the batched kernels, batch.cu).
+// time on matrix instructions, and the passes built on it: many instances at
+// once (batch.cu) and one instance's all-pairs run (pairs_wt.cu).
 //
 // Rows hold centred units v = u - 512 in [-512, 511] as FP16 (exact), padded
 // to 16 coordinates, so one mma.sync m16n8k16 gives the dot products of 16 x 8
@@ -32,6 +33,8 @@
 // so an item needs one record and no per-instance pointers.
 #pragma once
 
+#include <cuda_fp16.h>
+
 #include <climits>
 
 #include "internal.cuh"
@@ -52,7 +55,15 @@ struct __align__(16) TileRec {
     float Tp1;
     int inst;
     int point0;         // the instance's first point in point-indexed arrays
-    int pad[3];
+    int leave;          // count: rows stop mattering at this many neighbours (min_pts, or INT_MAX: exact counts)
+    int pad[2];
+};
+
+struct Hdr {  // device-side sizes of a run
+    int count;        // instances
+    int total_points;
+    int total_tiles;
+    int max_chunks;   // column chunks of the largest instance
 };
 
 struct Rows {  // by row of the batch (64 per tile), unless said otherwise
@@ -116,7 +127,7 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
 }
 
 // Out of line: keeps the union-find loops out of the tile's registers.
-__device__ __noinline__ int unite_rows(int *parent, int p, int q, unsigned *status) {
+static __device__ __noinline__ int unite_rows(int *parent, int p, int q, unsigned *status) {
     return db::uf_unite_root(parent, p, q, status);
 }
 
@@ -263,6 +274,12 @@ __device__ __forceinline__ void run_item(const Rows &R, const TileRec &I, int T,
         prior[i] = PASS == WT_COUNT ? (b > -1e29f ? R.count[row] : INT_MAX / 2) : 0;
     }
     if (!__any_sync(FULL, mine)) return;
+    if (PASS == WT_COUNT) {  // other chunks' items may have counted enough already
+        bool done = true;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) done &= prior[i] >= I.leave;
+        if (__all_sync(FULL, done)) return;
+    }
     unsigned long long evaluated = 0;
     const int rows_in = min(32, left), last = I.tile0 + I.ntiles - 1, nlast = I.n - (I.ntiles - 1) * BT;
     int visited = 0;
@@ -273,7 +290,7 @@ __device__ __forceinline__ void run_item(const Rows &R, const TileRec &I, int T,
         if (PASS != WT_COUNT || (visited > 2 && (visited & 1))) return true;
         bool done = true;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) done &= prior[i] + it.counted(i) >= I.min_pts;
+        for (int i = 0; i < 4; ++i) done &= prior[i] + it.counted(i) >= I.leave;
         return !__all_sync(FULL, done);
     };
     const int nct = ct1 - ct0, ngrp = (nct + 31) >> 5;
@@ -471,6 +488,185 @@ __device__ __forceinline__ void root_row(int *parent, int *least, bool is, int r
         const int m = __reduce_min_sync(peers, point);
         if (lane == __ffs(peers) - 1 && m < db::ld_relaxed(least + root)) atomicMin(least + root, m);
     }
+}
+
+// ---- the passes, as kernels ----
+
+// Work item w: half w mod 2 of tile (w / 2) mod total, the chunk (w / 2) / total
+// steps after the tile's own (wrapping around its instance), for one warp; the
+// next item is claimed while the current one runs.
+template <int PASS>
+static __global__ void __launch_bounds__(NT, 3) pass_kernel(Rows R, const Hdr *__restrict__ hdr, int ch_tiles,
+                                                     unsigned long long *work) {
+    db::wait_prior_grid();  // returns at once when launched the plain way
+    db::allow_next_grid();
+    const int total = hdr->total_tiles, lane = threadIdx.x & 31;
+    const unsigned long long nitems =
+        2ull * (unsigned long long)total * (PASS == WT_NEAR ? 1 : hdr->max_chunks);
+    unsigned long long next = 0;
+    if (lane == 0) next = atomicAdd(work, 1ull);
+    while (true) {
+        const unsigned long long item = __shfl_sync(FULL, next, 0);
+        if (item >= nitems) return;
+        if (lane == 0) next = atomicAdd(work, 1ull);
+        const unsigned long long two = item >> 1;
+        const int step = (int)(two / (unsigned)total), T = (int)(two - (unsigned long long)step * total);
+        const TileRec I = R.tiles[T];
+        const int end = I.tile0 + I.ntiles;
+        int ct0, ct1;
+        if (PASS == WT_NEAR) {
+            ct0 = T + 1;
+            ct1 = min(end, T + 1 + kNear);
+        } else {
+            const int nchunk = (I.ntiles + ch_tiles - 1) / ch_tiles;
+            if (step >= nchunk) continue;
+            int chunk = (T - I.tile0) / ch_tiles + step;
+            if (chunk >= nchunk) chunk -= nchunk;
+            ct0 = I.tile0 + chunk * ch_tiles;
+            ct1 = min(end, ct0 + ch_tiles);
+            if (PASS == WT_FAR) ct0 = max(ct0, T + 1 + kNear);
+        }
+        if (ct0 < ct1) run_item<PASS>(R, I, T, (int)(item & 1), ct0, ct1);
+    }
+}
+
+static __global__ void __launch_bounds__(NT, 3) core_kernel(Rows R, const Hdr *__restrict__ hdr) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
+    __shared__ unsigned long long adj[NT / 32][BT];
+    __shared__ int lab[NT / 32][BT];
+    const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5), wib = threadIdx.x >> 5;
+    for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps)
+        core_tile(R, R.tiles[T], T, adj[wib], lab[wib]);
+}
+
+static __global__ void __launch_bounds__(NT) flatten_kernel(Rows R, const Hdr *__restrict__ hdr) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
+    const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+    for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps) flatten_tile(R, T);
+}
+
+static __global__ void __launch_bounds__(NT) root_kernel(Rows R, const Hdr *__restrict__ hdr, int *least) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
+    const int total = hdr->total_tiles * BT, step = (int)(gridDim.x * blockDim.x);
+    for (int g0 = (int)(blockIdx.x * blockDim.x); g0 < total; g0 += step) {
+        const int g = g0 + (int)threadIdx.x;
+        const bool is = g < total && R.core[g];
+        root_row(R.parent, least, is, g, is ? R.perm[g] : 0);
+    }
+}
+
+// ---- packing ----
+
+// What packing writes, by row, tile or point (see Rows).
+struct PackOut {
+    TileRec *tiles;
+    int *perm, *inv, *count, *least;
+    uint2 *P16;
+    float *nb, *box;
+    long long cap_tiles;
+};
+
+__device__ __forceinline__ unsigned half2_bits(int lo, int hi) {
+    const __half2 h = __halves2half2(__int2half_rn(lo), __int2half_rn(hi));
+    return *reinterpret_cast<const unsigned *>(&h);
+}
+
+// Packs the 64 rows of tile tt of an instance (a warp, two rows a lane): grid
+// check, centred units, norm, the tile's box.  A lane reads its two rows whole
+// (the rows of a tile are scattered in the input), all loads independent.
+// order: point of each row (null: identity).  Returns true on off-grid input.
+template <int DP, typename Order>
+__device__ __forceinline__ bool pack_tile(const float *x, const TileRec &I, int tt, const Order *order,
+                                          const PackOut &w) {
+    const int lane = threadIdx.x & 31, n = I.n, d = I.d, T = I.tile0 + tt;
+    bool bad = false;
+    int v[2][DP];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int s = tt * BT + 32 * h + lane, row = T * BT + 32 * h + lane;
+        const int o = s < n ? (order ? (int)order[s] : s) : 0;
+        const float *src = x + (size_t)o * d;
+        float f[DP];
+#pragma unroll
+        for (int k = 0; k < DP; ++k) f[k] = s < n && k < d ? src[k] : 0.5f;
+        if (s < n) {
+            w.perm[row] = o;
+            w.inv[I.point0 + o] = row;
+        }
+        w.count[row] = 0;
+        w.least[row] = DB_NONE;
+        int s2 = 0;
+#pragma unroll
+        for (int k = 0; k < DP; ++k) {
+            int u;
+            bad |= !db::on_grid(f[k], u);
+            v[h][k] = u - 512;  // 0 for the padding
+            s2 += v[h][k] * v[h][k];
+        }
+        w.nb[row] = s < n ? -(float)s2 : -1e30f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {  // piece k: units 2k, 2k+1, 2k+8, 2k+9
+            uint2 pc;
+            pc.x = half2_bits(2 * k < DP ? v[h][2 * k] : 0, 2 * k + 1 < DP ? v[h][2 * k + 1] : 0);
+            pc.y = half2_bits(2 * k + 8 < DP ? v[h][2 * k + 8] : 0, 2 * k + 9 < DP ? v[h][2 * k + 9] : 0);
+            w.P16[(size_t)row * 4 + k] = pc;
+        }
+    }
+    const bool on0 = tt * BT + lane < n, on1 = tt * BT + 32 + lane < n;
+#pragma unroll
+    for (int k = 0; k < DP; ++k) {
+        const int lo = __reduce_min_sync(FULL, min(on0 ? v[0][k] : INT_MAX, on1 ? v[1][k] : INT_MAX));
+        const int hi = __reduce_max_sync(FULL, max(on0 ? v[0][k] : INT_MIN, on1 ? v[1][k] : INT_MIN));
+        if (lane == 0) {
+            w.box[(size_t)k * w.cap_tiles + T] = (float)lo;
+            w.box[(size_t)(16 + k) * w.cap_tiles + T] = (float)hi;
+        }
+    }
+    if (lane == 0) w.tiles[T] = I;
+    return bad;
+}
+template <typename Order>
+__device__ __forceinline__ bool pack_tile_d(const float *x, const TileRec &I, int tt, const Order *order,
+                                            const PackOut &w) {
+    switch (I.d) {  // warp-uniform
+        case 1: return pack_tile<1>(x, I, tt, order, w);
+        case 2: return pack_tile<2>(x, I, tt, order, w);
+        case 3: return pack_tile<3>(x, I, tt, order, w);
+        case 4: return pack_tile<4>(x, I, tt, order, w);
+        case 5:
+        case 6:
+        case 7:
+        case 8: return pack_tile<8>(x, I, tt, order, w);
+        default: return pack_tile<16>(x, I, tt, order, w);
+    }
+}
+
+// Morton (Z-order) dilation of a 10-bit coordinate: bit b moves to bit 3b.
+__device__ __forceinline__ unsigned dilate3(unsigned v) {
+    v &= 1023u;
+    v = (v | (v << 16)) & 0x030000FFu;
+    v = (v | (v << 8)) & 0x0300F00Fu;
+    v = (v | (v << 4)) & 0x030C30C3u;
+    v = (v | (v << 2)) & 0x09249249u;
+    return v;
+}
+
+// Z-order code of a point's first dz (at most three) grid coordinates, the top
+// `bits` bits of each interleaved.
+__device__ __forceinline__ unsigned zcode(const float *x, int dz, int bits) {
+    unsigned code = 0;
+    for (int j = 0; j < dz; ++j) {
+        int u;
+        db::on_grid(x[j], u);  // off-grid input is reported when the row is packed
+        code |= dilate3((unsigned)u >> (10 - bits)) << j;
+    }
+    if (dz == 3) return code;
+    unsigned c = 0;  // no third (second) axis: close the gaps
+    for (int b = 0; b < bits; ++b) c |= ((code >> (3 * b)) & ((1u << dz) - 1u)) << (dz * b);
+    return c;
 }
 
 }  // namespace wtile
