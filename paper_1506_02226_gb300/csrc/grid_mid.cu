@@ -42,6 +42,10 @@
 namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
+// score (by grouped position): 1 core, 0 not core, kIsolated not core and no
+// neighbour but itself (its count is exact: only core points stop counting
+// early), so the border pass has nothing to look for
+constexpr uint8_t kIsolated = 2;
 
 __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned *p) {
     unsigned v;
@@ -221,7 +225,7 @@ __global__ void __launch_bounds__(256) mid_count_kernel(MidArgs a, int min_pts, 
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nitems = *a.nitems;
     const int lim = exact ? INT_MAX : min_pts;
-    unsigned ev = 0;
+    unsigned ev = 0, ev1 = 0;
     for (int it = warp; it < nitems; it += nwarps) {
         const int2 item = a.items[it];
         const int A = item.x, i0 = item.y;
@@ -272,24 +276,65 @@ __global__ void __launch_bounds__(256) mid_count_kernel(MidArgs a, int min_pts, 
                 pend = __ballot_sync(FULL, mine && cnt < lim);
             }
         }
+        // The chunk's core points are joined here, in registers: each lane's
+        // neighbours among them as a bit mask, then smallest-lane propagation.
+        // A point starts in the merge under the smallest index of its group, so
+        // the merge meets a dense chunk as one set (200,000 x 8: merge 583 us
+        // with every point a set of its own).
+        const int o = mine ? a.sidx[pos] : DB_NONE;
+        const bool c = mine && cnt >= min_pts;
+        const unsigned cores = __ballot_sync(FULL, c);
+        unsigned nb = c ? 1u << lane : 0u;
+        if (cores & (cores - 1)) {
+            float qv[DP];  // this lane's units (pv holds them doubled)
+#pragma unroll
+            for (int k = 0; k < DP; ++k) qv[k] = 0.5f * pv[k];
+            const float qn = c ? cpm - a.g.Tp1 : -1e30f;
+            for (unsigned m = cores; m; m &= m - 1) {
+                const int i = __ffs(m) - 1;
+                float p2[DP];
+#pragma unroll
+                for (int k = 0; k < DP; ++k) p2[k] = __shfl_sync(FULL, pv[k], i);
+                const unsigned w = __ballot_sync(FULL, mid_nbr<DP>(__shfl_sync(FULL, cpm, i), p2, qv, qn));
+                if (lane == i) nb = w;
+            }
+            ev1 += (unsigned)(__popc(cores) * (__popc(cores) - 1) / 2);
+        }
+        int lab = nb ? __ffs(nb) - 1 : lane;
+        if (cores & (cores - 1)) {
+            while (true) {
+                int l = lab;
+                for (unsigned m = cores; m; m &= m - 1) {
+                    const int j = __ffs(m) - 1, lj = __shfl_sync(FULL, lab, j);
+                    if ((nb >> j) & 1u) l = min(l, lj);
+                }
+                const bool moved = l < lab;
+                lab = l;
+                if (!__any_sync(FULL, moved)) break;
+            }
+        }
+        const unsigned peers = __match_any_sync(FULL, lab);
+        const int least = __reduce_min_sync(peers, o);
         if (mine) {
-            const int o = a.sidx[pos];
-            const bool c = cnt >= min_pts;
             count[o] = cnt;
             core[o] = c;
-            score[pos] = c;
-            parent[o] = o;
-            hint[pos] = o;
+            score[pos] = c ? 1 : (cnt > 1 ? 0 : kIsolated);
+            parent[o] = c ? least : o;
+            hint[pos] = c ? least : o;
         }
     }
     db::block_sum_add(a.ev + 0, lane == 0 ? (unsigned long long)ev : 0ull);
+    __syncthreads();  // block_sum_add's scratch is free again
+    db::block_sum_add(a.ev + 1, lane == 0 ? (unsigned long long)ev1 : 0ull);
 }
 
 // Merge pass (Section IV-C): every core point of the chunk against the core
 // candidates after it (a larger cell id, or a later position in its own
 // cell), uniting the two sets at each eps-pair.  hint[pos] holds a member of
-// the point's set (its index, or a root seen later): equal hints mean one set,
-// so those pairs need neither a test nor a union.
+// the point's set (its group's index from the count pass, or a root seen
+// later): equal hints mean one set, so those pairs need neither a test nor a
+// union.  The warp makes one union at a time and then renames the two hints it
+// joined in all its lanes, so two sets that meet in many pairs are united once.
 template <int DP>
 __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t *__restrict__ score, int *parent,
                                                         int *hint, unsigned *status) {
@@ -303,7 +348,7 @@ __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t
         const int sA = a.cell_start[A], cA = a.cell_count[A];
         const bool inr = i0 + lane < cA;
         const int pos = sA + i0 + (inr ? lane : 0);
-        const bool mine = inr && score[pos];
+        const bool mine = inr && score[pos] == 1;
         const unsigned cores = __ballot_sync(FULL, mine);
         if (!cores) continue;
         float pv[DP];
@@ -311,8 +356,8 @@ __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t
         const float cpm = a.g.Tp1 + a.nrm[pos];
 #pragma unroll
         for (int k = 0; k < DP; ++k) pv[k] *= 2.f;
-        const int om = a.sidx[pos];
         int hm = mine ? db::ld_relaxed(hint + pos) : -1;
+        const int h_begin = hm;
         const int *row = a.nbr + (size_t)A * a.g.noff;
         const int nn = a.ncnt[A] & 0xffff;
         for (int k0 = 0; k0 < nn; k0 += 32) {
@@ -321,56 +366,85 @@ __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t
             const int s = take ? a.cell_start[B] : 0, c = take ? a.cell_count[B] : 0;
             const int incl = warp_incl_scan(c), total = __shfl_sync(FULL, incl, 31);
             for (int base = 0; base < total; base += 128) {
-                float qv[4][DP], qn[4];
-                int qp[4], qo[4], qh[4];
+                int qp[4], qh[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int j = base + 32 * u + lane;
                     const int q = locate(j, incl, c, s);
-                    qp[u] = -1;
-                    if (j < total && score[q]) {
-                        qp[u] = q;
-                        load_row<DP>(a.P, q, qv[u]);
-                        qn[u] = a.nrm[q];
-                        qo[u] = a.sidx[q];
-                        qh[u] = db::ld_relaxed(hint + q);
+                    const bool on = j < total && score[q] == 1;
+                    qp[u] = on ? q : -1;
+                    qh[u] = on ? db::ld_relaxed(hint + q) : -1;
+                }
+                // rows of the candidates some core point of the chunk may have to be united with
+                const int h0 = __shfl_sync(FULL, hm, __ffs(cores) - 1);
+                const bool uniform = __all_sync(FULL, !mine || hm == h0);
+                float qv[4][DP], qn[4];
+                bool load = false;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) load |= qp[u] >= 0 && !(uniform && qh[u] == h0);
+                if (!__any_sync(FULL, load)) continue;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (qp[u] >= 0) {
+                        load_row<DP>(a.P, qp[u], qv[u]);
+                        qn[u] = a.nrm[qp[u]];
                     } else {
 #pragma unroll
                         for (int k = 0; k < DP; ++k) qv[u][k] = 0.f;
                         qn[u] = -1e30f;
-                        qo[u] = -1;
-                        qh[u] = -1;
                     }
                 }
                 for (unsigned m = cores; m; m &= m - 1) {
                     const int i = __ffs(m) - 1;
+                    const int pi = __shfl_sync(FULL, pos, i);
+                    int h = __shfl_sync(FULL, hm, i);
+                    bool need = false;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) need |= qp[u] > pi && qh[u] != h;  // after p, and not one set already
+                    if (!__any_sync(FULL, need)) continue;
                     float p2[DP];
 #pragma unroll
                     for (int k = 0; k < DP; ++k) p2[k] = __shfl_sync(FULL, pv[k], i);
                     const float cp = __shfl_sync(FULL, cpm, i);
-                    const int pi = __shfl_sync(FULL, pos, i), oi = __shfl_sync(FULL, om, i);
-                    int h = __shfl_sync(FULL, hm, i);
-                    int root = INT_MAX;
+                    unsigned hit = 0;
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (qp[u] <= pi || qh[u] == h) continue;  // not after p, padding, or one set already
-                        ++ev;
-                        if (!mid_nbr<DP>(cp, p2, qv[u], qn[u])) continue;
-                        const int r = db::uf_unite_root(parent, oi, qo[u], status);
-                        if (r >= 0) {
-                            qh[u] = r;
-                            db::st_relaxed(hint + qp[u], r);
-                            root = min(root, r);
+                    for (int u = 0; u < 4; ++u)
+                        if (qp[u] > pi && qh[u] != h) {
+                            ++ev;
+                            hit |= (unsigned)mid_nbr<DP>(cp, p2, qv[u], qn[u]) << u;
                         }
-                    }
-                    root = (int)__reduce_min_sync(FULL, (unsigned)root);
-                    if (root != INT_MAX && lane == i) {
-                        hm = root;
-                        db::st_relaxed(hint + pos, root);
+                    unsigned any;
+                    while ((any = __ballot_sync(FULL, hit != 0)) != 0) {
+                        const int src = __ffs(any) - 1;
+                        int q = 0, hq = 0;
+#pragma unroll
+                        for (int u = 3; u >= 0; --u)
+                            if ((hit >> u) & 1u) {
+                                q = qp[u];
+                                hq = qh[u];
+                            }
+                        q = __shfl_sync(FULL, q, src);
+                        hq = __shfl_sync(FULL, hq, src);
+                        // h and hq are members of the two sets
+                        int r = 0;
+                        if (lane == src) {
+                            r = db::uf_unite_root(parent, h, hq, status);
+                            if (r >= 0) db::st_relaxed(hint + q, r);
+                        }
+                        r = __shfl_sync(FULL, r, src);
+                        if (r < 0) r = hq;
+                        if (hm == h || hm == hq) hm = r;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (qp[u] >= 0 && (qh[u] == h || qh[u] == hq)) qh[u] = r;
+                            if (qh[u] == r) hit &= ~(1u << u);
+                        }
+                        h = r;
                     }
                 }
             }
         }
+        if (mine && hm != h_begin) db::st_relaxed(hint + pos, hm);
     }
     db::block_sum_add(a.ev + 1, (unsigned long long)ev);
 }
@@ -391,7 +465,8 @@ __global__ void __launch_bounds__(256) mid_border_kernel(MidArgs a, const uint8_
         const int sA = a.cell_start[A], cA = a.cell_count[A];
         const bool inr = i0 + lane < cA;
         const int pos = sA + i0 + (inr ? lane : 0);
-        const bool mine = inr && !score[pos];
+        const bool mine = inr && score[pos] == 0;  // not core, and some neighbour
+        if (inr && score[pos] == kIsolated) border[a.sidx[pos]] = DB_NONE;
         const unsigned pend = __ballot_sync(FULL, mine);
         if (!pend) continue;
         float pv[DP];
@@ -414,7 +489,7 @@ __global__ void __launch_bounds__(256) mid_border_kernel(MidArgs a, const uint8_
                     const int j = base + 32 * u + lane;
                     const int q = locate(j, incl, c, s);
                     qi[u] = DB_NONE;
-                    if (j < total && score[q]) {
+                    if (j < total && score[q] == 1) {
                         qi[u] = a.sidx[q];
                         load_row<DP>(a.P, q, qv[u]);
                         qn[u] = a.nrm[q];
