@@ -175,9 +175,11 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     DeviceGuard dg(o.device);
     cudaStream_t st = plan->stream;
     const bool sync = o.synchronous || stats;
-    if (o.synchronous && cudaMemsetAsync(plan->w.status, 0, sizeof(unsigned), st) != cudaSuccess)
+    const bool want_grid = d <= 3 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0;
+    const bool small = want_grid && n <= kGridSmallMaxN;  // one kernel, which clears what it needs
+    if (!small && o.synchronous && cudaMemsetAsync(plan->w.status, 0, sizeof(unsigned), st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
-    if (cudaMemsetAsync(plan->w.ctr, 0, sizeof(unsigned long long) * DB_NCTR, st) != cudaSuccess)
+    if (!small && cudaMemsetAsync(plan->w.ctr, 0, sizeof(unsigned long long) * DB_NCTR, st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
     if (stats) cudaEventRecord(plan->ev0, st);
     plan->marks.begin(st);
@@ -186,14 +188,15 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     int path;
     GridGeom g;
     cudaError_t err;
-    const bool want_grid = d <= 3 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0;
     // the projected grid (4 <= d <= 8) needs the eps-grid's arrays and row stride >= 8 (4 for d = 4)
     const bool want_mid = d >= 4 && d <= 8 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0 &&
                           plan->w.dp_cap >= (d <= 4 ? 4 : 8);
     if (o.grid == DBSCAN_GRID_ON && !(want_grid || want_mid)) return DBSCAN_ERR_UNSUPPORTED;
     if (want_grid && grid_geometry(d, Tc, n, &g)) {
         path = DBSCAN_PATH_GRID;
-        err = launch_grid_path(plan->w, g, points, n, min_pts, exact, labels, counts_out, core_out, st);
+        err = small ? launch_grid_small(plan->w, g, points, n, min_pts, exact, o.label_mode == DBSCAN_LABEL_COMPACT,
+                                        stats != nullptr, o.synchronous, labels, counts_out, core_out, st)
+                    : launch_grid_path(plan->w, g, points, n, min_pts, exact, labels, counts_out, core_out, st);
     } else if (want_mid && mid_geometry(d, Tc, n, &g)) {
         path = DBSCAN_PATH_GRID_PROJECTED;
         err = launch_mid_grid_path(plan->w, g, points, n, d, min_pts, exact, labels, counts_out, core_out, st);
@@ -224,8 +227,8 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
             if (!err) err = launch_labels_allpairs(plan->w, n, labels, counts_out, core_out, st);
         }
     }
-    if (!err && o.label_mode == DBSCAN_LABEL_COMPACT) err = launch_compact(plan->w, n, labels, st);
-    if (!err && stats && (path == DBSCAN_PATH_GRID || path == DBSCAN_PATH_GRID_PROJECTED))
+    if (!err && !small && o.label_mode == DBSCAN_LABEL_COMPACT) err = launch_compact(plan->w, n, labels, st);
+    if (!err && !small && stats && (path == DBSCAN_PATH_GRID || path == DBSCAN_PATH_GRID_PROJECTED))
         err = launch_grid_candidates(plan->w, g, n, path == DBSCAN_PATH_GRID_PROJECTED, st);
     if (err != cudaSuccess) {
         std::fprintf(stderr, "dbscan: launch failed: %s\n", cudaGetErrorString(err));
@@ -234,8 +237,8 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     if (stats) cudaEventRecord(plan->ev1, st);
     if (!sync) return DBSCAN_OK;
 
-    if (cudaMemcpyAsync(plan->h_ctr, plan->w.ctr, sizeof(unsigned long long) * DB_NCTR, cudaMemcpyDeviceToHost, st) !=
-        cudaSuccess)
+    if (stats && cudaMemcpyAsync(plan->h_ctr, plan->w.ctr, sizeof(unsigned long long) * DB_NCTR,
+                                 cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
     const int s = plan_read_status(plan, !o.synchronous);
     if (s) return s;

@@ -171,6 +171,7 @@ struct TcArgs {
     int stall;                   // test hook: the MMA issuer issues nothing
     int ct_chunk;                // column tiles per work item: 1, 2, 4, 8, 16 or 32
     int rel_lo, rel_hi;          // chunks visited, relative to the one of the row unit's own tile
+    int near_lo, near_hi;        // union: column tiles visited, relative to the row unit's own tile
     int rotate;                  // 1: relative chunks wrap around (count, border of sorted points)
     const unsigned *pairs;       // surviving tile pairs, row stride `words` (null: all)
     int words;
@@ -501,7 +502,10 @@ __device__ __forceinline__ unsigned item_mask(const TcArgs &a, int w, int units,
     if (PASS == TC_COUNT) {
         if (a.min_pts > 0 && a.udone[u] == (1 << Shape<TC_COUNT, RTN == 1>::EPI) - 1) return 0u;
     }
-    if (PASS == TC_UNION && c0 < i) m &= ~((1u << (i - c0)) - 1u);  // tiles from the unit's own on
+    if (PASS == TC_UNION) {  // tiles [i + near_lo, i + near_hi]
+        if (c0 < i + a.near_lo) m = i + a.near_lo - c0 >= 32 ? 0u : m & ~((1u << (i + a.near_lo - c0)) - 1u);
+        if (i + a.near_hi < c0 + 31) m = i + a.near_hi < c0 ? 0u : m & ((2u << (i + a.near_hi - c0)) - 1u);
+    }
     if (PASS == TC_BORDER && !a.rowneed[i]) return 0u;
     if (a.pairs) m &= a.pairs[(size_t)i * a.words + (c0 >> 5)] >> (c0 & 31);
     if (PASS == TC_UNION || PASS == TC_BORDER) {
@@ -1279,25 +1283,33 @@ __global__ void __launch_bounds__(256) tc_pack_kernel(PackArgs a) {
     src_s[tid] = !valid ? -1 : (a.n_src ? pivot_point(pos, a.n, a.n_src) : (a.list ? a.list[pos] : pos));
     __syncthreads();
     bool ok = true;
-#pragma unroll 4
-    for (int rr = 0; rr < 32; ++rr) {
-        const int row = warp * 32 + rr, src = src_s[row];
-        int s = 0;
+#pragma unroll 1
+    for (int r0 = 0; r0 < 32; r0 += 16) {  // 16 rows of the warp in flight
+        float f[16][2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const int k = lane + 32 * h;
-            if (k >= K) continue;
-            int v = 0;
-            if (k < a.d && src >= 0) {
-                int u;
-                ok &= db::on_grid(a.x[(size_t)src * a.d + k], u);
-                v = u - 512;
+        for (int rr = 0; rr < 16; ++rr) {
+            const int src = src_s[warp * 32 + r0 + rr];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int k = lane + 32 * h;
+                f[rr][h] = k < a.d && src >= 0 ? a.x[(size_t)src * a.d + k] : 0.5f;
             }
-            rows[row][k] = (int16_t)v;
-            s += v * v;
         }
-        s = __reduce_add_sync(FULL, s);
-        if (lane == 0) nrm_s[row] = s;
+#pragma unroll
+        for (int rr = 0; rr < 16; ++rr) {
+            const int row = warp * 32 + r0 + rr;
+            int s = 0;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                int u;
+                ok &= db::on_grid(f[rr][h], u);
+                const int v = u - 512;  // 0 for the padding
+                if (lane + 32 * h < K) rows[row][lane + 32 * h] = (int16_t)v;
+                s += v * v;
+            }
+            s = __reduce_add_sync(FULL, s);
+            if (lane == 0) nrm_s[row] = s;
+        }
     }
     if (!__all_sync(FULL, ok) && lane == 0) atomicOr(a.status, DB_EBIT_NOT_QUANTISED);
     __syncthreads();
@@ -1459,22 +1471,45 @@ __global__ void __launch_bounds__(256) tc_pack_kernel(PackArgs a) {
 }
 
 // Each pivot under the first pivot before it within twice eps (a warp per
-// pivot; the search stops there), and the bucket sizes cleared.
+// pivot, 64 earlier pivots staged at a time for the block's eight; a search
+// stops at its first hit), and the bucket sizes cleared.
 __global__ void __launch_bounds__(256) tc_pivot_link_kernel(const int16_t *__restrict__ v16, int K, int P, int T4,
                                                             int *__restrict__ link, int *__restrict__ hist, int nhist) {
     db::wait_prior_grid();  // started as a programmatic dependent
     db::allow_next_grid();
-    const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x), k = t >> 5, lane = threadIdx.x & 31;
+    __shared__ int rows[64][33], mine[8][33];  // two units a word; rows start in different banks
+    const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x), lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int k = t >> 5, kw = K / 2, kmax = blockIdx.x * 8 + 7;  // P is a multiple of 8
+    const int *src = reinterpret_cast<const int *>(v16);
     for (int e = t; e < nhist; e += (int)(gridDim.x * blockDim.x)) hist[e] = 0;
-    if (k >= P) return;
+    for (int c = lane; c < kw; c += 32) mine[wid][c] = src[k * kw + c];
     int to = k;
-    for (int j0 = 0; j0 < k; j0 += 32) {
-        const int j = j0 + lane;
-        const unsigned hit = __ballot_sync(FULL, j < k && exact_sqdist(v16, K, k, j) <= T4);
-        if (hit) {
-            to = j0 + __ffs(hit) - 1;
-            break;
+    bool found = false;
+    for (int j0 = 0; j0 < kmax; j0 += 64) {
+        __syncthreads();
+        for (int e = threadIdx.x; e < 64 * kw; e += 256) {
+            const int r = e / kw, c = e - r * kw;
+            rows[r][c] = j0 + r < P ? src[(j0 + r) * kw + c] : 0;
         }
+        __syncthreads();
+        if (!found) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int j = j0 + 32 * h + lane;
+                int D = 0;
+                for (int c = 0; c < kw; ++c) {
+                    const int x = mine[wid][c], y = rows[32 * h + lane][c];
+                    const int d0 = (int)(int16_t)(x & 0xffff) - (int)(int16_t)(y & 0xffff), d1 = (x >> 16) - (y >> 16);
+                    D += d0 * d0 + d1 * d1;
+                }
+                const unsigned hit = __ballot_sync(FULL, j < k && D <= T4);
+                if (hit && !found) {
+                    to = j0 + 32 * h + __ffs(hit) - 1;
+                    found = true;
+                }
+            }
+        }
+        if (__syncthreads_and(found)) break;
     }
     if (lane == 0) link[k] = to;
 }
@@ -1711,6 +1746,9 @@ int chunk_tiles(int64_t units, int64_t nct, int sms) {
     return c;
 }
 
+// Merge: the tiles after a row unit's own that are taken first.
+constexpr int kNearTiles = 2;
+
 // Points from which they are ordered and tile pairs culled (see the header).
 constexpr int kSortMinN = 32768;
 
@@ -1882,8 +1920,8 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     w.marks->kernel("core_init", st);
 
     // pass 2: union of core-core neighbours.  First each core point under its
-    // first core neighbour of its own tile; then the tile pairs of the row
-    // unit's own chunk; then the rest, most of which the sets found so far skip.
+    // first core neighbour of its own tile; then the near tiles; then the rest,
+    // most of which the sets found so far skip.
     a.metaR = a.metaC = mcore;
     a.fold = 0;
     const int ch_union = chunk_tiles(units1, nt, sms), nch = (nt + ch_union - 1) / ch_union;
@@ -1894,16 +1932,23 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     w.marks->kernel("tc_hook", st);
     launch_dependent(tc_tag_kernel, nt, 256, st, n, w.core, w.parent, w.tc_tag);
     w.marks->kernel("tc_tag", st);
-    if (sorted && nch > 1) {
-        if ((e = launch_pass<TC_UNION>(a, bf16, sms, st))) return e;
-        w.marks->kernel("tc_union_near", st);
+    // (the tiles right after a row unit's own first: they link most of what
+    // belongs together, and the tags then skip most of the rest)
+    a.near_lo = 0;
+    a.near_hi = kNearTiles;
+    a.rel_hi = std::min(nch, 1 + (kNearTiles + ch_union - 1) / ch_union);
+    if ((e = launch_pass<TC_UNION>(a, bf16, sms, st))) return e;
+    w.marks->kernel("tc_union_near", st);
+    if (nt > 1 + kNearTiles) {
         launch_dependent(tc_tag_kernel, nt, 256, st, n, w.core, w.parent, w.tc_tag);
         w.marks->kernel("tc_tag", st);
-        a.rel_lo = 1;
+        a.near_lo = 1 + kNearTiles;
+        a.near_hi = nt;
+        a.rel_lo = 0;
+        a.rel_hi = nch;
+        if ((e = launch_pass<TC_UNION>(a, bf16, sms, st))) return e;
+        w.marks->kernel("tc_union", st);
     }
-    a.rel_hi = nch;
-    if ((e = launch_pass<TC_UNION>(a, bf16, sms, st))) return e;
-    w.marks->kernel("tc_union", st);
 
     // pass 3: smallest core neighbour of the rows that need one
     a.metaR = mneed;

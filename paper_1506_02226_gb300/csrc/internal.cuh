@@ -293,6 +293,13 @@ bool grid_geometry(int32_t d, int64_t Tc, int64_t n, GridGeom *g);
 cudaError_t launch_grid_path(const DbWork &w, const GridGeom &g, const float *x, int64_t n, int32_t min_pts,
                              bool exact_counts, int32_t *labels, int32_t *counts_out, uint8_t *core_out,
                              cudaStream_t st);
+// The whole eps-grid run of up to kGridSmallMaxN points in one launch
+// (grid_small.cu), labels dense when `compact`; clears the run's counters, and
+// the status word when `reset` is set.
+constexpr int kGridSmallMaxN = 4096;
+cudaError_t launch_grid_small(const DbWork &w, const GridGeom &g, const float *x, int64_t n, int32_t min_pts, bool exact,
+                              bool compact, bool stats, bool reset, int32_t *labels, int32_t *counts_out,
+                              uint8_t *core_out, cudaStream_t st);
 // Ordered candidate pairs of a grid run (own cell listed: the projected grid).
 cudaError_t launch_grid_candidates(const DbWork &w, const GridGeom &g, int64_t n, bool own_cell_listed,
                                    cudaStream_t st);
