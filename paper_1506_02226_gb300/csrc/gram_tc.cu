@@ -107,6 +107,7 @@
 #include <atomic>
 #include <climits>
 #include <cmath>
+#include <type_traits>
 
 #include "internal.cuh"
 
@@ -123,20 +124,21 @@ __host__ __device__ constexpr int bf16_band(int K) { return 16 * K; }
 // rho^2 of the band factor, the same for every point (rounded to FP32 once).
 __host__ __device__ inline float bf16_rho(int K) { return sqrtf((float)bf16_band(K)) * (1.f + 1.f / 1024.f); }
 
-// TC_HOOK: the merge's first step, each core point under its first core
-// neighbour of its own tile.  TC_ORDER: nearest pivot.  TC_CULL: ball tests.
-enum { TC_COUNT = 0, TC_UNION = 1, TC_BORDER = 2, TC_VERIFY = 3, TC_HOOK = 4, TC_ORDER = 5, TC_CULL = 6 };
+// TC_ADJ: the merge's first step, the neighbours of each core point among the
+// core points of its own tile, as bits.  TC_LINK, TC_ORDER: first pivot within
+// twice eps, nearest pivot.  TC_CULL: ball tests.
+enum { TC_COUNT = 0, TC_UNION = 1, TC_BORDER = 2, TC_VERIFY = 3, TC_ADJ = 4, TC_ORDER = 5, TC_CULL = 6, TC_LINK = 7 };
 
 // Shape of each pass.  Rows: two row tiles per item (256 rows) for the FP16
 // passes with a cheap or no consumer, one (128 rows) otherwise.  Epilogue
 // warps: 8 for the FP16 count, order and cull (one warp per lane quadrant and
-// row tile, each deciding all 256 columns), 16 for the FP16 border and hook
+// row tile, each deciding all 256 columns), 16 for the FP16 border and adjacency
 // (two warps per quadrant and row tile), 16 for the merge and the BF16 passes
 // (four per quadrant), 8 for the verification.
 template <int PASS, bool BF16>
 struct Shape {
-    static constexpr bool kWide = PASS == TC_ORDER || PASS == TC_CULL || (PASS == TC_COUNT && !BF16);
-    static constexpr int RTN = kWide || (!BF16 && (PASS == TC_BORDER || PASS == TC_HOOK)) ? 2 : 1;
+    static constexpr bool kWide = PASS == TC_ORDER || PASS == TC_CULL || PASS == TC_LINK || (PASS == TC_COUNT && !BF16);
+    static constexpr int RTN = kWide || (!BF16 && (PASS == TC_BORDER || PASS == TC_ADJ)) ? 2 : 1;
     static constexpr int EPI = kWide || PASS == TC_VERIFY ? 8 : 16;
     static constexpr int GW = PASS == TC_VERIFY ? 64 : 32;  // columns per group
     static constexpr int THREADS = 32 * (2 + EPI);
@@ -178,6 +180,9 @@ struct TcArgs {
     const int *bmax_ptr;  // FP16 count: largest |v|^2 of the input (decides the folded form)
     int *udone;           // count: per row unit, one bit per epilogue warp whose rows are all done
     const int *tag;       // per tile: -2 no core point, -1 core points of several sets, else their common root
+    int4 *items;          // work items that are not empty: unit, first tile, tile bits (null: found by the producers)
+    int *nlist, *ticket;  // their number, the next to be taken
+    unsigned *adj;        // adjacency: 8 words a row, its neighbours in its own tile
     const int *rowneed;   // border: per tile, some row needs the pass
     const int16_t *v16;   // centred units by position, row stride K (exact recheck)
     int *count;
@@ -418,6 +423,17 @@ __device__ __noinline__ int exact_sqdist(const int16_t *__restrict__ v16, int K,
     return s;
 }
 
+// 64 consecutive accumulator columns of this thread's TMEM lane (no wait), and
+// the wait for them (see tmem_wait_ld_dep).
+__device__ __forceinline__ void tmem_ld64_nowait(uint32_t taddr, uint32_t (&r)[64]) {
+    tmem_ld32_nowait(taddr, r);
+    tmem_ld32_nowait(taddr + 32, r + 32);
+}
+__device__ __forceinline__ void tmem_wait_ld_dep64(uint32_t (&r)[64]) {
+    tmem_wait_ld_dep(*reinterpret_cast<uint32_t(*)[32]>(r));
+    tmem_wait_ld_dep(*reinterpret_cast<uint32_t(*)[32]>(r + 32));
+}
+
 // Shared memory of one CTA: KC stored operand columns per row, NS stages of B
 // tiles, NM events (a tile's metadata and what the event is).  A B stage is
 // free again once its MMAs have completed; the epilogue holds only events, so
@@ -462,20 +478,10 @@ struct TcSmem {
     static_assert(bytes <= 232448, "shared memory of one CTA");
 };
 
-// Rare path of the epilogue: a pair that may be a neighbour.  Returns bit 0 =
-// neighbour, bit 1 = it was inside the rounding band and was rechecked.
-template <bool BF16>
-__device__ __noinline__ int decide_candidate(float wv, float alpha, float rho2, const int16_t *v16, int K, int p,
-                                             int q, int T) {
-    const bool sure = BF16 ? (wv - rho2 >= alpha) : (wv > alpha + (float)FP16_BAND);
-    if (sure) return 1;
-    return (exact_sqdist(v16, K, p, q) <= T ? 1 : 0) | 2;
-}
-
-// Union of p's and q's sets; returns a root the merged set had at some moment
+// Union of two members' sets; returns a root the merged set had at some moment
 // (out of line: keeps the union-find loop out of the epilogue's registers).
-__device__ __noinline__ int unite_root(int *parent, int p, int q, unsigned *status) {
-    return db::uf_unite_root(parent, p, q, status);
+__device__ __noinline__ int unite_sets(int *parent, int x, int y, unsigned *status) {
+    return db::uf_unite_root(parent, x, y, status);
 }
 
 // Work item w: row unit u and the column tiles of one chunk, as a bit mask of
@@ -490,15 +496,15 @@ __device__ __forceinline__ unsigned item_mask(const TcArgs &a, int w, int units,
     u = w - (w / units) * units;
     const int i = RTN == 2 ? u : u >> 1;  // the unit's tile
     int ch = rel;
-    if (PASS == TC_UNION || PASS == TC_HOOK || a.rotate) ch += i / a.ct_chunk;
+    if (PASS == TC_UNION || PASS == TC_ADJ || a.rotate) ch += i / a.ct_chunk;
     if (ch >= nchunk) {
-        if (PASS == TC_UNION || PASS == TC_HOOK) return 0u;
+        if (PASS == TC_UNION || PASS == TC_ADJ) return 0u;
         ch -= nchunk;
     }
     c0 = ch * a.ct_chunk;
     const int nt = min(a.ct_chunk, nct - c0);
     unsigned m = nt >= 32 ? FULL : ((1u << nt) - 1u);
-    if (PASS == TC_HOOK) return a.tag[i] != -2 ? 1u << (i - c0) : 0u;
+    if (PASS == TC_ADJ) return a.tag[i] != -2 ? 1u << (i - c0) : 0u;
     if (PASS == TC_COUNT) {
         if (a.min_pts > 0 && a.udone[u] == (1 << Shape<TC_COUNT, RTN == 1>::EPI) - 1) return 0u;
     }
@@ -517,6 +523,25 @@ __device__ __forceinline__ unsigned item_mask(const TcArgs &a, int w, int units,
         }
     }
     return m;
+}
+
+// The work items that are not empty, in about the order of their numbers, so
+// that the pass's CTAs can take them one by one (200,000 x 64: dealt out by
+// number, the busiest CTA of the count had 1.4 times the mean work).
+template <int PASS, int RTN>
+__global__ void __launch_bounds__(256) tc_items_kernel(TcArgs a) {
+    db::wait_prior_grid();  // started as a programmatic dependent
+    db::allow_next_grid();
+    const int units = (a.nR + TM * RTN - 1) / (TM * RTN), nct = (a.nC + TN - 1) / TN;
+    const int nitems = units * (a.rel_hi - a.rel_lo), lane = threadIdx.x & 31;
+    const int w = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    int u = 0, c0 = 0;
+    const unsigned m = w < nitems ? item_mask<PASS, RTN>(a, w, units, nct, u, c0) : 0u;
+    const unsigned on = __ballot_sync(FULL, m != 0);
+    int base = 0;
+    if (lane == 0 && on) base = atomicAdd(a.nlist, __popc(on));
+    base = __shfl_sync(FULL, base, 0);
+    if (m) a.items[base + __popc(on & db::lanemask_lt())] = make_int4(u, c0, (int)m, 0);
 }
 
 template <int PASS, bool BF16>
@@ -590,78 +615,109 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
     const uint32_t a_bytes = (uint32_t)(TM * a.kv * 2), bv_bytes = 2 * a_bytes;
     const uint32_t b_bytes = bv_bytes + (fold ? TN * 16 * 2 : 0);
 
+    long long w_prod = 0, w_mma_b = 0, w_mma_t = 0, w_epi = 0, t_start = clock64();
+    (void)w_prod, (void)w_mma_b, (void)w_mma_t, (void)w_epi, (void)t_start;
     if (warp == 0) {
         // ---------------- producer ----------------
         int ia = 0, tb = 0, te = 0;  // items, column tiles and events so far
         bool ok = true;
-        for (int base = blockIdx.x; base < nitems && ok; base += (int)gridDim.x * 32) {
-            const int w = base + lane * (int)gridDim.x;
-            int u = 0, c0 = 0;
-            unsigned mask = 0;
-            if (w < nitems && w >= 0) mask = item_mask<PASS, RTN>(a, w, units, nct, u, c0);
-            unsigned live = __ballot_sync(FULL, mask != 0);
-            while (live && ok) {
-                const int l = __ffs(live) - 1;
-                live &= live - 1;
-                const int iu = __shfl_sync(FULL, u, l), ic = __shfl_sync(FULL, c0, l);
-                unsigned m = __shfl_sync(FULL, mask, l);
-                const int itile = RTN == 2 ? iu : iu >> 1;
-                // (one lane's reading decides for the warp: other CTAs and warps write these)
+        // One item: unit iu, the column tiles ic + (bits of m).  done: what the
+        // unit's udone word was a little earlier.
+        auto run = [&](int iu, int ic, unsigned m, int done) {
+            const int itile = RTN == 2 ? iu : iu >> 1;
+            if (PASS == TC_COUNT && a.min_pts > 0 && done == DONE_ALL) return;
+            if (PASS == TC_UNION) {
+                // two tiles, each of one set: skipped when the sets are one by now
+                const int ti = a.tag[itile];
+                if (ti >= 0) {
+                    const int tj = ((m >> lane) & 1u) ? a.tag[ic + lane] : -1;
+                    const bool same = tj >= 0 && db::uf_find(a.parent, ti) == db::uf_find(a.parent, tj);
+                    m &= ~__ballot_sync(FULL, same);
+                }
+                if (!m) return;
+            }
+            const int ab = ia % NA;
+            if (!(ok = mbar_wait_warp(&S.a_empty[ab], ((ia / NA) & 1) ^ 1, abort_flag, a.wait_ns))) return;
+            if (elect_one()) {
+                S.unit[ab] = iu;
+                S.done[ab] = 0;
+                const uint16_t *src = a.opR + (size_t)itile * a.tile_r + (RTN == 1 ? (iu & 1) * (TM * a.kv) : 0);
+                mbar_arrive_expect_tx(&S.a_full[ab], RTN * a_bytes + (uint32_t)sizeof(MetaTile));
+                bulk_g2s(S.A[ab * RTN], src, RTN * a_bytes, &S.a_full[ab]);
+                bulk_g2s(&S.metaA[ab], a.metaR + itile, (uint32_t)sizeof(MetaTile), &S.a_full[ab]);
+            }
+            __syncwarp();
+            ++ia;
+            while (m) {
+                const int ct = ic + __ffs(m) - 1;
+                m &= m - 1;
+                // (one lane's reading decides for the warp: epilogue warps write it)
                 if (PASS == TC_COUNT && a.min_pts > 0 &&
-                    __shfl_sync(FULL, db::ld_relaxed(a.udone + iu), 0) == DONE_ALL)
-                    continue;
-                if (PASS == TC_UNION) {
-                    // two tiles, each of one set: skipped when the sets are one by now
-                    const int ti = a.tag[itile];
-                    if (ti >= 0) {
-                        const int tj = ((m >> lane) & 1u) ? a.tag[ic + lane] : -1;
-                        const bool same = tj >= 0 && db::uf_find(a.parent, ti) == db::uf_find(a.parent, tj);
-                        m &= ~__ballot_sync(FULL, same);
-                    }
-                    if (!m) continue;
-                }
-                const int ab = ia % NA;
-                if (!(ok = mbar_wait_warp(&S.a_empty[ab], ((ia / NA) & 1) ^ 1, abort_flag, a.wait_ns))) break;
+                    __shfl_sync(FULL, *(volatile int *)&S.done[ab], 0) == DONE_ALL)
+                    break;
+                const int s = tb % NSTAGE, me = te % NMETA;
+                if (!(ok = TC_WAIT(w_prod, mbar_wait_warp(&S.b_empty[s], ((tb / NSTAGE) & 1) ^ 1, abort_flag, a.wait_ns) &&
+                           mbar_wait_warp(&S.m_empty[me], ((te / NMETA) & 1) ^ 1, abort_flag, a.wait_ns))))
+                    return;
                 if (elect_one()) {
-                    S.unit[ab] = iu;
-                    S.done[ab] = 0;
-                    const uint16_t *src = a.opR + (size_t)itile * a.tile_r + (RTN == 1 ? (iu & 1) * (TM * a.kv) : 0);
-                    mbar_arrive_expect_tx(&S.a_full[ab], RTN * a_bytes + (uint32_t)sizeof(MetaTile));
-                    bulk_g2s(S.A[ab * RTN], src, RTN * a_bytes, &S.a_full[ab]);
-                    bulk_g2s(&S.metaA[ab], a.metaR + itile, (uint32_t)sizeof(MetaTile), &S.a_full[ab]);
+                    S.ev[me] = ct;
+                    mbar_arrive_expect_tx(&S.m_full[me], (uint32_t)sizeof(MetaTile));
+                    bulk_g2s(&S.metaB[me], a.metaC + ct, (uint32_t)sizeof(MetaTile), &S.m_full[me]);
+                    mbar_arrive_expect_tx(&S.b_full[s], b_bytes);
+                    bulk_g2s(S.B[s], a.opC + (size_t)ct * a.tile_c, b_bytes, &S.b_full[s]);
                 }
                 __syncwarp();
-                ++ia;
-                while (m) {
-                    const int ct = ic + __ffs(m) - 1;
-                    m &= m - 1;
-                    if (PASS == TC_COUNT && a.min_pts > 0 &&
-                        __shfl_sync(FULL, *(volatile int *)&S.done[ab], 0) == DONE_ALL)
-                        break;
-                    const int s = tb % NSTAGE, me = te % NMETA;
-                    if (!(ok = mbar_wait_warp(&S.b_empty[s], ((tb / NSTAGE) & 1) ^ 1, abort_flag, a.wait_ns) &&
-                               mbar_wait_warp(&S.m_empty[me], ((te / NMETA) & 1) ^ 1, abort_flag, a.wait_ns)))
-                        break;
-                    if (elect_one()) {
-                        S.ev[me] = ct;
-                        mbar_arrive_expect_tx(&S.m_full[me], (uint32_t)sizeof(MetaTile));
-                        bulk_g2s(&S.metaB[me], a.metaC + ct, (uint32_t)sizeof(MetaTile), &S.m_full[me]);
-                        mbar_arrive_expect_tx(&S.b_full[s], b_bytes);
-                        bulk_g2s(S.B[s], a.opC + (size_t)ct * a.tile_c, b_bytes, &S.b_full[s]);
-                    }
-                    __syncwarp();
-                    ++tb;
-                    ++te;
-                }
-                if (!ok) break;
-                const int me = te % NMETA;
-                if (!(ok = mbar_wait_warp(&S.m_empty[me], ((te / NMETA) & 1) ^ 1, abort_flag, a.wait_ns))) break;
-                if (elect_one()) {
-                    S.ev[me] = EV_END;
-                    mbar_arrive(&S.m_full[me]);
-                }
-                __syncwarp();
+                ++tb;
                 ++te;
+            }
+            const int me = te % NMETA;
+            if (!(ok = mbar_wait_warp(&S.m_empty[me], ((te / NMETA) & 1) ^ 1, abort_flag, a.wait_ns))) return;
+            if (elect_one()) {
+                S.ev[me] = EV_END;
+                mbar_arrive(&S.m_full[me]);
+            }
+            __syncwarp();
+            ++te;
+        };
+        // A unit's udone word, one lane's reading for the warp (other CTAs write it).
+        auto done_of = [&](int iu) {
+            return PASS == TC_COUNT && a.min_pts > 0 ? __shfl_sync(FULL, db::ld_relaxed(a.udone + iu), 0) : 0;
+        };
+        if (a.items) {
+            // from the list, one at a time: the claim, the entry and the unit's
+            // state are each fetched an item ahead of their use
+            const int nlist = *a.nlist;
+            auto claim = [&]() {
+                int t = 0;
+                if (lane == 0) t = atomicAdd(a.ticket, 1);
+                return __shfl_sync(FULL, t, 0);
+            };
+            auto entry = [&](int t) { return t < nlist ? a.items[t] : make_int4(-1, 0, 0, 0); };
+            int4 e0 = entry(claim()), e1 = entry(claim());
+            int t2 = claim(), d0 = e0.x >= 0 ? done_of(e0.x) : 0;
+            while (e0.x >= 0 && ok) {
+                const int d1 = e1.x >= 0 ? done_of(e1.x) : 0;
+                const int4 e2 = entry(t2);
+                t2 = claim();
+                run(e0.x, e0.y, (unsigned)e0.z, d0);
+                e0 = e1;
+                d0 = d1;
+                e1 = e2;
+            }
+        } else {
+            for (int base = blockIdx.x; base < nitems && ok; base += (int)gridDim.x * 32) {
+                const int w = base + lane * (int)gridDim.x;
+                int u = 0, c0 = 0;
+                unsigned mask = 0;
+                if (w < nitems && w >= 0) mask = item_mask<PASS, RTN>(a, w, units, nct, u, c0);
+                unsigned live = __ballot_sync(FULL, mask != 0);
+                while (live && ok) {
+                    const int l = __ffs(live) - 1;
+                    live &= live - 1;
+                    const int iu = __shfl_sync(FULL, u, l), ic = __shfl_sync(FULL, c0, l);
+                    const unsigned m = __shfl_sync(FULL, mask, l);
+                    run(iu, ic, m, done_of(iu));
+                }
             }
         }
         if (ok) {
@@ -698,7 +754,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
             unsigned long long evaluated = 0;  // pairs of the tiles multiplied
             while (true) {
                 const int me = te % NMETA;
-                if (!(clean = mbar_wait(&S.m_full[me], (te / NMETA) & 1, abort_flag, a.wait_ns))) break;
+                if (!(clean = TC_WAIT(w_mma_b, mbar_wait(&S.m_full[me], (te / NMETA) & 1, abort_flag, a.wait_ns)))) break;
                 const int ev = *(volatile int *)&S.ev[me];
                 mbar_arrive(&S.m_empty[me]);
                 ++te;
@@ -711,12 +767,12 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                     continue;
                 }
                 if (!in_item) {
-                    if (!(clean = mbar_wait(&S.a_full[ab], (ia / NA) & 1, abort_flag, a.wait_ns))) break;
+                    if (!(clean = TC_WAIT(w_mma_b, mbar_wait(&S.a_full[ab], (ia / NA) & 1, abort_flag, a.wait_ns)))) break;
                     in_item = true;
                     row0 = *(volatile int *)&S.unit[ab] * TMU;
                 }
                 const int s = tb % NSTAGE;
-                if (!(clean = mbar_wait(&S.b_full[s], (tb / NSTAGE) & 1, abort_flag, a.wait_ns))) break;
+                if (!(clean = TC_WAIT(w_mma_b, mbar_wait(&S.b_full[s], (tb / NSTAGE) & 1, abort_flag, a.wait_ns)))) break;
                 const uint32_t b_addr = smem_u32(S.B[s]);
 #pragma unroll
                 for (int r = 0; r < RTN; ++r) {
@@ -724,7 +780,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                     // buffer serves one of them on every B tile; otherwise the
                     // buffers alternate between tiles
                     const int b = RTN == 2 ? r : (tb & 1), use = RTN == 2 ? tb : (tb >> 1);
-                    if (!(clean = mbar_wait(&S.t_empty[b], (use & 1) ^ 1, abort_flag, a.wait_ns))) break;
+                    if (!(clean = TC_WAIT(w_mma_t, mbar_wait(&S.t_empty[b], (use & 1) ^ 1, abort_flag, a.wait_ns)))) break;
                     tc_fence_after();
                     // the RTN row tiles lie back to back (a_bytes each) from the buffer's start
                     const uint32_t a_addr = smem_u32(S.A[ab * RTN]) + (uint32_t)r * a_bytes;
@@ -760,8 +816,8 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                 for (int ab = 0; ab < NA && ab < ia; ++ab)
                     mbar_wait(&S.a_empty[ab], ((ia - 1 - ab) / NA) & 1, abort_flag, a.wait_ns);
             }
-            if ((PASS == TC_COUNT || PASS == TC_UNION || PASS == TC_BORDER || PASS == TC_HOOK) && evaluated)
-                atomicAdd(a.ctr + DB_CTR_EVAL + (PASS == TC_HOOK ? TC_UNION : PASS), evaluated);
+            if ((PASS == TC_COUNT || PASS == TC_UNION || PASS == TC_BORDER || PASS == TC_ADJ) && evaluated)
+                atomicAdd(a.ctr + DB_CTR_EVAL + (PASS == TC_ADJ ? TC_UNION : PASS), evaluated);
             if (FOLDABLE && fold && blockIdx.x == 0) a.ctr[DB_CTR_TC_FOLD] = 1ull;
             // After an abort: one more commit, which arrives once every MMA this
             // thread issued has completed, and a bounded wait for it.
@@ -789,12 +845,13 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
         float beta_p = 0.f, alpha = 0.f, c_even = 0.f, c_odd = 0.f;
         int cnt = 0, prior = 0, bmin = INT_MAX, rootp = -2;
         bool told = false;           // count: this warp's rows are all done and the producer knows
+        bool first = true;           // count: no tile of the item seen (its prior counts are still on their way)
         unsigned best = 0;           // order: least squared distance so far (bits, column in the low 8)
         int besti = 0;               // and its pivot
         float reach = 0.f;           // cull: (r + eps)^2, an overestimate
         while (true) {
             const int me = te % NMETA;
-            if (!mbar_wait_warp(&S.m_full[me], (te / NMETA) & 1, abort_flag, a.wait_ns)) break;
+            if (!TC_WAIT(w_epi, mbar_wait_warp(&S.m_full[me], (te / NMETA) & 1, abort_flag, a.wait_ns))) break;
             const int ev = *(volatile int *)&S.ev[me];
             ++te;
             if (ev == EV_STOP) break;
@@ -817,6 +874,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                 } else {
                     beta_p = S.metaA[ab].beta[rin];
                 }
+                if (PASS == TC_LINK) reach = 4.f * (float)a.T;  // twice eps
                 alpha = beta_p - (float)a.T;  // |v_p|^2 - T, exact (1e30 for a masked row: never passes)
                 if (PASS == TC_COUNT && !BF16) {
                     // folded form: 1 - thr_f for the even (f = 0) and odd (f = 1)
@@ -829,6 +887,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                 if (PASS == TC_COUNT && a.min_pts > 0) {
                     prior = row_ok ? db::ld_relaxed(a.count + p) : a.min_pts;
                     told = false;
+                    first = true;
                 }
                 bmin = INT_MAX;
                 // union: a member of p's set (its parent, then the last root seen)
@@ -840,7 +899,8 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                 if (row_ok) {
                     if ((PASS == TC_COUNT || PASS == TC_VERIFY) && cnt) atomicAdd(a.count + p, cnt);
                     if (PASS == TC_BORDER && bmin != INT_MAX) atomicMin(a.border + p, bmin);
-                    if (PASS == TC_HOOK && bmin != INT_MAX) atomicMin(a.parent + p, bmin);
+                    // (a pivot is within reach of itself, unless rounding says otherwise)
+                    if (PASS == TC_LINK) a.key[p] = (int)min(best, (unsigned)p);
                     if (PASS == TC_ORDER) {
                         // class: the ratio of the squared distance to T, in powers of 4
                         const float ratio = __uint_as_float(best & 0x7fffff00u) / (float)max(a.T, 1);
@@ -865,24 +925,34 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
             const int ct = ev;
             const int b = RTN == 2 ? rsel : (tb & 1), use = RTN == 2 ? tb : (tb >> 1);
             ++tb;
-            if (!mbar_wait_warp(&S.t_full[b], use & 1, abort_flag, a.wait_ns)) break;
+            if (!TC_WAIT(w_epi, mbar_wait_warp(&S.t_full[b], use & 1, abort_flag, a.wait_ns))) break;
             tc_fence_after();
             const MetaTile &mc = S.metaB[me];
             const uint32_t tb_addr = tmem + lane_base + (uint32_t)(b * TN);
             if constexpr (Sh::kWide) {
-                // all 256 columns in eight groups of 32: the next group's TMEM load
-                // is in flight while this group is decided
-                uint32_t ga[32], gb[32];
+                // all 256 columns in four groups of 64: the next group's TMEM load is
+                // in flight while this group is decided, and the accumulator goes
+                // back to the issuer before the last group is (groups of 32, given
+                // back at the end: 385 instead of COUNT64 us for the count of
+                // 200,000 x 64, its warps waiting on tensor memory)
+                uint32_t ga[64], gb[64];
                 auto all_groups = [&](auto &&decide) {
-                    tmem_ld32_nowait(tb_addr, ga);
-                    tmem_wait_ld_dep(ga);
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        uint32_t(&cur)[32] = (i & 1) ? gb : ga;
-                        uint32_t(&nxt)[32] = (i & 1) ? ga : gb;
-                        if (i + 1 < 8) tmem_ld32_nowait(tb_addr + (uint32_t)(32 * (i + 1)), nxt);
-                        decide(cur, 32 * i);
-                        if (i + 1 < 8) tmem_wait_ld_dep(nxt);
+                    tmem_ld64_nowait(tb_addr, ga);
+                    tmem_wait_ld_dep64(ga);
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {
+                        tmem_ld64_nowait(tb_addr + (uint32_t)(128 * h + 64), gb);
+                        decide(ga, 128 * h);
+                        tmem_wait_ld_dep64(gb);
+                        if (h == 0) {
+                            tmem_ld64_nowait(tb_addr + 128, ga);
+                        } else {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(&S.t_empty[b]);
+                        }
+                        decide(gb, 128 * h + 64);
+                        if (h == 0) tmem_wait_ld_dep64(ga);
                     }
                 };
                 if constexpr (PASS == TC_COUNT) {
@@ -895,18 +965,18 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                         // otherwise: one saturating add per pair, one packed add per
                         // two pairs, no column data.  f = 0 for the first n_even columns.
                         const int ne = mc.n_even;
-                        all_groups([&](uint32_t(&g)[32], int col) {
-                            if (ne >= col + 32 || ne <= col) {
+                        all_groups([&](uint32_t(&g)[64], int col) {
+                            if (ne >= col + 64 || ne <= col) {
                                 const float cf = ne <= col ? c_odd : c_even;
 #pragma unroll
-                                for (int h = 0; h < 16; ++h)
+                                for (int h = 0; h < 32; ++h)
                                     acc[h & 3] =
                                         f2_add(acc[h & 3], f2_pack(__saturatef(__uint_as_float(g[2 * h]) + cf),
                                                                    __saturatef(__uint_as_float(g[2 * h + 1]) + cf)));
                             } else {  // the one group with columns of both parities
                                 const int bd = ne - col;
 #pragma unroll
-                                for (int h = 0; h < 16; ++h)
+                                for (int h = 0; h < 32; ++h)
                                     acc[h & 3] = f2_add(
                                         acc[h & 3],
                                         f2_pack(__saturatef(__uint_as_float(g[2 * h]) + (2 * h < bd ? c_even : c_odd)),
@@ -923,10 +993,10 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                         // rounding as before) and one packed add per two pairs.
                         const float c1 = 1.f - alpha;
                         const unsigned long long m2 = f2_pack(-2.f, -2.f);
-                        all_groups([&](uint32_t(&g)[32], int col) {
+                        all_groups([&](uint32_t(&g)[64], int col) {
                             const float *bet = mc.beta + col;
 #pragma unroll
-                            for (int j8 = 0; j8 < 4; ++j8) {
+                            for (int j8 = 0; j8 < 8; ++j8) {
                                 const float4 ba = *reinterpret_cast<const float4 *>(bet + 8 * j8);
                                 const float4 bb = *reinterpret_cast<const float4 *>(bet + 8 * j8 + 4);
                                 const float bq[8] = {ba.x, ba.y, ba.z, ba.w, bb.x, bb.y, bb.z, bb.w};
@@ -950,12 +1020,12 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                     const unsigned long long m2 = f2_pack(-2.f, -2.f), bp = f2_pack(beta_p, beta_p);
                     float lo = 3.0e38f;
                     unsigned least = 0xffffffffu;
-                    all_groups([&](uint32_t(&g)[32], int col) {
+                    all_groups([&](uint32_t(&g)[64], int col) {
 #pragma unroll
-                        for (int j4 = 0; j4 < 8; ++j4) {
+                        for (int j4 = 0; j4 < 16; ++j4) {
                             const float4 b4 = *reinterpret_cast<const float4 *>(mc.beta + col + 4 * j4);
                             unsigned long long q01 = f2_pack(b4.x, b4.y), q23 = f2_pack(b4.z, b4.w);
-                            if (PASS == TC_ORDER) {
+                            if (PASS != TC_CULL) {
                                 q01 = f2_add(q01, bp);
                                 q23 = f2_add(q23, bp);
                             }
@@ -964,7 +1034,11 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                                              q01), w[0], w[1]);
                             f2_unpack(f2_fma(f2_pack(__uint_as_float(g[4 * j4 + 2]), __uint_as_float(g[4 * j4 + 3])),
                                              m2, q23), w[2], w[3]);
-                            if (PASS == TC_ORDER) {
+                            if (PASS == TC_LINK) {
+#pragma unroll
+                                for (int h = 0; h < 4; ++h)
+                                    if (w[h] <= reach) least = min(least, (unsigned)(ct * TN + col + 4 * j4 + h));
+                            } else if (PASS == TC_ORDER) {
                                 // squared distances (>= 0, so they order as integers) with
                                 // the column in the low 8 bits: the nearest pivot up to 2^-15
                                 // of its distance, which is all a sort key needs
@@ -978,6 +1052,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                             }
                         }
                     });
+                    if (PASS == TC_LINK) best = min(best, least);
                     if (PASS == TC_ORDER && least < best) {
                         best = least;
                         besti = ct * TN + (int)(least & 255u);
@@ -1075,10 +1150,11 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                         mx = -fminf(fminf(fminf(nv[0], nv[1]), fminf(nv[2], nv[3])),
                                     fminf(fminf(nv[4], nv[5]), fminf(nv[6], nv[7])));
                     }
-                    // hook: columns before the row, and only until one is found (they ascend)
-                    const bool need = row_ok && mx >= thr &&
-                                      (PASS != TC_HOOK || (bmin == INT_MAX && ct * TN + cb < p));
-                    if (!__any_sync(FULL, need)) continue;
+                    const bool need = row_ok && mx >= thr;
+                    if (!__any_sync(FULL, need)) {
+                        if (PASS == TC_ADJ && row_ok) a.adj[(size_t)p * 8 + (cb >> 5)] = 0u;
+                        continue;
+                    }
                     if (PASS == TC_UNION && !hints) {
                         // the parents loaded at the tile's start, for this warp's columns
                         // (the warps of the other lane quadrants that share them write
@@ -1096,7 +1172,8 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                     // Only the residues j mod 8 whose minimum passes the filter in
                     // some lane of the warp are scanned (warp-uniform branches, so the
                     // column indices stay compile-time constants).
-                    unsigned mask = 0;
+                    unsigned mask = 0;  // possible neighbours
+                    unsigned sure = 0;  // BF16: those beyond the rounding band, neighbours without a recheck
                     {
                         unsigned rm = 0;
                         if (need) {
@@ -1104,9 +1181,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                             for (int i = 0; i < 8; ++i) rm |= (unsigned)(-nv[i] >= thr) << i;
                         }
                         const unsigned um = __reduce_or_sync(FULL, rm);
-                        // merge: columns after the row; hook: columns before it
-                        const int col_lim = PASS == TC_UNION ? p - ct * TN : -1;
-                        const int col_end = PASS == TC_HOOK ? p - ct * TN : INT_MAX;
+                        const int col_lim = PASS == TC_UNION ? p - ct * TN : -1;  // merge: columns after the row
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
                             if (!((um >> i) & 1u)) continue;
@@ -1116,30 +1191,21 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                                 const float w1 = fmaf(2.f, __uint_as_float(g[j]), -mc.beta[cb + j]);
                                 bool c = need && (BF16 ? (w1 + rho2 >= alpha) : (w1 >= alpha));
                                 if (PASS == TC_UNION) c = c && colroot[cb + j] != rootp;
-                                mask |= (unsigned)(c && (cb + j) > col_lim && (cb + j) < col_end) << j;
+                                c = c && (cb + j) > col_lim;
+                                mask |= (unsigned)c << j;
+                                if (BF16) sure |= (unsigned)(c && w1 - rho2 >= alpha) << j;
                             }
                         }
                     }
-                    unsigned nbm = mask;  // confirmed neighbours among the mask
-                    if (BF16) {
-                        nbm = 0;
-                        for (unsigned mm = mask; mm; mm &= mm - 1) {
+                    unsigned nbm = BF16 ? sure : mask;  // confirmed neighbours among the mask
+                    if (BF16)
+                        for (unsigned mm = mask & ~sure; mm; mm &= mm - 1) {
                             const int j = __ffs((int)mm) - 1;
-                            // recompute 2G - |v_q|^2 for column j from the accumulator copy in g
-                            float gj = 0.f;
-#pragma unroll
-                            for (int k = 0; k < 32; ++k)
-                                if (k == j) gj = __uint_as_float(g[k]);
-                            const float wj = fmaf(2.f, gj, -mc.beta[cb + j]);
-                            const int res = decide_candidate<BF16>(wj, alpha, rho2, a.v16, K, p, ct * TN + cb + j, a.T);
-                            band_cnt += res >> 1;
-                            if (!(res & 1)) continue;
-                            nbm |= 1u << j;
-                            if (PASS == TC_HOOK) break;  // ascending columns: the first is the smallest
+                            ++band_cnt;
+                            nbm |= (unsigned)(exact_sqdist(a.v16, K, p, ct * TN + cb + j) <= a.T) << j;
                         }
-                    }
                     if (PASS == TC_COUNT) cnt += __popc(nbm);
-                    if (PASS == TC_HOOK && nbm) bmin = min(bmin, ct * TN + cb + __ffs((int)nbm) - 1);
+                    if (PASS == TC_ADJ && row_ok) a.adj[(size_t)p * 8 + (cb >> 5)] = nbm;
                     if (PASS == TC_BORDER)
                         for (unsigned mm = nbm; mm; mm &= mm - 1) bmin = min(bmin, mc.idx[cb + __ffs((int)mm) - 1]);
                     if (PASS == TC_UNION) {
@@ -1153,32 +1219,54 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                         // itself, whose link another thread may have set), so later
                         // tiles find the forest flat and a converged cluster costs one
                         // shared-memory compare per pair.
-                        for (unsigned mm = nbm; mm; mm &= mm - 1) {
-                            const int j = cb + __ffs((int)mm) - 1;
-                            const int hq = colroot[j];
-                            if (hq == rootp || hq == hm0 || hq == hm1) continue;
-                            const int q = ct * TN + j;
-                            const int rt = unite_root(a.parent, p, q, a.status);
-                            if (rt >= 0) {
-                                if (q != rt) db::st_relaxed(a.parent + q, rt);
-                                if (p != rt && rt != rootp) db::st_relaxed(a.parent + p, rt);
+                        // Lanes that would join the same two sets leave it to one of
+                        // them: a tile pair of two groups is one union a warp.
+                        unsigned left = nbm;
+                        while (true) {
+                            int j = -1, hq = 0;
+                            while (left) {
+                                const int k = cb + __ffs((int)left) - 1;
+                                left &= left - 1;
+                                hq = colroot[k];
+                                if (hq == rootp || hq == hm0 || hq == hm1) continue;
+                                j = k;
+                                break;
                             }
-                            hm0 = hq;
-                            if (rt != rootp) hm1 = rootp;
-                            rootp = rt;
-                            colroot[j] = rt;
+                            if (!__any_sync(FULL, j >= 0)) break;
+                            const unsigned long long key =
+                                j >= 0 ? ((unsigned long long)(unsigned)rootp << 32) | (unsigned)hq : ~(unsigned long long)lane;
+                            const int leader = __ffs((int)__match_any_sync(FULL, key)) - 1;
+                            int rt = 0;
+                            if (j >= 0 && lane == leader) {
+                                const int q = ct * TN + j;
+                                rt = unite_sets(a.parent, rootp, hq, a.status);
+                                if (rt >= 0) {
+                                    if (q != rt) db::st_relaxed(a.parent + q, rt);
+                                    if (p != rt && rt != rootp) db::st_relaxed(a.parent + p, rt);
+                                }
+                            }
+                            rt = __shfl_sync(FULL, rt, leader);
+                            if (j >= 0) {
+                                hm0 = hq;
+                                if (rt != rootp) hm1 = rootp;
+                                rootp = rt;
+                                colroot[j] = rt;
+                            }
                         }
                     }
                 }
             }
-            tc_fence_before();
-            if (PASS == TC_COUNT && a.min_pts > 0 && !told && __all_sync(FULL, prior + cnt >= a.min_pts)) {
-                told = true;
-                if (lane == 0) atomicOr(&S.done[ab], 1 << ew);
+            if (!Sh::kWide) tc_fence_before();
+            if (PASS == TC_COUNT && a.min_pts > 0 && !told) {
+                if (!first && __all_sync(FULL, prior + cnt >= a.min_pts)) {
+                    told = true;
+                    if (lane == 0) atomicOr(&S.done[ab], 1 << ew);
+                }
+                first = false;
             }
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(&S.t_empty[b]);
+                if (!Sh::kWide) mbar_arrive(&S.t_empty[b]);
                 mbar_arrive(&S.m_empty[me]);
             }
         }
@@ -1187,6 +1275,21 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
         if (maxerr) atomicMax(a.ctr + 8, (unsigned long long)maxerr);
     }
 
+#ifdef DB_TC_WAIT_STATS
+    // slots 9..13 (count), 20..24 (merge), 25..29 (border): producer, MMA issuer
+    // on events and operands, MMA issuer on accumulators, one epilogue warp,
+    // issuer total
+    if (PASS == TC_COUNT || PASS == TC_UNION || PASS == TC_BORDER) {
+        unsigned long long *ws = a.ctr + (PASS == TC_COUNT ? 9 : (PASS == TC_UNION ? 20 : 25));
+        if (threadIdx.x == 0) atomicAdd(ws, (unsigned long long)w_prod);
+        if (warp == 1 && w_mma_b) {
+            atomicAdd(ws + 1, (unsigned long long)w_mma_b);
+            atomicAdd(ws + 2, (unsigned long long)w_mma_t);
+            atomicAdd(ws + 4, (unsigned long long)(clock64() - t_start));
+        }
+        if (threadIdx.x == 64) atomicAdd(ws + 3, (unsigned long long)w_epi);
+    }
+#endif
     // ---------------- teardown ----------------
     tc_fence_before();
     __syncthreads();
@@ -1470,60 +1573,19 @@ __global__ void __launch_bounds__(256) tc_pack_kernel(PackArgs a) {
     }
 }
 
-// Each pivot under the first pivot before it within twice eps (a warp per
-// pivot, 64 earlier pivots staged at a time for the block's eight; a search
-// stops at its first hit), and the bucket sizes cleared.
-__global__ void __launch_bounds__(256) tc_pivot_link_kernel(const int16_t *__restrict__ v16, int K, int P, int T4,
-                                                            int *__restrict__ link, int *__restrict__ hist, int nhist) {
-    db::wait_prior_grid();  // started as a programmatic dependent
-    db::allow_next_grid();
-    __shared__ int rows[64][33], mine[8][33];  // two units a word; rows start in different banks
-    const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x), lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int k = t >> 5, kw = K / 2, kmax = blockIdx.x * 8 + 7;  // P is a multiple of 8
-    const int *src = reinterpret_cast<const int *>(v16);
-    for (int e = t; e < nhist; e += (int)(gridDim.x * blockDim.x)) hist[e] = 0;
-    for (int c = lane; c < kw; c += 32) mine[wid][c] = src[k * kw + c];
-    int to = k;
-    bool found = false;
-    for (int j0 = 0; j0 < kmax; j0 += 64) {
-        __syncthreads();
-        for (int e = threadIdx.x; e < 64 * kw; e += 256) {
-            const int r = e / kw, c = e - r * kw;
-            rows[r][c] = j0 + r < P ? src[(j0 + r) * kw + c] : 0;
-        }
-        __syncthreads();
-        if (!found) {
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = j0 + 32 * h + lane;
-                int D = 0;
-                for (int c = 0; c < kw; ++c) {
-                    const int x = mine[wid][c], y = rows[32 * h + lane][c];
-                    const int d0 = (int)(int16_t)(x & 0xffff) - (int)(int16_t)(y & 0xffff), d1 = (x >> 16) - (y >> 16);
-                    D += d0 * d0 + d1 * d1;
-                }
-                const unsigned hit = __ballot_sync(FULL, j < k && D <= T4);
-                if (hit && !found) {
-                    to = j0 + 32 * h + __ffs(hit) - 1;
-                    found = true;
-                }
-            }
-        }
-        if (__syncthreads_and(found)) break;
-    }
-    if (lane == 0) link[k] = to;
-}
-
 // Rank of each pivot in the order (group, pivot), groups being the trees of
-// the links: the pivots of one group of points, and so their buckets, lie side
-// by side (a bitonic sort by one block of P threads).
+// the links (each pivot to the first one within twice eps): the pivots of one
+// group of points, and so their buckets, lie side by side (a bitonic sort by
+// one block of P threads).  Also clears the bucket sizes.
 __global__ void __launch_bounds__(1024) tc_pivot_rank_kernel(const int *__restrict__ link, int P,
-                                                             int *__restrict__ prank) {
+                                                             int *__restrict__ prank, int *__restrict__ hist,
+                                                             int nhist) {
     db::wait_prior_grid();  // started as a programmatic dependent
     db::allow_next_grid();
     __shared__ int up[1024];
     __shared__ unsigned s[1024];
     const int t = threadIdx.x;
+    for (int e = t; e < nhist; e += (int)blockDim.x) hist[e] = 0;
     up[t] = link[t];
     __syncthreads();
     int r = t;
@@ -1613,6 +1675,55 @@ __global__ void __launch_bounds__(256) tc_core_kernel(int n, int min_pts, const 
         tag[tile] = any ? -1 : -2;
         rowneed[tile] = anyn;
     }
+}
+
+// The core points of a tile joined among themselves, from the adjacency words
+// of the tile with itself: every row under its first neighbour, flattened, then
+// smaller labels of any neighbour until none is left, in shared memory.  The
+// merge then only crosses tiles (200,000 x 64: with each row only hooked under
+// its first earlier neighbour some 55 sets a tile were left, and the near tiles
+// took 238 us).  A block per tile; sets the tile's tag.
+__global__ void __launch_bounds__(256) tc_join_kernel(int n, const uint8_t *__restrict__ core,
+                                                      const uint4 *__restrict__ adj, int *__restrict__ parent,
+                                                      int *__restrict__ tag) {
+    db::wait_prior_grid();  // started as a programmatic dependent
+    db::allow_next_grid();
+    __shared__ int lab[TN];
+    const int tile = blockIdx.x, t = threadIdx.x, p = tile * TN + t;
+    const bool is = p < n && core[p];
+    if (!__syncthreads_or(is)) return;  // the tag says so already
+    unsigned m[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (is) {
+        const uint4 x = adj[(size_t)p * 2], y = adj[(size_t)p * 2 + 1];
+        m[0] = x.x, m[1] = x.y, m[2] = x.z, m[3] = x.w, m[4] = y.x, m[5] = y.y, m[6] = y.z, m[7] = y.w;
+    }
+    int l = t;
+#pragma unroll
+    for (int k = 7; k >= 0; --k)
+        if (m[k]) l = 32 * k + __ffs((int)m[k]) - 1;
+    lab[t] = min(l, t);
+    __syncthreads();
+    while (true) {
+        l = t;
+        while (lab[l] < l) l = lab[l];  // labels point to earlier rows
+        __syncthreads();
+        lab[t] = l;
+        if (__syncthreads_count(is && l == t) <= 1) break;
+        int least = l;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            for (unsigned w = m[k]; w; w &= w - 1) least = min(least, lab[32 * k + __ffs((int)w) - 1]);
+        const bool moved = least < l;
+        if (!__syncthreads_or(moved)) break;
+        if (moved) {
+            atomicMin(&lab[l], least);  // the group's first row, too
+            atomicMin(&lab[t], least);
+        }
+        __syncthreads();
+    }
+    if (is) parent[p] = tile * TN + l;
+    const int roots = __syncthreads_count(is && l == t);
+    if (is && l == t && roots == 1) tag[tile] = p;
 }
 
 // Every core point straight under its root, and per tile the root its core
@@ -1801,31 +1912,30 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
         pp.n_src = n;
         pp.op = w.opNon;
         pp.meta = mneed;
-        pp.v16 = w.v16;
         launch_dependent(tc_pack_kernel, P / TN, 256, st, pp);
         w.marks->kernel("tc_pack_pivots", st);
-        launch_dependent(tc_pivot_link_kernel, P / 8, 256, st, w.v16, K, P,
-                         (int)std::min<int64_t>(4 * Tc, INT32_MAX), link, hist, nhist);
+        TcArgs o = a;
+        o.opR = o.opC = w.opNon;
+        o.metaR = o.metaC = mneed;
+        o.nR = o.nC = P;
+        o.kv = K;
+        o.tile_r = o.tile_c = TN * K;
+        o.ct_chunk = P / TN;
+        o.rel_lo = 0;
+        o.rel_hi = 1;
+        o.key = link;
+        if ((e = launch_pass_t<TC_LINK, false>(o, sms, st))) return e;
         w.marks->kernel("tc_pivot_link", st);
-        launch_dependent(tc_pivot_rank_kernel, 1, P, st, link, P, prank);
+        launch_dependent(tc_pivot_rank_kernel, 1, P, st, link, P, prank, hist, nhist);
         w.marks->kernel("tc_pivot_rank", st);
         PackArgs pu = pk;  // all points in index order
         pu.op = w.opCore;
         pu.meta = mcore;
         launch_dependent(tc_pack_kernel, nt, 256, st, pu);
         w.marks->kernel("tc_prep", st);
-        TcArgs o = a;
         o.opR = w.opCore;
         o.metaR = mcore;
-        o.opC = w.opNon;
-        o.metaC = mneed;
         o.nR = n;
-        o.nC = P;
-        o.kv = K;
-        o.tile_r = o.tile_c = TN * K;
-        o.ct_chunk = P / TN;
-        o.rel_lo = 0;
-        o.rel_hi = 1;
         o.n_piv = P;
         o.prank = prank;
         o.key = key;
@@ -1911,7 +2021,31 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     a.ct_chunk = chunk_tiles(bf16 ? units1 : nt, nt, sms);
     a.rel_lo = 0;
     a.rel_hi = (nt + a.ct_chunk - 1) / a.ct_chunk;
+    // opCore is free from here on: adjacency words, then the item list (when it fits)
+    a.adj = reinterpret_cast<unsigned *>(w.opCore);
+    int4 *list = reinterpret_cast<int4 *>(w.opCore + (size_t)nt * TN * 16);
+    const int64_t list_cap = (w.tc_cap_pad * 64 - (int64_t)nt * TN * 16) / 8;
+    int next_list = 1;  // tc_lens[1..6]: length and ticket of up to three lists, cleared above
+    auto use_list = [&](auto pass) -> cudaError_t {
+        constexpr int PASS = decltype(pass)::value;
+        const int64_t units = bf16 || PASS == TC_UNION ? (n + TM - 1) / TM : nt, nit = units * (a.rel_hi - a.rel_lo);
+        a.items = nullptr;
+        if (!sorted || nit > list_cap) return cudaSuccess;
+        a.nlist = w.tc_lens + next_list++;
+        a.ticket = w.tc_lens + next_list++;
+        TcArgs q = a;
+        q.items = list;
+        const int blocks = (int)((nit + 255) / 256);
+        if constexpr (PASS == TC_UNION) launch_dependent(tc_items_kernel<PASS, 1>, blocks, 256, st, q);
+        else if (bf16) launch_dependent(tc_items_kernel<PASS, 1>, blocks, 256, st, q);
+        else launch_dependent(tc_items_kernel<PASS, 2>, blocks, 256, st, q);
+        w.marks->kernel("tc_items", st);
+        a.items = list;
+        return cudaGetLastError();
+    };
+    if ((e = use_list(std::integral_constant<int, TC_COUNT>{}))) return e;
     if ((e = launch_pass<TC_COUNT>(a, bf16, sms, st))) return e;
+    a.items = nullptr;
     w.marks->kernel("tc_count", st);
     a.stall = 0;
     a.wait_ns = 2000000000ull;
@@ -1919,19 +2053,19 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
                      mneed, w.tc_tag, w.tc_rowneed);
     w.marks->kernel("core_init", st);
 
-    // pass 2: union of core-core neighbours.  First each core point under its
-    // first core neighbour of its own tile; then the near tiles; then the rest,
-    // most of which the sets found so far skip.
+    // pass 2: union of core-core neighbours.  First inside every tile; then the
+    // near tiles; then the rest, most of which the sets found so far skip.
     a.metaR = a.metaC = mcore;
     a.fold = 0;
     const int ch_union = chunk_tiles(units1, nt, sms), nch = (nt + ch_union - 1) / ch_union;
     a.ct_chunk = ch_union;
     a.rel_lo = 0;
     a.rel_hi = 1;
-    if ((e = launch_pass<TC_HOOK>(a, bf16, sms, st))) return e;
-    w.marks->kernel("tc_hook", st);
-    launch_dependent(tc_tag_kernel, nt, 256, st, n, w.core, w.parent, w.tc_tag);
-    w.marks->kernel("tc_tag", st);
+    if ((e = launch_pass<TC_ADJ>(a, bf16, sms, st))) return e;
+    w.marks->kernel("tc_adj", st);
+    launch_dependent(tc_join_kernel, nt, 256, st, n, w.core, reinterpret_cast<const uint4 *>(a.adj), w.parent,
+                     w.tc_tag);
+    w.marks->kernel("tc_join", st);
     // (the tiles right after a row unit's own first: they link most of what
     // belongs together, and the tags then skip most of the rest)
     a.near_lo = 0;
@@ -1946,7 +2080,9 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
         a.near_hi = nt;
         a.rel_lo = 0;
         a.rel_hi = nch;
+        if ((e = use_list(std::integral_constant<int, TC_UNION>{}))) return e;
         if ((e = launch_pass<TC_UNION>(a, bf16, sms, st))) return e;
+        a.items = nullptr;
         w.marks->kernel("tc_union", st);
     }
 
@@ -1956,6 +2092,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     a.ct_chunk = chunk_tiles(bf16 ? units1 : nt, nt, sms);
     a.rel_lo = 0;
     a.rel_hi = (nt + a.ct_chunk - 1) / a.ct_chunk;
+    if ((e = use_list(std::integral_constant<int, TC_BORDER>{}))) return e;
     if ((e = launch_pass<TC_BORDER>(a, bf16, sms, st))) return e;
     w.marks->kernel("tc_border", st);
 

@@ -127,8 +127,8 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
 }
 
 // Out of line: keeps the union-find loops out of the tile's registers.
-static __device__ __noinline__ int unite_rows(int *parent, int p, int q, unsigned *status) {
-    return db::uf_unite_root(parent, p, q, status);
+static __device__ __noinline__ int unite_sets(int *parent, int x, int y, unsigned *status) {
+    return db::uf_unite_root(parent, x, y, status);
 }
 
 // The state of one work item's 32 rows.  Lane l holds rows l/4 + 8 i, i < 4,
@@ -206,7 +206,7 @@ struct Item {
                         const int old = i < 2 ? (i ? root[1] : root[0]) : (i == 2 ? root[2] : root[3]);
                         const int hq = e ? hq1 : hq0;
                         if (hq == old) continue;
-                        const int r = unite_rows(R.parent, row0 + (lane >> 2) + 8 * i, col + e, R.status);
+                        const int r = unite_sets(R.parent, old, hq, R.status);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             if (root[k] == old || root[k] == hq) root[k] = r;
@@ -218,7 +218,7 @@ struct Item {
         }
         // both tiles' core rows are one set each: one hit joins them
         if ((PASS == WT_NEAR || PASS == WT_FAR) && __any_sync(FULL, any) && lane == 0)
-            unite_rows(R.parent, mytag, ctag, R.status);
+            unite_sets(R.parent, mytag, ctag, R.status);
     }
 
     // Neighbours counted so far of row i of this lane (the same in its quad).
