@@ -53,13 +53,14 @@ size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
     w.status = c.take<unsigned>(4);
     w.ctr = c.take<unsigned long long>(DB_NCTR);
     const bool grid = o.grid != DBSCAN_GRID_OFF && o.max_d >= 1;
+    w.rk = nullptr;
     if (grid) {
         int bits = 10;
         while ((int64_t(1) << bits) < 2 * n) ++bits;
         w.hcap = int64_t(1) << bits;
         w.hbits = bits;
+        w.hcount = c.take<int32_t>(w.hcap);  // right behind status and ctr: one clear covers all three
         w.hkey = c.take<uint32_t>(w.hcap);
-        w.hcount = c.take<int32_t>(w.hcap);
         w.hpack = c.take<int2>(w.hcap);
         w.occ_cap = std::max<int64_t>(int64_t(1) << 15, 4 * n);
         w.occ = c.take<uint32_t>(w.occ_cap);
@@ -76,10 +77,14 @@ size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
         w.cell_mid = c.take<float4>(n);
         w.cell_key = c.take<uint32_t>(n);
         const int dg = std::min(o.max_d, 3);
-        w.noff_cap = dg == 1 ? 4 : (dg == 2 ? 24 : 124);
+        w.noff_cap = dg == 1 ? 8 : (dg == 2 ? 24 : 124);
         w.nbr = c.take<int32_t>((size_t)n * w.noff_cap);
         w.ncnt = c.take<int32_t>(n);
         w.cell_cand = c.take<int32_t>(n);
+        if (dg == o.max_d || !exact_d) {  // the eps-grid's (d <= 3)
+            w.rk = c.take<uint2>(w.occ_cap);
+            w.rg_part = c.take<unsigned long long>(std::max(w.hcap, w.occ_cap) / 2048 + 8);
+        }
     } else {
         w.hcap = 0;
         w.noff_cap = 0;
@@ -176,27 +181,32 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     cudaStream_t st = plan->stream;
     const bool sync = o.synchronous || stats;
     const bool want_grid = d <= 3 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0;
-    const bool small = want_grid && n <= kGridSmallMaxN;  // one kernel, which clears what it needs
-    if (!small && o.synchronous && cudaMemsetAsync(plan->w.status, 0, sizeof(unsigned), st) != cudaSuccess)
+    GridGeom g;
+    const bool eps_grid = want_grid && grid_geometry(d, Tc, n, &g);
+    // these clear what they need themselves
+    const bool small = eps_grid && n <= kGridSmallMaxN, rows = eps_grid && !small && grid_rows_serves(plan->w, g, n);
+    const bool clears = small || rows;
+    if (!clears && o.synchronous && cudaMemsetAsync(plan->w.status, 0, sizeof(unsigned), st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
-    if (!small && cudaMemsetAsync(plan->w.ctr, 0, sizeof(unsigned long long) * DB_NCTR, st) != cudaSuccess)
+    if (!clears && cudaMemsetAsync(plan->w.ctr, 0, sizeof(unsigned long long) * DB_NCTR, st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
     if (stats) cudaEventRecord(plan->ev0, st);
     plan->marks.begin(st);
 
     const bool exact = counts_out != nullptr;
     int path;
-    GridGeom g;
     cudaError_t err;
     // the projected grid (4 <= d <= 8) needs the eps-grid's arrays and row stride >= 8 (4 for d = 4)
     const bool want_mid = d >= 4 && d <= 8 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0 &&
                           plan->w.dp_cap >= (d <= 4 ? 4 : 8);
     if (o.grid == DBSCAN_GRID_ON && !(want_grid || want_mid)) return DBSCAN_ERR_UNSUPPORTED;
-    if (want_grid && grid_geometry(d, Tc, n, &g)) {
+    if (eps_grid) {
         path = DBSCAN_PATH_GRID;
         err = small ? launch_grid_small(plan->w, g, points, n, min_pts, exact, o.label_mode == DBSCAN_LABEL_COMPACT,
                                         stats != nullptr, o.synchronous, labels, counts_out, core_out, st)
-                    : launch_grid_path(plan->w, g, points, n, min_pts, exact, labels, counts_out, core_out, st);
+              : rows ? launch_grid_rows(plan->w, g, points, n, min_pts, exact, stats != nullptr, o.synchronous, labels,
+                                        counts_out, core_out, st)
+                     : launch_grid_path(plan->w, g, points, n, min_pts, exact, labels, counts_out, core_out, st);
     } else if (want_mid && mid_geometry(d, Tc, n, &g)) {
         path = DBSCAN_PATH_GRID_PROJECTED;
         err = launch_mid_grid_path(plan->w, g, points, n, d, min_pts, exact, labels, counts_out, core_out, st);
@@ -228,7 +238,7 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
         }
     }
     if (!err && !small && o.label_mode == DBSCAN_LABEL_COMPACT) err = launch_compact(plan->w, n, labels, st);
-    if (!err && !small && stats && (path == DBSCAN_PATH_GRID || path == DBSCAN_PATH_GRID_PROJECTED))
+    if (!err && !clears && stats && (path == DBSCAN_PATH_GRID || path == DBSCAN_PATH_GRID_PROJECTED))
         err = launch_grid_candidates(plan->w, g, n, path == DBSCAN_PATH_GRID_PROJECTED, st);
     if (err != cudaSuccess) {
         std::fprintf(stderr, "dbscan: launch failed: %s\n", cudaGetErrorString(err));

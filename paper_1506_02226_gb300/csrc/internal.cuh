@@ -238,6 +238,8 @@ struct DbWork {
     int32_t *ncnt;          // (adjacent count << 16) | count [cap_n]
     int32_t *cell_cand;     // points in the cells of each neighbour list [cap_n]
     int32_t noff_cap;
+    uint2 *rk;              // cells in key order: per 32 cells {occupied cells before, bits} [occ_cap]
+    unsigned long long *rg_part;  // block totals of its scans
     // tensor-core path (max_d >= 16)
     int64_t tc_cap_pad;     // rows of each packed operand (cap_n rounded up to 256, plus 256)
     int16_t *v16;           // centred units by position, row stride K (BF16 recheck, verification) [cap_n * 64]
@@ -300,6 +302,13 @@ constexpr int kGridSmallMaxN = 4096;
 cudaError_t launch_grid_small(const DbWork &w, const GridGeom &g, const float *x, int64_t n, int32_t min_pts, bool exact,
                               bool compact, bool stats, bool reset, int32_t *labels, int32_t *counts_out,
                               uint8_t *core_out, cudaStream_t st);
+// The eps-grid run with cells in key order (grid_rows.cu): whether it serves an
+// instance, and the run; clears the run's counters, and the status word when
+// `reset` is set.
+bool grid_rows_serves(const DbWork &w, const GridGeom &g, int64_t n);
+cudaError_t launch_grid_rows(const DbWork &w, const GridGeom &g, const float *x, int64_t n, int32_t min_pts, bool exact,
+                             bool stats, bool reset, int32_t *labels, int32_t *counts_out, uint8_t *core_out,
+                             cudaStream_t st);
 // Ordered candidate pairs of a grid run (own cell listed: the projected grid).
 cudaError_t launch_grid_candidates(const DbWork &w, const GridGeom &g, int64_t n, bool own_cell_listed,
                                    cudaStream_t st);
