@@ -20,16 +20,21 @@
 // take grid.cu.
 //
 // Kernels: prep, scans (2 kernels direct, 5 with the bitmap), scatter beside
-// rows (the range lists), count, border beside the merge, labels.  The merge's
-// forest is over cells, linked towards smaller representatives, so a root's
-// representative is its cluster's label:
-//   hook     every cell with cores under the neighbouring cell with the smallest
-//            representative whose central core point is within eps of its own:
-//            plain stores, no search;
+// rows (the range lists), count, border beside the merge, roots, labels.  The
+// merge's forest is over cells, linked towards smaller ids:
+//   hook     every cell with cores under the first neighbouring cell before it
+//            whose central core point is within eps of its own: plain stores, no
+//            search.  Only cells with no such neighbour stay roots, a few at the
+//            lower rim of each group (under the neighbour with the smallest
+//            representative, every local minimum of the representatives stayed
+//            one, and the union took 138 us for 500,000 points in space);
 //   flatten  every cell straight under its root;
-//   union    cell pairs whose roots still differ: central points, then a search
-//            of the core pairs by the warp; most pairs are skipped by one
-//            comparison.
+//   union    cell pairs whose roots still differ: central points, then, when the
+//            cells hold few pairs, all of them, a lane per cell pair; most cell
+//            pairs are skipped by one comparison;
+//   search   what is left, a list, a warp per cell pair (searched where they
+//            were found, a cell with a score of them held up its warp: the merge
+//            of 500,000 points in space took 141 us instead of MERGE_NOW).
 #include <algorithm>
 #include <climits>
 #include <type_traits>
@@ -40,6 +45,8 @@
 namespace {
 
 constexpr int64_t kMaxN = int64_t(1) << 22;
+constexpr int kWalkThreads = 64; // count and border blocks: a warp next to a tight blob holds up few others
+constexpr int kLaneTests = 64;   // merge: pairs of two cells that a single lane tests
 constexpr int kScanTile = 2048;  // entries per block of a scan: 256 threads x 8
 
 struct RowGeom {
@@ -56,7 +63,7 @@ struct RowArgs {
     const unsigned long long *ctr0;  // (cells << 32) | points
     const uint2 *rk;          // bitmap: {occupied cells before the word, its bits}
     const int *idx;           // direct: occupied cells before each key
-    const unsigned *cell_key; // by id
+    const unsigned *cell_at;  // by id: cell coordinates cx | cy << 10 | cz << 20
     int *start;               // first position of each cell's points, [cells + 1]
     int4 *rows;               // {first id, end id, first position, end position}, stride g.nrows
     int *nent, *cand;         // entries of a cell's list, points in them
@@ -66,10 +73,19 @@ struct RowArgs {
     int *rep;                 // smallest core index of each cell
     unsigned long long *mid;  // (squared distance to the centre << 32) | packed point
     int *par;                 // forest of cells
+    int *least;               // smallest representative of each set, at its root
     int *bord;
+    int2 *pairs;              // merge: cell pairs left to a warp each, and their number
+    int *npairs, pair_cap;
     unsigned *status;
     unsigned long long *ev;   // pair tests: [0] count, [1] merge, [2] border
 };
+
+// Cell coordinates of a key (the divisions are made once per cell).
+__device__ __forceinline__ unsigned cell_of_key(unsigned key, int G) {
+    const unsigned row = key / (unsigned)G, cx = key - row * (unsigned)G, cz = row / (unsigned)G, cy = row - cz * (unsigned)G;
+    return cx | (cy << 10) | (cz << 20);
+}
 
 __device__ __forceinline__ unsigned key_of_point(const int *u, const RowGeom &g) {
     const unsigned cx = (unsigned)(u[0] / g.c), cy = g.d > 1 ? (unsigned)(u[1] / g.c) : 0u,
@@ -134,9 +150,9 @@ struct ScanArgs {
     int n;
     uint2 *rk;
     int *idx;
-    unsigned *cell_key;
-    int *start, *rep, *par;
-    unsigned long long *mid;
+    unsigned *cell_at;
+    int *start;
+    int G;
 };
 
 template <int WHAT>
@@ -198,12 +214,6 @@ __global__ void __launch_bounds__(256) rows_apply_kernel(ScanArgs a) {
 #pragma unroll
     for (int w = 0; w < 8; ++w)
         if (w < wid) at += wt[w];
-    auto new_cell = [&](int id, int first) {
-        a.start[id] = first;
-        a.rep[id] = DB_NONE;
-        a.mid[id] = ~0ull;
-        a.par[id] = id;
-    };
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const int i = i0 + k;
@@ -212,13 +222,13 @@ __global__ void __launch_bounds__(256) rows_apply_kernel(ScanArgs a) {
             if (WHAT == SCAN_DIRECT) {
                 a.idx[i] = id;
                 if (v[k]) {
-                    a.cell_key[id] = (unsigned)i;
-                    new_cell(id, first);
+                    a.cell_at[id] = cell_of_key((unsigned)i, a.G);
+                    a.start[id] = first;
                 }
             } else if (WHAT == SCAN_WORDS) {
                 a.rk[i] = make_uint2((unsigned)id, v[k]);
             } else {
-                new_cell(i, first);
+                a.start[i] = first;
             }
             at += scan_value<WHAT>(v[k]);
             if (i == m - 1) {  // the last entry: what the whole scan adds up to
@@ -241,7 +251,7 @@ __device__ __forceinline__ int cells_before(const RowArgs &a, unsigned key) {
 // Bitmap: the id of every point's cell, points per cell and the point's place
 // among them (one atomic per distinct cell of the warp).
 __global__ void __launch_bounds__(256) rows_cellcount_kernel(RowArgs a, unsigned *__restrict__ key_io,
-                                                             unsigned *__restrict__ cell_key, int *cnt,
+                                                             unsigned *__restrict__ cell_at, int *cnt,
                                                              int *__restrict__ rank) {
     db::wait_prior_grid();
     db::allow_next_grid();
@@ -254,7 +264,7 @@ __global__ void __launch_bounds__(256) rows_cellcount_kernel(RowArgs a, unsigned
     int base = 0;
     if (valid && lane == leader) {
         base = atomicAdd(cnt + id, __popc(peers));
-        if (base == 0) cell_key[id] = key;
+        if (base == 0) cell_at[id] = cell_of_key(key, a.g.G);
     }
     base = __shfl_sync(FULL, base, leader);
     if (!valid) return;
@@ -290,34 +300,52 @@ __global__ void __launch_bounds__(256) rows_list_kernel(RowArgs a) {
     const int ncells = (int)(*a.ctr0 >> 32), G = a.g.G;
     const char4 o = srow[r];
     const int step = (int)(gridDim.x * blockDim.x) / RL;
-    for (int c0 = (int)(blockIdx.x * blockDim.x + threadIdx.x - r) / RL; c0 - grp / RL < ncells; c0 += step) {
-        const int c = c0;  // the warp's cells are consecutive: the loop ends for all its lanes at once
-        int4 e = make_int4(0, 0, 0, 0);
-        if (c < ncells && r < a.g.nrows) {
-            const unsigned key = a.cell_key[c];
-            const int cx = (int)(key % (unsigned)G), cy = (int)((key / (unsigned)G) % (unsigned)G),
-                      cz = (int)(key / ((unsigned)G * (unsigned)G));
-            const int y = cy + o.x, z = cz + o.y;
-            if (y >= 0 && y < G && z >= 0 && z < G) {
-                const unsigned row = ((unsigned)z * (unsigned)G + (unsigned)y) * (unsigned)G;
-                const int lo = max(0, cx - o.z), hi = min(G - 1, cx + o.z);
-                e.x = o.w == 2 ? c + 1 : cells_before<DIRECT>(a, row + lo);
-                e.y = o.w == 1 ? c : cells_before<DIRECT>(a, row + hi + 1);
-                if (e.x < e.y) {
-                    e.z = a.start[e.x];
-                    e.w = a.start[e.y];
+    // two cells per round: their lookups are independent chains
+    for (int c0 = (int)(blockIdx.x * blockDim.x + threadIdx.x - r) / RL; c0 - grp / RL < ncells; c0 += 2 * step) {
+        int4 e[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = c0 + h * step;
+            e[h] = make_int4(0, 0, 0, 0);
+            if (c < ncells && r < a.g.nrows) {
+                const unsigned at = a.cell_at[c];
+                const int cx = (int)(at & 1023u), cy = (int)((at >> 10) & 1023u), cz = (int)(at >> 20);
+                const int y = cy + o.x, z = cz + o.y;
+                if (y >= 0 && y < G && z >= 0 && z < G) {
+                    const unsigned row = ((unsigned)z * (unsigned)G + (unsigned)y) * (unsigned)G;
+                    const int lo = max(0, cx - o.z), hi = min(G - 1, cx + o.z);
+                    e[h].x = o.w == 2 ? c + 1 : cells_before<DIRECT>(a, row + lo);
+                    e[h].y = o.w == 1 ? c : cells_before<DIRECT>(a, row + hi + 1);
                 }
             }
         }
-        const bool on = e.x < e.y;
-        const unsigned m = (__ballot_sync(FULL, on) >> grp) & (RL == 32 ? FULL : ((1u << (RL & 31)) - 1u));
-        if (on) a.rows[(size_t)c * a.g.nrows + __popc(m & ((1u << r) - 1u))] = e;
-        int t = e.w - e.z;
 #pragma unroll
-        for (int k = RL / 2; k > 0; k >>= 1) t += __shfl_xor_sync(FULL, t, k);
-        if (r == 0 && c < ncells) {
-            a.nent[c] = __popc(m);
-            a.cand[c] = t;
+        for (int h = 0; h < 2; ++h)
+            if (e[h].x < e[h].y) {
+                e[h].z = a.start[e[h].x];
+                e[h].w = a.start[e[h].y];
+            }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int c = c0 + h * step;
+            const bool on = e[h].x < e[h].y;
+            const unsigned m = (__ballot_sync(FULL, on) >> grp) & (RL == 32 ? FULL : ((1u << (RL & 31)) - 1u));
+            if (on) a.rows[(size_t)c * a.g.nrows + __popc(m & ((1u << r) - 1u))] = e[h];
+            int t = e[h].w - e[h].z;
+#pragma unroll
+            for (int k = RL / 2; k > 0; k >>= 1) t += __shfl_xor_sync(FULL, t, k);
+            if (c < ncells) {
+                if (r == 0) {
+                    a.nent[c] = __popc(m);
+                    a.cand[c] = t;
+                    a.rep[c] = DB_NONE;
+                }
+                if (r == 1) {  // and the first state of the later passes
+                    a.mid[c] = ~0ull;
+                    a.par[c] = c;
+                    a.least[c] = DB_NONE;
+                }
+            }
         }
     }
 }
@@ -328,7 +356,7 @@ __global__ void __launch_bounds__(256) rows_list_kernel(RowArgs a) {
 // hold few points and together with the warp's other points of that cell, 128
 // candidates a step, when they hold many.  Otherwise as in grid.cu.
 template <int D>
-__global__ void __launch_bounds__(256) rows_count_kernel(RowArgs a, int min_pts, int exact, int *counts_out,
+__global__ void __launch_bounds__(kWalkThreads) rows_count_kernel(RowArgs a, int min_pts, int exact, int *counts_out,
                                                          uint8_t *core_out) {
     db::wait_prior_grid();
     db::allow_next_grid();
@@ -430,23 +458,6 @@ __global__ void __launch_bounds__(256) rows_count_kernel(RowArgs a, int min_pts,
 
 // ---- merge (Section IV-C) ----
 
-// Union of two cells' sets: the root with the larger representative under the
-// other, so a root's representative is the smallest of its set.
-__device__ __forceinline__ void unite_cells(int *par, const int *rep, int x, int y, unsigned *status) {
-    for (int it = 0; it < (1 << 24); ++it) {
-        x = db::uf_find(par, x);
-        y = db::uf_find(par, y);
-        if (x == y) return;
-        if (rep[x] > rep[y]) {
-            const int t = x;
-            x = y;
-            y = t;
-        }
-        if (atomicCAS(par + y, y, x) == y) return;
-    }
-    atomicOr(status, DB_EBIT_TIMEOUT);
-}
-
 template <int D, int RL>
 __global__ void __launch_bounds__(256) rows_hook_kernel(RowArgs a) {
     db::wait_prior_grid();
@@ -458,30 +469,29 @@ __global__ void __launch_bounds__(256) rows_hook_kernel(RowArgs a) {
         const int c = c0;
         const int repc = c < ncells ? a.rep[c] : DB_NONE;
         if (!__any_sync(FULL, repc != DB_NONE)) continue;
-        unsigned long long best = ~0ull;  // (representative << 32) | cell
+        int best = INT_MAX;
         if (repc != DB_NONE && r < a.nent[c]) {
             const int4 e = a.rows[(size_t)c * a.g.nrows + r];
+            const int end = min(e.y, c);
             const float4 m = unpack_point(a.mid[c]);
             const float cp = a.g.Tp1 + m.w, mx2 = 2.f * m.x, my2 = 2.f * m.y, mz2 = 2.f * m.z;
-#pragma unroll 5
-            for (int id = e.x; id < e.y; ++id) {
-                const int rq = a.rep[id];
-                const unsigned long long mq = a.mid[id];
-                if (rq < repc) {  // has cores, and a smaller representative
-                    ++ev;
-                    if (is_nbr<D>(cp, mx2, my2, mz2, unpack_point(mq))) {
-                        const unsigned long long k = ((unsigned long long)(unsigned)rq << 32) | (unsigned)id;
-                        best = k < best ? k : best;
-                    }
-                }
-            }
-        }
+            unsigned long long mq[5];  // a row holds at most five cells; no core point: all ones
 #pragma unroll
-        for (int k = RL / 2; k > 0; k >>= 1) {
-            const unsigned long long y = __shfl_xor_sync(FULL, best, k);
-            best = y < best ? y : best;
+            for (int k = 0; k < 5; ++k) mq[k] = e.x + k < end ? a.mid[e.x + k] : ~0ull;
+#pragma unroll
+            for (int k = 4; k >= 0; --k)
+                if (mq[k] != ~0ull) {
+                    ++ev;
+                    if (is_nbr<D>(cp, mx2, my2, mz2, unpack_point(mq[k]))) best = e.x + k;
+                }
         }
-        if (r == 0 && best != ~0ull) a.par[c] = (int)(unsigned)best;
+        if (RL == 32) {
+            best = __reduce_min_sync(FULL, best);
+        } else {
+#pragma unroll
+            for (int k = RL / 2; k > 0; k >>= 1) best = min(best, __shfl_xor_sync(FULL, best, k));
+        }
+        if (r == 0 && best != INT_MAX) a.par[c] = best;
     }
     db::block_sum_add(a.ev + 1, ev);
 }
@@ -500,12 +510,8 @@ template <int D, int RL>
 __global__ void __launch_bounds__(256) rows_union_kernel(RowArgs a) {
     db::wait_prior_grid();
     db::allow_next_grid();
-    __shared__ float4 ybuf[8][128];
-    __shared__ uint8_t ycore[8][128];
-    const int lane = threadIdx.x & 31, r = lane & (RL - 1), grp = lane & ~(RL - 1), wib = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, r = lane & (RL - 1), grp = lane & ~(RL - 1);
     const int ncells = (int)(*a.ctr0 >> 32), step = (int)(gridDim.x * blockDim.x) / RL;
-    float4 *yb = ybuf[wib];
-    uint8_t *yc = ycore[wib];
     unsigned long long ev = 0;
     for (int c0 = (int)(blockIdx.x * blockDim.x + threadIdx.x - r) / RL; c0 - grp / RL < ncells; c0 += step) {
         const int c = c0;
@@ -518,70 +524,120 @@ __global__ void __launch_bounds__(256) rows_union_kernel(RowArgs a) {
             e.x = max(e.x, c + 1);  // each cell pair from its smaller id
             root = db::ld_relaxed(a.par + c);
         }
-        for (int k = 0; k < 5; ++k) {  // a row holds at most five cells
-            const int id = e.x + k;
-            bool need = id < e.y;
-            if (!__any_sync(FULL, need)) break;
-            // roots as the flattening left them: equal ones are one set (sets only merge)
-            if (need) need = a.rep[id] != DB_NONE && db::ld_relaxed(a.par + id) != root;
+        // roots as the flattening left them: equal ones are one set (sets only
+        // merge); a row holds at most five cells, looked at together
+        unsigned differ = 0;
+#pragma unroll
+        for (int k = 0; k < 5; ++k)
+            if (e.x + k < e.y)
+                differ |= (unsigned)(a.rep[e.x + k] != DB_NONE && db::ld_relaxed(a.par + e.x + k) != root) << k;
+        while (__any_sync(FULL, differ)) {
+            const int id = e.x + (differ ? __ffs((int)differ) - 1 : 0);
+            bool need = differ != 0;
+            differ &= differ - 1;
             if (need) need = db::uf_find(a.par, c) != db::uf_find(a.par, id);
             if (need) {  // the two central core points first, lanes in parallel
                 const float4 m = unpack_point(a.mid[c]);
                 ++ev;
-                if (is_nbr<D>(a.g.Tp1 + m.w, 2.f * m.x, 2.f * m.y, 2.f * m.z, unpack_point(a.mid[id]))) {
-                    unite_cells(a.par, a.rep, c, id, a.status);
+                bool hit = is_nbr<D>(a.g.Tp1 + m.w, 2.f * m.x, 2.f * m.y, 2.f * m.z, unpack_point(a.mid[id]));
+                const int sA = a.start[c], eA = a.start[c + 1], sB = a.start[id], eB = a.start[id + 1];
+                if (!hit && (eA - sA) * (eB - sB) <= kLaneTests) {  // few pairs: the lane tests them itself
+                    need = false;
+                    for (int qa = sA; qa < eA && !hit; ++qa) {
+                        if (!a.score[qa]) continue;
+                        const float4 pa = a.spts[qa];
+                        const float cp = a.g.Tp1 + pa.w, px2 = 2.f * pa.x, py2 = 2.f * pa.y, pz2 = 2.f * pa.z;
+#pragma unroll 4
+                        for (int qb = sB; qb < eB; ++qb) {
+                            const bool t = a.score[qb];
+                            ev += t;
+                            hit |= t && is_nbr<D>(cp, px2, py2, pz2, a.spts[qb]);
+                        }
+                    }
+                }
+                if (hit) {
+                    db::uf_unite(a.par, c, id, a.status);
                     need = false;
                 }
             }
-            unsigned todo = __ballot_sync(FULL, need);
-            bool first = true;
-            while (todo) {
-                const int l = __ffs(todo) - 1;
-                todo &= todo - 1;
-                const int A = __shfl_sync(FULL, c, l), B = __shfl_sync(FULL, id, l);
-                if (!first) {  // an earlier union may have joined them
-                    int same = 0;
-                    if (lane == 0) same = db::uf_find(a.par, A) == db::uf_find(a.par, B);
-                    if (__shfl_sync(FULL, same, 0)) continue;
-                }
-                first = false;
-                const int sA = a.start[A], cA = a.start[A + 1] - sA, sB = a.start[B], cB = a.start[B + 1] - sB;
-                const bool swap = cB > cA;  // lanes over the larger cell
-                const int sX = swap ? sB : sA, cX = swap ? cB : cA, sY = swap ? sA : sB, cY = swap ? cA : cB;
-                bool found = false;
-                for (int y0 = 0; y0 < cY && !found; y0 += 128) {
-                    const int ny = min(128, cY - y0);
-                    __syncwarp();
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int q = lane + 32 * u;
-                        if (q < ny) {
-                            yb[q] = a.spts[sY + y0 + q];
-                            yc[q] = a.score[sY + y0 + q];
+            const unsigned left = __ballot_sync(FULL, need);  // many pairs: a warp each, in the next kernel
+            if (left) {
+                int base = 0;
+                if (lane == __ffs(left) - 1) base = atomicAdd(a.npairs, __popc(left));
+                base = __shfl_sync(FULL, base, __ffs(left) - 1) + __popc(left & db::lanemask_lt());
+                // (the list holds two pairs a point; what it cannot take the lane searches)
+                if (need && base < a.pair_cap) {
+                    a.pairs[base] = make_int2(c, id);
+                } else if (need) {
+                    bool hit = false;
+                    for (int qa = a.start[c]; qa < a.start[c + 1] && !hit; ++qa)
+                        for (int qb = a.start[id]; qb < a.start[id + 1] && !hit && a.score[qa]; ++qb) {
+                            const float4 pa = a.spts[qa];
+                            hit = a.score[qb] &&
+                                  is_nbr<D>(a.g.Tp1 + pa.w, 2.f * pa.x, 2.f * pa.y, 2.f * pa.z, a.spts[qb]);
                         }
-                    }
-                    __syncwarp();
-                    for (int x0 = 0; x0 < cX && !found; x0 += 32) {
-                        const int xi = x0 + lane;
-                        const bool vx = xi < cX && a.score[sX + xi];
-                        const unsigned vxm = __ballot_sync(FULL, vx);
-                        if (!vxm) continue;
-                        const float4 px = a.spts[sX + (xi < cX ? xi : 0)];
-                        const float cp = a.g.Tp1 + px.w, px2 = 2.f * px.x, py2 = 2.f * px.y, pz2 = 2.f * px.z;
-                        for (int q = 0; q < ny; ++q) {
-                            if (!yc[q]) continue;
-                            if (lane == 0) ev += (unsigned)__popc(vxm);
-                            if (__any_sync(FULL, vx && is_nbr<D>(cp, px2, py2, pz2, yb[q]))) {
-                                found = true;
-                                break;
-                            }
-                        }
-                    }
+                    if (hit) db::uf_unite(a.par, c, id, a.status);
                 }
-                if (found && lane == 0) unite_cells(a.par, a.rep, A, B, a.status);
-                __syncwarp();
             }
         }
+    }
+    db::block_sum_add(a.ev + 1, ev);
+}
+
+// The listed cell pairs, a warp each: 128 points of the smaller cell staged at
+// a time, the lanes over the larger one.
+template <int D>
+__global__ void __launch_bounds__(256) rows_search_kernel(RowArgs a) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
+    __shared__ float4 ybuf[8][128];
+    __shared__ uint8_t ycore[8][128];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int npairs = min(*a.npairs, a.pair_cap), nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+    float4 *yb = ybuf[wib];
+    uint8_t *yc = ycore[wib];
+    unsigned long long ev = 0;
+    for (int k = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); k < npairs; k += nwarps) {
+        const int2 pr = a.pairs[k];
+        const int A = pr.x, B = pr.y;
+        const int sA = a.start[A], cA = a.start[A + 1] - sA, sB = a.start[B], cB = a.start[B + 1] - sB;
+        int same = 0;
+        if (lane == 0) same = db::uf_find(a.par, A) == db::uf_find(a.par, B);
+        if (__shfl_sync(FULL, same, 0)) continue;
+        const bool swap = cB > cA;  // lanes over the larger cell
+        const int sX = swap ? sB : sA, cX = swap ? cB : cA, sY = swap ? sA : sB, cY = swap ? cA : cB;
+        bool found = false;
+        for (int y0 = 0; y0 < cY && !found; y0 += 128) {
+            const int ny = min(128, cY - y0);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int q = lane + 32 * u;
+                if (q < ny) {
+                    yb[q] = a.spts[sY + y0 + q];
+                    yc[q] = a.score[sY + y0 + q];
+                }
+            }
+            __syncwarp();
+            for (int x0 = 0; x0 < cX && !found; x0 += 32) {
+                const int xi = x0 + lane;
+                const bool vx = xi < cX && a.score[sX + xi];
+                const unsigned vxm = __ballot_sync(FULL, vx);
+                if (!vxm) continue;
+                const float4 px = a.spts[sX + (xi < cX ? xi : 0)];
+                const float cp = a.g.Tp1 + px.w, px2 = 2.f * px.x, py2 = 2.f * px.y, pz2 = 2.f * px.z;
+                for (int q = 0; q < ny; ++q) {
+                    if (!yc[q]) continue;
+                    if (lane == 0) ev += (unsigned)__popc(vxm);
+                    if (__any_sync(FULL, vx && is_nbr<D>(cp, px2, py2, pz2, yb[q]))) {
+                        found = true;
+                        break;
+                    }
+                }
+            }
+        }
+        if (found && lane == 0) db::uf_unite(a.par, A, B, a.status);
+        __syncwarp();
     }
     db::block_sum_add(a.ev + 1, ev);
 }
@@ -590,7 +646,7 @@ __global__ void __launch_bounds__(256) rows_union_kernel(RowArgs a) {
 // thread per grouped position, with the count's split of the walks; bord[p]
 // gets the cell of the chosen core point (DB_NONE for noise).
 template <int D>
-__global__ void __launch_bounds__(256) rows_border_kernel(RowArgs a) {
+__global__ void __launch_bounds__(kWalkThreads) rows_border_kernel(RowArgs a) {
     db::wait_prior_grid();
     db::allow_next_grid();
     const int lane = threadIdx.x & 31, p = blockIdx.x * blockDim.x + threadIdx.x;
@@ -693,9 +749,30 @@ __global__ void __launch_bounds__(256) rows_border_kernel(RowArgs a) {
     db::block_sum_add(a.ev + 2, ev);
 }
 
-// Labels, a thread per grouped point: the representative of the root of its
-// cell (core) or of its chosen core neighbour's cell (border), noise -1; and
-// the statistics (a cluster's label is the index of one of its core points).
+// Root of every cell with cores, and the smallest representative of each set.
+__global__ void __launch_bounds__(256) rows_root_kernel(RowArgs a) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
+    const int ncells = (int)(*a.ctr0 >> 32), step = (int)(gridDim.x * blockDim.x), lane = threadIdx.x & 31;
+    for (int c0 = (int)(blockIdx.x * blockDim.x); c0 < ncells; c0 += step) {
+        const int c = c0 + (int)threadIdx.x, rep = c < ncells ? a.rep[c] : DB_NONE;
+        int root = -1 - lane;
+        if (rep != DB_NONE) {
+            root = db::uf_find(a.par, c);
+            if (root != c) db::st_relaxed(a.par + c, root);
+        }
+        // one atomic per distinct root of the warp, and none that cannot lower the value
+        const unsigned peers = __match_any_sync(FULL, root);
+        if (rep != DB_NONE) {
+            const int m = __reduce_min_sync(peers, rep);
+            if (lane == __ffs(peers) - 1 && m < db::ld_relaxed(a.least + root)) atomicMin(a.least + root, m);
+        }
+    }
+}
+
+// Labels, a thread per grouped point: the label of its cell's set (core) or of
+// the set of its chosen core neighbour's cell (border), noise -1; and the
+// statistics (a cluster's label is the index of one of its core points).
 __global__ void __launch_bounds__(256) rows_label_kernel(RowArgs a, int *__restrict__ labels, unsigned long long *ctr) {
     db::wait_prior_grid();
     db::allow_next_grid();
@@ -711,7 +788,7 @@ __global__ void __launch_bounds__(256) rows_label_kernel(RowArgs a, int *__restr
         const int c = core ? a.scell[p] : a.bord[p];
         int lab = -1;
         kind = core ? 0 : (c == DB_NONE ? 2 : 1);
-        if (kind != 2) lab = a.rep[db::uf_find(a.par, c)];
+        if (kind != 2) lab = a.least[a.par[c]];
         root = core && lab == o;
         labels[o] = lab;
     }
@@ -791,7 +868,7 @@ cudaError_t run_rows(const DbWork &w, const RowGeom &g, const float *x, int n, i
     a.ctr0 = w.ctr;
     a.rk = w.rk;
     a.idx = reinterpret_cast<const int *>(w.hkey);
-    a.cell_key = w.cell_key;
+    a.cell_at = w.cell_key;
     a.start = start;
     a.rows = reinterpret_cast<int4 *>(w.nbr);
     a.nent = w.ncnt;
@@ -803,7 +880,11 @@ cudaError_t run_rows(const DbWork &w, const RowGeom &g, const float *x, int n, i
     a.rep = w.cell_rep;
     a.mid = mid;
     a.par = w.cell_start;
+    a.least = w.hcursor;
     a.bord = w.border;
+    a.pairs = reinterpret_cast<int2 *>(w.pts4);  // free after the scatter: two pairs a point
+    a.pair_cap = 2 * n;
+    a.npairs = reinterpret_cast<int *>(w.ctr + DB_CTR_PAIRS);
     a.status = w.status;
     a.ev = w.ctr + DB_CTR_EVAL;
     ScanArgs s{};
@@ -812,11 +893,9 @@ cudaError_t run_rows(const DbWork &w, const RowGeom &g, const float *x, int n, i
     s.n = n;
     s.rk = w.rk;
     s.idx = reinterpret_cast<int *>(w.hkey);
-    s.cell_key = w.cell_key;
+    s.cell_at = w.cell_key;
     s.start = start;
-    s.rep = w.cell_rep;
-    s.par = w.cell_start;
-    s.mid = mid;
+    s.G = g.G;
     const int nb = (n + 255) / 256;
     auto scan = [&](auto what, const unsigned *in, int m, const char *nm) {
         constexpr int WHAT = decltype(what)::value;
@@ -846,11 +925,11 @@ cudaError_t run_rows(const DbWork &w, const RowGeom &g, const float *x, int n, i
     launch_dependent(rows_scatter_kernel<DIRECT>, nb, 256, st, a, key, rank, w.pts4, w.spts, w.sidx, w.scell);
     w.marks->kernel("grid_scatter", st);
     join(w, st, s2, 1);
-    launch_dependent(rows_count_kernel<D>, nb, 256, st, a, min_pts, exact ? 1 : 0, counts_out, core_out);
+    launch_dependent(rows_count_kernel<D>, (n + kWalkThreads - 1) / kWalkThreads, kWalkThreads, st, a, min_pts, exact ? 1 : 0, counts_out, core_out);
     w.marks->kernel("grid_count", st);
     // the border pass needs the core flags but not the merge: it runs beside it
     s2 = fork(w, st, 2);
-    launch_dependent(rows_border_kernel<D>, nb, 256, s2, a);
+    launch_dependent(rows_border_kernel<D>, (n + kWalkThreads - 1) / kWalkThreads, kWalkThreads, s2, a);
     w.marks->kernel("grid_border", s2);
     launch_dependent(rows_hook_kernel<D, RL>, cgrid, 256, st, a);
     w.marks->kernel("grid_hook", st);
@@ -858,6 +937,10 @@ cudaError_t run_rows(const DbWork &w, const RowGeom &g, const float *x, int n, i
     w.marks->kernel("grid_flatten", st);
     launch_dependent(rows_union_kernel<D, RL>, cgrid, 256, st, a);
     w.marks->kernel("grid_union_near", st);
+    launch_dependent(rows_search_kernel<D>, std::min(nb, 152 * 6), 256, st, a);
+    w.marks->kernel("grid_search", st);
+    launch_dependent(rows_root_kernel, std::min(nb, 152 * 8), 256, st, a);
+    w.marks->kernel("grid_root", st);
     join(w, st, s2, 3);
     launch_dependent(rows_label_kernel, nb, 256, st, a, labels, w.ctr);
     w.marks->kernel("grid_label", st);

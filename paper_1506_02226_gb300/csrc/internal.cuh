@@ -25,10 +25,12 @@
 //   diagnostics of the tensor-core count, merge and border passes,
 //   15 FP16 tensor-core count ran the folded form (1),
 //   16..19 pair tests evaluated by the count, merge, border and (grid path)
-//   outer-ring merge passes, 31 work items of the projected grid (int).
+//   outer-ring merge passes, 30 cell pairs left to the eps-grid's search (int),
+//   31 work items of the projected grid (int).
 #define DB_NCTR 32
 #define DB_CTR_EVAL 16
 #define DB_CTR_TC_FOLD 15      // 1: the FP16 count ran the folded form
+#define DB_CTR_PAIRS 30
 #define DB_CTR_MID_ITEMS 31
 #define DB_HASH_EMPTY 0xffffffffu
 
