@@ -4,13 +4,16 @@
 // The grid path (grid.cu) is a chain of some ten kernels; with a few thousand
 // points each of them works for a microsecond or two, and the launches, the
 // clears and the gaps between them are what a call takes (2,000 points in the
-// plane: 100 us).  Here one thread block cluster runs the whole method: every
-// block bins all points into its own shared memory (the binning is cheaper than
-// sharing it), counts neighbours and finds border neighbours for its eighth of
-// the points, and takes its eighth of the cell pairs in the merge.  The blocks
-// meet twice (cluster barriers): when the core flags are known (each block
-// writes its points' flags into every block's shared memory) and when the
-// merge, a union-find in global memory, is complete.
+// plane: 99 us a call, 70 with the merge on a forest in global memory, 60
+// as it is).  Here one thread block cluster runs the whole method: every block
+// bins all points into its own shared memory (the binning is cheaper than
+// sharing it) and counts neighbours and finds border neighbours for its eighth
+// of the points.  The blocks meet when the core flags are known (each block
+// writes its points' flags into every block's shared memory), and again after
+// the merge: each tests the cell pairs of its eighth of the cells on a forest of
+// its own in shared memory, then takes over the other blocks' links, one parent
+// a set and block.  One forest in global memory, with eight blocks linking the
+// same few roots, took 25 us of the call; all pairs in every block took 58.
 //
 // The geometry, the exact test, the order of decisions and so the labels are
 // grid.cu's: cells are cliques, cell pairs within the kept offsets are
@@ -29,27 +32,30 @@ namespace {
 constexpr int kMaxN = kGridSmallMaxN;  // 4,096
 constexpr int NB = 8, NT = 512;        // blocks of the cluster, threads of a block: at most one own point a thread
 constexpr int kSlots = 2 * kMaxN;      // cell hash
-constexpr int kList = 2048;            // merge: cell pairs left to a whole warp
-constexpr int kThreadTests = 64;       // merge: pair tests a thread makes before it leaves a cell pair to a warp
+constexpr int kList = 2048;            // merge: cell pairs in two sets, a warp each
+constexpr float kFar = -1e30f;         // near nothing
 constexpr unsigned FULL = 0xffffffffu;
+static_assert(kList * sizeof(unsigned) >= kMaxN * sizeof(uint16_t), "the list's place holds a forest");
 
 struct SmallSmem {
-    float4 pt[kMaxN];         // {u0, u1, u2, -|u|^2} grouped by cell
+    float4 pt[kMaxN];         // {u0, u1, u2, -|u|^2} grouped by cell; from the merge on w = kFar if not core
     unsigned key[kSlots];     // cell hash
     unsigned range[kSlots];   // (first position << 16) | points of the cell
     int rep[kSlots];          // smallest core index of the cell (first: fill cursor)
-    unsigned list[kList];     // (slot << 16) | slot
+    unsigned list[kList];     // (slot << 16) | slot; then the forest after this block's pairs
     uint16_t cell[kMaxN];     // slots of the occupied cells
     uint16_t idx[kMaxN];      // point at each position
     uint16_t pos[kMaxN];      // position of each point; then this block's cells in the merge
     uint16_t slot[kMaxN];     // cell of each position
+    uint16_t par[kMaxN];      // forest, by point
     uint8_t core[kMaxN];      // by point (written by all blocks)
-    uint8_t score[kMaxN];     // by position
     char4 off[128];
     int wsum[NT / 32], wocc[NT / 32];
-    unsigned bits[kMaxN / 32 + 1];  // roots, when labels are made dense
+    unsigned other[NT];       // this block's other points: (position << 16) | thread
+    unsigned found[NT];       // (smallest core neighbour << 16) | its cell's slot, by thread
+    unsigned bits[kMaxN / 32 + 1];  // roots: those that the hooking left, then those of the labels
     int before[kMaxN / 32 + 1];
-    int nlist, nown;
+    int nlist, nown, nother;
     int red[4];
 };
 
@@ -57,7 +63,7 @@ struct SmallArgs {
     const float *x;
     int n, hbits, min_pts, exact, compact, stats, reset;
     GridGeom g;
-    int *parent, *labels, *counts_out;
+    int *labels, *counts_out;
     uint8_t *core_out;
     unsigned *status;
     unsigned long long *ctr;
@@ -87,6 +93,60 @@ __device__ __forceinline__ int find_cell(const SmallSmem &S, unsigned key, int b
     return -1;
 }
 
+// Union-find over point indices in shared memory.
+__device__ __forceinline__ int find_root(volatile uint16_t *par, int x) {
+    while (true) {
+        const int p = par[x];
+        if (p == x) return x;
+        const int gp = par[p];
+        if (gp == p) return p;
+        par[x] = (uint16_t)gp;
+        x = gp;
+    }
+}
+__device__ __forceinline__ void unite(uint16_t *par, int a, int b, unsigned *status) {
+    for (int it = 0; it < (1 << 20); ++it) {
+        a = find_root(par, a);
+        b = find_root(par, b);
+        if (a == b) return;
+        if (a > b) {
+            const int t = a;
+            a = b;
+            b = t;
+        }
+        if (atomicCAS(reinterpret_cast<unsigned short *>(par + b), (unsigned short)b, (unsigned short)a) == b) return;
+    }
+    atomicOr(status, DB_EBIT_TIMEOUT);
+}
+
+// The cells at four offsets, their first probes side by side (-1: none).
+struct Four {
+    int slot[4];
+};
+__device__ __forceinline__ Four find_four(const SmallSmem &S, int cx, int cy, int cz, int o, int noff, int G, int bits) {
+    const unsigned mask = (1u << bits) - 1u;
+    Four f;
+    unsigned key[4], h[4], k[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const char4 off = S.off[min(o + u, noff - 1)];
+        const int x = cx + off.x, y = cy + off.y, z = cz + off.z;
+        const bool in = o + u < noff && x >= 0 && x < G && y >= 0 && y < G && z >= 0 && z < G;
+        key[u] = ((unsigned)z * (unsigned)G + (unsigned)y) * (unsigned)G + (unsigned)x;
+        h[u] = db::hash_slot(key[u], bits) & mask;
+        k[u] = in ? S.key[h[u]] : DB_HASH_EMPTY;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        for (unsigned probe = 0; probe <= mask && k[u] != key[u] && k[u] != DB_HASH_EMPTY; ++probe) {
+            h[u] = (h[u] + 1) & mask;
+            k[u] = S.key[h[u]];
+        }
+        f.slot[u] = k[u] == key[u] && k[u] != DB_HASH_EMPTY ? (int)h[u] : -1;
+    }
+    return f;
+}
+
 __device__ __forceinline__ unsigned key_of(int cx, int cy, int cz, int G) {
     return ((unsigned)cz * (unsigned)G + (unsigned)cy) * (unsigned)G + (unsigned)cx;
 }
@@ -101,6 +161,27 @@ __device__ __forceinline__ bool key_at(int cx, int cy, int cz, char4 o, int G, u
 // T + 1 - D(p,q) >= 1, exact (grid.cu).
 __device__ __forceinline__ bool near(float cp, float px2, float py2, float pz2, float4 q) {
     return fmaf(pz2, q.z, fmaf(py2, q.y, fmaf(px2, q.x, cp + q.w))) >= 1.f;
+}
+
+// Is a core point of cell a near one of cell b?  By GL lanes, a product of the
+// two cells' points each (a thread alone walks a chain of two dependent loads a
+// test); `mask` holds the group's lanes.
+template <int GL>
+__device__ __forceinline__ bool cells_near(const SmallSmem &S, float Tp1, int sa, int sb, int sub, unsigned mask,
+                                           unsigned long long &tests) {
+    const unsigned ra = S.range[sa], rb = S.range[sb], nb = rb & 0xffffu, all = (ra & 0xffffu) * nb;
+    for (unsigned k0 = 0; k0 < all; k0 += GL) {
+        const unsigned k = k0 + (unsigned)sub;
+        bool hit = false;
+        if (k < all) {
+            const unsigned q = k / nb;
+            const float4 pa = S.pt[(ra >> 16) + q], pb = S.pt[(rb >> 16) + k - q * nb];
+            hit = near(Tp1 + pa.w, 2.f * pa.x, 2.f * pa.y, 2.f * pa.z, pb);
+            ++tests;
+        }
+        if (__ballot_sync(mask, hit) & mask) return true;
+    }
+    return false;
 }
 
 __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_kernel(SmallArgs a) {
@@ -119,7 +200,8 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
         S.range[h] = 0u;
     }
     if (tid < 128) S.off[tid] = tid < noff ? a.g.off[tid] : make_char4(0, 0, 0, 0);
-    if (tid == 0) S.nlist = S.nown = 0;
+    if (tid == 0) S.nlist = S.nown = S.nother = 0;
+    for (int q = tid; q < n; q += NT) S.par[q] = (uint16_t)q;
     if (tid < 4) S.red[tid] = 0;
     if (rank == 0 && tid < DB_NCTR) a.ctr[tid] = 0ull;
     if (rank == 0 && tid == 0 && a.reset) *a.status = 0u;
@@ -207,182 +289,241 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
     __syncthreads();
     for (int c = tid; c < ncells; c += NT) S.rep[S.cell[c]] = DB_NONE;
 
-    // ---- neighbour counts of this block's points ----
-    const int own = (n + NB - 1) / NB, i = rank * own + tid;
-    const bool mine = tid < own && i < n;
+    // ---- neighbour counts of this block's points: a group of lanes each ----
+    const int own = (n + NB - 1) / NB;
+    int gl = 0;  // log2 of the group, as many lanes as there are threads for
+    while (gl < 3 && (own << (gl + 1)) <= NT) ++gl;
+    const int sub = tid & ((1 << gl) - 1), local = tid >> gl, i = rank * own + local;
+    const bool has = local < own && i < n, mine = has && sub == 0;
     float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-    int A = 0, cx = 0, cy = 0, cz = 0, count = 0;
+    int A = 0, at_i = 0, cx = 0, cy = 0, cz = 0, count = 0;
     unsigned long long ev_count = 0, ev_merge = 0, ev_border = 0, cand = 0;
-    if (mine) {
-        const int q = S.pos[i];
-        p = S.pt[q];
-        A = S.slot[q];
+    if (has) {
+        at_i = S.pos[i];
+        p = S.pt[at_i];
+        A = S.slot[at_i];
         const unsigned keyA = S.key[A];
         cx = (int)(keyA % (unsigned)G);
         cy = (int)((keyA / (unsigned)G) % (unsigned)G);
         cz = (int)(keyA / ((unsigned)G * (unsigned)G));
         count = (int)(S.range[A] & 0xffffu);  // the cell is a clique
-        a.parent[i] = i;
     }
-    const float cp = Tp1 + p.w, px2 = 2.f * p.x, py2 = 2.f * p.y, pz2 = 2.f * p.z;
     const int lim = a.exact ? INT_MAX : a.min_pts;
-    if (mine) {
-        cand = (unsigned)count;
-        for (int o = 0; o < noff; ++o) {
-            if (count >= lim && !a.stats) break;
-            unsigned key;
-            if (!key_at(cx, cy, cz, S.off[o], G, key)) continue;
-            const int B = find_cell(S, key, a.hbits);
-            if (B < 0) continue;
-            const unsigned r = S.range[B];
-            const int q0 = (int)(r >> 16), q1 = q0 + (int)(r & 0xffffu);
-            cand += r & 0xffffu;
-            if (count >= lim) continue;
-            for (int q = q0; q < q1; ++q) count += near(cp, px2, py2, pz2, S.pt[q]);
-            ev_count += r & 0xffffu;
+    {
+        const float cp = Tp1 + p.w, px2 = 2.f * p.x, py2 = 2.f * p.y, pz2 = 2.f * p.z;
+        if (mine) cand = (unsigned)count;
+        for (int o0 = 0; o0 < noff; o0 += 4 << gl) {
+            // a group goes on while its point needs it: every lane has the group's count
+            const bool go = has && (count < lim || a.stats);
+            if (!__any_sync(FULL, go)) break;
+            int add = 0;
+            const int o = o0 + 4 * sub;
+            if (go && o < noff) {
+                const Four f = find_four(S, cx, cy, cz, o, noff, G, a.hbits);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (f.slot[u] < 0) continue;
+                    const unsigned r = S.range[f.slot[u]];
+                    const int q0 = (int)(r >> 16), q1 = q0 + (int)(r & 0xffffu);
+                    cand += r & 0xffffu;
+                    if (count + add >= lim) continue;
+#pragma unroll 4
+                    for (int q = q0; q < q1; ++q) add += near(cp, px2, py2, pz2, S.pt[q]);
+                    ev_count += r & 0xffffu;
+                }
+            }
+            __syncwarp();
+            for (int b = 1; b < 1 << gl; b <<= 1) add += __shfl_xor_sync(FULL, add, b);
+            count += add;
         }
     }
     cluster_wait();
     if (mine)
         for (int r = 0; r < NB; ++r) cluster.map_shared_rank(S.core, r)[i] = count >= a.min_pts;
     cluster_arrive();
-    cluster_wait();  // core flags, the forest's first state and the cleared counters are everywhere
+    cluster_wait();  // core flags and the cleared counters are everywhere
     if (!ok) atomicOr(a.status, DB_EBIT_NOT_QUANTISED);
 
     // ---- representatives, by every block ----
     for (int q = tid; q < n; q += NT) {
         const int o = S.idx[q];
         const uint8_t c = S.core[o];
-        S.score[q] = c;
-        if (c) atomicMin(&S.rep[S.slot[q]], o);
+        if (c)
+            atomicMin(&S.rep[S.slot[q]], o);
+        else
+            S.pt[q].w = kFar;
     }
     __syncthreads();
 
-    // ---- merge: the cell pairs of this block's cells ----
-    // A cell belongs to a block by its representative: the blocks filled their
-    // hashes each in its own order, so slots and list places mean nothing to
-    // another block.
-    uint16_t *own_cell = S.pos;
+    // ---- merge ----
+    // This block's cells (dealt out by their smallest core index: the hash of
+    // each block fills in its own order) and its points that are not core.
+    uint16_t *own_cell = S.pos, *par = S.par;
     for (int c = tid; c < ncells; c += NT) {
         const int r = S.rep[S.cell[c]];
         if (r != DB_NONE && (r & (NB - 1)) == rank) own_cell[atomicAdd(&S.nown, 1)] = S.cell[c];
     }
+    for (int w = tid; w <= kMaxN / 32; w += NT) S.bits[w] = 0u;
+    const bool core = mine && S.core[i];
+    if (mine && !core) S.other[atomicAdd(&S.nother, 1)] = ((unsigned)at_i << 16) | (unsigned)tid;
     __syncthreads();
-    const int npairs = S.nown * noff;
-    for (int k = tid; k < npairs; k += NT) {
-        const int c = k / noff, sa = own_cell[c], ra = S.rep[sa];
-        const unsigned keyA = S.key[sa];
-        unsigned key;
-        if (!key_at((int)(keyA % (unsigned)G), (int)((keyA / (unsigned)G) % (unsigned)G),
-                    (int)(keyA / ((unsigned)G * (unsigned)G)), S.off[k - c * noff], G, key) ||
-            key <= keyA)  // each cell pair from its smaller key
-            continue;
-        const int sb = find_cell(S, key, a.hbits);
-        if (sb < 0 || S.rep[sb] == DB_NONE) continue;
-        const unsigned rga = S.range[sa], rgb = S.range[sb];
-        const int a0 = (int)(rga >> 16), a1 = a0 + (int)(rga & 0xffffu), b0 = (int)(rgb >> 16),
-                  b1 = b0 + (int)(rgb & 0xffffu);
-        bool hit = false, all = true;
-        int tests = 0;
-        for (int qa = a0; qa < a1 && !hit && all; ++qa) {
-            if (!S.score[qa]) continue;
-            const float4 pa = S.pt[qa];
-            for (int qb = b0; qb < b1; ++qb) {
-                if (!S.score[qb]) continue;
-                if (++tests > kThreadTests) {
-                    all = false;
-                    break;
-                }
-                if (near(Tp1 + pa.w, 2.f * pa.x, 2.f * pa.y, 2.f * pa.z, S.pt[qb])) {
-                    hit = true;
-                    break;
+    // First every cell is hooked to one adjacent cell of smaller key, in all
+    // blocks' forests at once: no exchange, and dense sets come down to a few
+    // roots, where linking pair by pair has all threads at the same few.
+    {
+        const int sub8 = lane & 7;
+        const unsigned mask = 0xffu << (lane & 24);
+        for (int c = tid >> 3; c < S.nown; c += NT / 8) {
+            const int sa = own_cell[c];
+            const unsigned keyA = S.key[sa];
+            const int ax = (int)(keyA % (unsigned)G), ay = (int)((keyA / (unsigned)G) % (unsigned)G),
+                      az = (int)(keyA / ((unsigned)G * (unsigned)G));
+            bool hit = false;
+            for (int o0 = 0; o0 < a.g.nnear && !hit; o0 += 8) {  // a lane looks one neighbour up
+                unsigned key;
+                int mb = -1;
+                if (o0 + sub8 < a.g.nnear && key_at(ax, ay, az, S.off[o0 + sub8], G, key) && key < keyA)
+                    mb = find_cell(S, key, a.hbits);
+                if (mb >= 0 && S.rep[mb] == DB_NONE) mb = -1;
+                for (unsigned left = __ballot_sync(mask, mb >= 0) & mask; left && !hit; left &= left - 1) {
+                    const int sb = __shfl_sync(mask, mb, __ffs(left) - 1);
+                    hit = cells_near<8>(S, Tp1, sa, sb, sub8, mask, ev_merge);
+                    if (hit) cluster.map_shared_rank(par, sub8)[S.rep[sa]] = (uint16_t)S.rep[sb];
                 }
             }
         }
-        if (!hit && !all) {  // many pairs: a warp takes it, or this thread when the list is full
-            const int at2 = atomicAdd(&S.nlist, 1);
-            if (at2 < kList) {
-                S.list[at2] = ((unsigned)sa << 16) | (unsigned)sb;
-            } else {
-                for (int qa = a0; qa < a1 && !hit; ++qa) {
-                    if (!S.score[qa]) continue;
-                    const float4 pa = S.pt[qa];
-                    for (int qb = b0; qb < b1 && !hit; ++qb)
-                        if (S.score[qb]) {
-                            ++tests;
-                            hit = near(Tp1 + pa.w, 2.f * pa.x, 2.f * pa.y, 2.f * pa.z, S.pt[qb]);
-                        }
-                }
-            }
-        }
-        ev_merge += (unsigned)tests;
-        if (hit) db::uf_unite(a.parent, ra, S.rep[sb], a.status);
-    }
-    __syncthreads();
-    for (int e = wid; e < min(S.nlist, kList); e += NT / 32) {
-        const int sa = (int)(S.list[e] >> 16), sb = (int)(S.list[e] & 0xffffu);
-        int same = 0;
-        if (lane == 0) same = db::uf_find(a.parent, S.rep[sa]) == db::uf_find(a.parent, S.rep[sb]);
-        if (__shfl_sync(FULL, same, 0)) continue;
-        const unsigned rga = S.range[sa], rgb = S.range[sb];
-        const int a0 = (int)(rga >> 16), a1 = a0 + (int)(rga & 0xffffu), b0 = (int)(rgb >> 16),
-                  b1 = b0 + (int)(rgb & 0xffffu);
-        bool hit = false;
-        for (int x0 = a0; x0 < a1 && !hit; x0 += 32) {
-            const int qa = x0 + lane;
-            const bool on = qa < a1 && S.score[qa];
-            const unsigned rows = __ballot_sync(FULL, on);
-            if (!rows) continue;
-            const float4 pa = S.pt[on ? qa : a0];
-            for (int qb = b0; qb < b1 && !hit; ++qb) {
-                if (!S.score[qb]) continue;
-                if (lane == 0) ev_merge += (unsigned)__popc(rows);
-                hit = __any_sync(FULL, on && near(Tp1 + pa.w, 2.f * pa.x, 2.f * pa.y, 2.f * pa.z, S.pt[qb]));
-            }
-        }
-        if (hit && lane == 0) db::uf_unite(a.parent, S.rep[sa], S.rep[sb], a.status);
         __syncwarp();
     }
+    cluster_arrive();
+    cluster_wait();
+    for (int c = tid; c < ncells; c += NT) {
+        const int r = S.rep[S.cell[c]];
+        if (r != DB_NONE) {
+            const int root = find_root(par, r);
+            if (root != r)
+                *(volatile uint16_t *)(par + r) = (uint16_t)root;
+            else
+                atomicOr(&S.bits[r >> 5], 1u << (r & 31));
+        }
+    }
+    __syncthreads();
+    // Then the cell pairs of this block's cells that are in two sets yet, on its
+    // own forest, the adjacent ones first.
+    for (int ring = 0; ring < 2; ++ring) {
+        const int o0 = ring ? a.g.nnear : 0, no = (ring ? noff : a.g.nnear) - o0, npairs = S.nown * no;
+        for (int k0 = 0; k0 < npairs; k0 += kList) {
+            __syncthreads();
+            if (tid == 0) S.nlist = 0;
+            __syncthreads();
+            for (int k = k0 + tid; k < min(k0 + kList, npairs); k += NT) {
+                const int c = k / no, sa = own_cell[c];
+                const unsigned keyA = S.key[sa];
+                unsigned key;
+                if (!key_at((int)(keyA % (unsigned)G), (int)((keyA / (unsigned)G) % (unsigned)G),
+                            (int)(keyA / ((unsigned)G * (unsigned)G)), S.off[o0 + k - c * no], G, key) ||
+                    key <= keyA)  // each cell pair from its smaller key
+                    continue;
+                const int sb = find_cell(S, key, a.hbits);
+                if (sb < 0 || S.rep[sb] == DB_NONE || find_root(par, S.rep[sa]) == find_root(par, S.rep[sb])) continue;
+                S.list[atomicAdd(&S.nlist, 1)] = ((unsigned)sa << 16) | (unsigned)sb;
+            }
+            __syncthreads();
+            for (int e = wid; e < S.nlist; e += NT / 32) {
+                const int sa = (int)(S.list[e] >> 16), sb = (int)(S.list[e] & 0xffffu);
+                const int same = lane == 0 && find_root(par, S.rep[sa]) == find_root(par, S.rep[sb]);
+                if (__shfl_sync(FULL, same, 0)) continue;
+                if (cells_near<32>(S, Tp1, sa, sb, lane, FULL, ev_merge) && lane == 0)
+                    unite(par, S.rep[sa], S.rep[sb], a.status);
+                __syncwarp();
+            }
+        }
+    }
 
-    // ---- border: the smallest-index core neighbour of this block's other points ----
-    int best = DB_NONE, bslot = A;
-    const bool core = mine && S.core[i];
-    if (mine && !core) {
-        best = S.rep[A];
-        for (int o = 0; o < noff; ++o) {
+    // The other blocks read a copy: this block goes on linking, and a parent
+    // that is shortened past a link they have not seen would lose the set between.
+    __syncthreads();
+    uint16_t *links = reinterpret_cast<uint16_t *>(S.list);
+    for (int q = tid; q < n; q += NT) links[q] = par[q];
+    cluster_arrive();
+
+    // ---- border: the smallest-index core neighbour of this block's other
+    // points, a warp each and a lane a neighbour cell ----
+    for (int e = wid; e < S.nother; e += NT / 32) {
+        const unsigned ent = S.other[e];
+        const float4 pe = S.pt[ent >> 16];  // not core: its w is gone
+        const float cp = Tp1 - (pe.x * pe.x + pe.y * pe.y + pe.z * pe.z);
+        const int sa = S.slot[ent >> 16];
+        const unsigned keyA = S.key[sa];
+        const int ax = (int)(keyA % (unsigned)G), ay = (int)((keyA / (unsigned)G) % (unsigned)G),
+                  az = (int)(keyA / ((unsigned)G * (unsigned)G));
+        int best = S.rep[sa], bslot = sa;
+        for (int o = lane; o < noff; o += 32) {
             unsigned key;
-            if (!key_at(cx, cy, cz, S.off[o], G, key)) continue;
+            if (!key_at(ax, ay, az, S.off[o], G, key)) continue;
             const int B = find_cell(S, key, a.hbits);
             if (B < 0 || S.rep[B] >= best) continue;  // no core index of B can beat the current best
             const unsigned r = S.range[B];
             const int q0 = (int)(r >> 16), q1 = q0 + (int)(r & 0xffffu);
             for (int q = q0; q < q1; ++q) {
-                if (!S.score[q] || S.idx[q] >= best) continue;
+                if (S.idx[q] >= best) continue;
                 ++ev_border;
-                if (near(cp, px2, py2, pz2, S.pt[q])) {
+                if (near(cp, 2.f * pe.x, 2.f * pe.y, 2.f * pe.z, S.pt[q])) {
                     best = S.idx[q];
                     bslot = B;
                 }
             }
         }
+        __syncwarp();
+        const unsigned low = __reduce_min_sync(
+            FULL, best == DB_NONE ? 0xffffffffu : ((unsigned)best << 16) | (unsigned)bslot);
+        if (lane == 0) S.found[ent & 0xffffu] = low;
     }
-    cluster_arrive();
-    cluster_wait();  // the forest is complete
 
-    // ---- labels ----
+    // ---- the other blocks' links, where they can differ: at the roots that the
+    // hooking left (with all cells' parents, hundreds of threads tried the same
+    // few links, 25,000 cycles) ----
+    cluster_wait();
+    for (int c = tid; c < ncells; c += NT) {
+        const int r = S.rep[S.cell[c]];
+        if (r == DB_NONE || !(S.bits[r >> 5] >> (r & 31) & 1u)) continue;
+        int up[NB];
+#pragma unroll
+        for (int o = 1; o < NB; ++o)
+            up[o] = cluster.map_shared_rank(links, (rank + o) & (NB - 1))[r];
+#pragma unroll
+        for (int o = 1; o < NB; ++o)
+            if (up[o] != r) unite(par, r, up[o], a.status);
+    }
+    cluster_arrive();  // waited for at the end: no block leaves while its links are read
+
+    // ---- labels: the smallest core index of each set ----
+    int *least = reinterpret_cast<int *>(S.range);  // by root (the cells are not looked at any more)
+    for (int q = tid; q < n; q += NT) least[q] = DB_NONE;
+    for (int w = tid; w <= kMaxN / 32; w += NT) S.bits[w] = 0u;
+    __syncthreads();
+    for (int c0 = 0; c0 < ncells; c0 += NT) {
+        const int c = c0 + tid, r = c < ncells ? S.rep[S.cell[c]] : DB_NONE;
+        const int root = r != DB_NONE ? find_root(par, r) : -1;
+        const unsigned on = __ballot_sync(FULL, root >= 0);
+        if (!on) continue;
+        const int root0 = __shfl_sync(FULL, root, __ffs(on) - 1);  // most warps see one set
+        const unsigned same = __ballot_sync(FULL, root == root0);
+        const int low = (int)__reduce_min_sync(FULL, root == root0 ? (unsigned)r : 0xffffffffu);
+        if (root == root0 ? lane == __ffs(same) - 1 : root >= 0) atomicMin(&least[root], root == root0 ? low : r);
+    }
+    __syncthreads();
     int lab = -1, kind = -1;
     bool root = false;
     if (mine) {
-        kind = core ? 0 : (best != DB_NONE ? 1 : 2);
-        if (kind != 2) lab = db::uf_find(a.parent, S.rep[bslot]);
+        const unsigned f = core ? 0u : S.found[tid];
+        kind = core ? 0 : (f != 0xffffffffu ? 1 : 2);
+        if (kind != 2) lab = least[find_root(par, S.rep[core ? A : (int)(f & 0xffffu)])];
         root = core && lab == i;
     }
     if (a.compact) {  // rank of each root: every block marks all of them
-        for (int w = tid; w <= kMaxN / 32; w += NT) S.bits[w] = 0u;
-        __syncthreads();
         for (int c = tid; c < ncells; c += NT) {
             const int r = S.rep[S.cell[c]];
-            if (r != DB_NONE && db::ld_relaxed(a.parent + r) == r) atomicOr(&S.bits[r >> 5], 1u << (r & 31));
+            if (r != DB_NONE && least[find_root(par, r)] == r) atomicOr(&S.bits[r >> 5], 1u << (r & 31));
         }
         __syncthreads();
         if (wid == 0) {
@@ -424,6 +565,7 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
     db::block_sum_add(a.ctr + DB_CTR_EVAL + 2, ev_border);
     __syncthreads();
     if (a.stats) db::block_sum_add(a.ctr + 1, cand);
+    cluster_wait();
 }
 
 }  // namespace
@@ -442,7 +584,6 @@ cudaError_t launch_grid_small(const DbWork &w, const GridGeom &g, const float *x
     a.stats = stats ? 1 : 0;
     a.reset = reset ? 1 : 0;
     a.g = g;
-    a.parent = w.parent;
     a.labels = labels;
     a.counts_out = counts_out;
     a.core_out = core_out;
