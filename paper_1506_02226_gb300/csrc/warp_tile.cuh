@@ -140,6 +140,7 @@ struct Item {
     unsigned long long cnt[4];    // count: neighbours, even and odd columns apart
     int root[4];                  // merge: a member of each row's set
     int best[4];                  // border
+    int was[2], now[2];           // merge: members lately joined, and a root found for each
     int row0;
 
     // Scores one column tile (64 columns from col0).
@@ -198,8 +199,8 @@ struct Item {
                     // members of the columns' sets; equal members need no union
                     int hq0 = 0, hq1 = 0;
                     if (hit) {
-                        hq0 = db::ld_relaxed(R.parent + col);
-                        hq1 = db::ld_relaxed(R.parent + col + 1);
+                        hq0 = member(db::ld_relaxed(R.parent + col));
+                        hq1 = member(db::ld_relaxed(R.parent + col + 1));
                     }
                     for (; hit; hit &= hit - 1) {
                         const int bit = __ffs(hit) - 1, i = bit >> 1, e = bit & 1;
@@ -210,6 +211,10 @@ struct Item {
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             if (root[k] == old || root[k] == hq) root[k] = r;
+                        was[1] = was[0];
+                        now[1] = now[0];
+                        was[0] = hq;
+                        now[0] = r;
                         if (hq0 == old || hq0 == hq) hq0 = r;
                         if (hq1 == old || hq1 == hq) hq1 = r;
                     }
@@ -220,6 +225,11 @@ struct Item {
         if ((PASS == WT_NEAR || PASS == WT_FAR) && __any_sync(FULL, any) && lane == 0)
             unite_sets(R.parent, mytag, ctag, R.status);
     }
+
+    // A row's parent, or the root that was found for it: rows not flattened since
+    // the join would each ask for the same union again, two chained loads from
+    // global memory at a time.
+    __device__ __forceinline__ int member(int p) const { return p == was[0] ? now[0] : (p == was[1] ? now[1] : p); }
 
     // Neighbours counted so far of row i of this lane (the same in its quad).
     __device__ __forceinline__ int counted(int i) const {
@@ -257,6 +267,8 @@ __device__ __forceinline__ void run_item(const Rows &R, const TileRec &I, int T,
     it.row0 = T * BT + 32 * half;
     load_rows16(R.P16, it.row0, it.a[0]);
     load_rows16(R.P16, it.row0 + 16, it.a[1]);
+    it.was[0] = it.was[1] = -3;  // no row
+    it.now[0] = it.now[1] = -3;
     int prior[4];
     bool mine = false;
 #pragma unroll
