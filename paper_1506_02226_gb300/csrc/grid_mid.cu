@@ -56,6 +56,8 @@ __device__ __forceinline__ unsigned ld_relaxed_u32(const unsigned *p) {
 // Grid check of all d coordinates, cell key of the first three, hash insert.
 __global__ void mid_prep_kernel(const float *__restrict__ x, int n, int d, GridGeom g, unsigned *hkey,
                                 int *hcount, int *__restrict__ slot_of, unsigned *status) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const bool valid = i < n;
@@ -106,6 +108,8 @@ template <int DP>
 __global__ void mid_scatter_kernel(const float *__restrict__ x, int n, int d, const int *__restrict__ slot_of,
                                    int *hcursor, float *__restrict__ P, float *__restrict__ nrm,
                                    int *__restrict__ sidx) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const bool valid = i < n;
@@ -137,23 +141,27 @@ __global__ void mid_scatter_kernel(const float *__restrict__ x, int n, int d, co
     sidx[pos] = i;
 }
 
-// Chunks per cell (32 points each), zero past the last cell.
-__global__ void mid_chunk_count_kernel(int n, const unsigned long long *ctr0, const int *__restrict__ cell_count,
-                                       int *__restrict__ cc) {
-    const int ncells = (int)(*ctr0 >> 32);
-    for (int A = blockIdx.x * blockDim.x + threadIdx.x; A < n; A += gridDim.x * blockDim.x)
-        cc[A] = A < ncells ? (cell_count[A] + 31) >> 5 : 0;
-}
-
-// Work items (cell, first point of the chunk) from the exclusive scan of the
-// chunk counts; *nitems receives the item count.
-__global__ void mid_chunk_table_kernel(int n, const unsigned long long *ctr0, const int *__restrict__ cell_count,
-                                       const int *__restrict__ scan, int2 *__restrict__ items, int *nitems) {
-    const int ncells = (int)(*ctr0 >> 32);
-    for (int A = blockIdx.x * blockDim.x + threadIdx.x; A < ncells; A += gridDim.x * blockDim.x) {
-        const int k0 = scan[A], nc = (cell_count[A] + 31) >> 5;
-        for (int k = 0; k < nc; ++k) items[k0 + k] = make_int2(A, 32 * k);
-        if (A == ncells - 1) *nitems = k0 + nc;
+// Work items (cell, first point of the chunk), in no particular order beyond the
+// 32 cells of a warp, which take their places at one go; *nitems counts them.
+// (One launch where a count, a scan of three and a fill were five; with the
+// path's other launches made dependent, 50,021 x 5: 337 us a call, now 310.)
+__global__ void mid_chunk_table_kernel(const unsigned long long *ctr0, const int *__restrict__ cell_count,
+                                       int2 *__restrict__ items, int *nitems) {
+    db::wait_prior_grid();  // started as a programmatic dependent
+    db::allow_next_grid();
+    const int ncells = (int)(*ctr0 >> 32), lane = threadIdx.x & 31;
+    for (int A0 = (int)(blockIdx.x * blockDim.x + threadIdx.x) - lane; A0 < ncells; A0 += gridDim.x * blockDim.x) {
+        const int A = A0 + lane, nc = A < ncells ? (cell_count[A] + 31) >> 5 : 0;
+        int inc = nc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += y;
+        }
+        int at = 0;
+        if (lane == 31) at = atomicAdd(nitems, inc);
+        at = __shfl_sync(FULL, at, 31) + inc - nc;
+        for (int k = 0; k < nc; ++k) items[at + k] = make_int2(A, 32 * k);
     }
 }
 
@@ -221,6 +229,8 @@ template <int DP>
 __global__ void __launch_bounds__(256) mid_count_kernel(MidArgs a, int min_pts, int exact, int *__restrict__ count,
                                                         uint8_t *__restrict__ core, uint8_t *__restrict__ score,
                                                         int *__restrict__ parent, int *__restrict__ hint) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nitems = *a.nitems;
@@ -338,6 +348,8 @@ __global__ void __launch_bounds__(256) mid_count_kernel(MidArgs a, int min_pts, 
 template <int DP>
 __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t *__restrict__ score, int *parent,
                                                         int *hint, unsigned *status) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nitems = *a.nitems;
@@ -455,6 +467,8 @@ __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t
 template <int DP>
 __global__ void __launch_bounds__(256) mid_border_kernel(MidArgs a, const uint8_t *__restrict__ score,
                                                          int *__restrict__ border) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nitems = *a.nitems;
@@ -536,30 +550,26 @@ cudaError_t mid_passes(const DbWork &w, const GridGeom &g, const float *x, int n
                        cudaStream_t st) {
     // Arrays of the eps-grid's workspace the projected path reuses: P holds the
     // grouped rows (stride DP <= the plan's row stride), pts4 the grouped
-    // -|u|^2, cell_mid the chunk table, cell_rep the chunks per cell, slot_of
+    // -|u|^2, cell_mid the chunk table, slot_of
     // (free after the scatter) the set hints.
     float *nrm = reinterpret_cast<float *>(w.pts4);
     int2 *items = reinterpret_cast<int2 *>(w.cell_mid);
     int *nitems = reinterpret_cast<int *>(w.ctr + DB_CTR_MID_ITEMS);
-    int *cc = w.cell_rep;
     int *hint = w.slot_of;
     const int nb = (n + 255) / 256;
-    mid_scatter_kernel<DP><<<nb, 256, 0, st>>>(x, n, d, w.slot_of, w.hcursor, w.P, nrm, w.sidx);
+    launch_dependent(mid_scatter_kernel<DP>, nb, 256, st, x, n, d, w.slot_of, w.hcursor, w.P, nrm, w.sidx);
     w.marks->kernel("mid_scatter", st);
     cudaError_t e;
     if ((e = launch_grid_nbrs(w, g, occ, st))) return e;
-    mid_chunk_count_kernel<<<std::min(nb, 152 * 8), 256, 0, st>>>(n, w.ctr, w.cell_count, cc);
-    w.marks->kernel("mid_chunks", st);
-    if ((e = launch_exclusive_scan(cc, w.scan, n, w.scan_part, w.scan_part_cap, st, w.marks))) return e;
-    mid_chunk_table_kernel<<<std::min(nb, 152 * 8), 256, 0, st>>>(n, w.ctr, w.cell_count, w.scan, items, nitems);
+    launch_dependent(mid_chunk_table_kernel, std::min(nb, 152 * 8), 256, st, w.ctr, w.cell_count, items, nitems);
     w.marks->kernel("mid_chunk_table", st);
     MidArgs a{g, w.cell_start, w.cell_count, w.nbr, w.ncnt, w.P, nrm, w.sidx, items, nitems, w.ctr + DB_CTR_EVAL};
     const int wgrid = 152 * 16;  // 8 warps per block, warps stride over the chunks
-    mid_count_kernel<DP><<<wgrid, 256, 0, st>>>(a, min_pts, exact ? 1 : 0, w.count, w.core, w.score, w.parent, hint);
+    launch_dependent(mid_count_kernel<DP>, wgrid, 256, st, a, min_pts, exact ? 1 : 0, w.count, w.core, w.score, w.parent, hint);
     w.marks->kernel("mid_count", st);
-    mid_union_kernel<DP><<<wgrid, 256, 0, st>>>(a, w.score, w.parent, hint, w.status);
+    launch_dependent(mid_union_kernel<DP>, wgrid, 256, st, a, w.score, w.parent, hint, w.status);
     w.marks->kernel("mid_union", st);
-    mid_border_kernel<DP><<<wgrid, 256, 0, st>>>(a, w.score, w.border);
+    launch_dependent(mid_border_kernel<DP>, wgrid, 256, st, a, w.score, w.border);
     w.marks->kernel("mid_border", st);
     if ((e = cudaGetLastError())) return e;
     return launch_labels_allpairs(w, n, labels, counts_out, core_out, st);
@@ -609,7 +619,7 @@ cudaError_t launch_mid_grid_path(const DbWork &w, const GridGeom &g, const float
     unsigned *occ = occ_words <= w.occ_cap ? w.occ : nullptr;
     if (occ && (e = cudaMemsetAsync(occ, 0, sizeof(unsigned) * occ_words, st))) return e;
     const int nb = (n + 255) / 256;
-    mid_prep_kernel<<<nb, 256, 0, st>>>(x, n, d, g, w.hkey, w.hcount, w.slot_of, w.status);
+    launch_dependent(mid_prep_kernel, nb, 256, st, x, n, d, g, w.hkey, w.hcount, w.slot_of, w.status);
     w.marks->kernel("mid_prep", st);
     if ((e = launch_grid_cells(w, g, occ, nullptr, st))) return e;
     return DP == 4 ? mid_passes<4>(w, g, x, n, d, min_pts, exact, labels, counts_out, core_out, occ, st)

@@ -29,6 +29,8 @@ __global__ void labels_allpairs_kernel(int n, const uint8_t *__restrict__ core, 
                                        const int *__restrict__ border, const int *__restrict__ count,
                                        int *__restrict__ labels, int *__restrict__ counts_out,
                                        uint8_t *__restrict__ core_out, unsigned long long *ctr) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     __shared__ int red[32];
     int nc = 0, nb = 0, nn = 0, nr = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -83,6 +85,8 @@ __device__ __forceinline__ int block_excl_scan(int v, int *warp_tot, int &total)
 }
 
 __global__ void scan_tile_sums(const int *__restrict__ in, int64_t n, int *__restrict__ part) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     __shared__ int red[32];
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_IPT;
     int s = 0;
@@ -94,6 +98,8 @@ __global__ void scan_tile_sums(const int *__restrict__ in, int64_t n, int *__res
 }
 
 __global__ void scan_partials(int *part, int64_t m) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     __shared__ int wt[32];
     int carry = 0;
     for (int64_t b = 0; b < m; b += blockDim.x) {
@@ -110,6 +116,8 @@ __global__ void scan_partials(int *part, int64_t m) {
 
 __global__ void scan_tiles(const int *__restrict__ in, int64_t n, const int *__restrict__ part,
                            int *__restrict__ out) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     __shared__ int wt[32];
     const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_IPT;
     int v[SCAN_IPT];
@@ -183,11 +191,15 @@ __global__ void __launch_bounds__(1024) bucket_scan_kernel(int *__restrict__ v, 
 }
 
 __global__ void root_flags_kernel(int n, const int *__restrict__ labels, int *__restrict__ flags) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         flags[i] = labels[i] == i;
 }
 
 __global__ void compact_kernel(int n, int *__restrict__ labels, const int *__restrict__ rank) {
+    db::wait_prior_grid();
+    db::allow_next_grid();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         int l = labels[i];
         if (l >= 0) labels[i] = rank[l];
@@ -203,11 +215,11 @@ cudaError_t launch_exclusive_scan(const int32_t *in, int32_t *out, int64_t n, in
     const int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
     if (tiles + 1 > part_cap) return cudaErrorInvalidValue;
     if (tiles == 0) return cudaMemsetAsync(out, 0, sizeof(int32_t), st);
-    scan_tile_sums<<<(unsigned)tiles, SCAN_NT, 0, st>>>(in, n, part);
+    launch_dependent(scan_tile_sums, (unsigned)tiles, SCAN_NT, st, in, n, part);
     if (pm) pm->kernel("scan_sums", st);
-    scan_partials<<<1, 1024, 0, st>>>(part, tiles);
+    launch_dependent(scan_partials, 1, 1024, st, part, tiles);
     if (pm) pm->kernel("scan_partials", st);
-    scan_tiles<<<(unsigned)tiles, SCAN_NT, 0, st>>>(in, n, part, out);
+    launch_dependent(scan_tiles, (unsigned)tiles, SCAN_NT, st, in, n, part, out);
     if (pm) pm->kernel("scan_tiles", st);
     return cudaGetLastError();
 }
@@ -218,7 +230,7 @@ cudaError_t launch_bucket_scan(int32_t *v, int32_t n, cudaStream_t st) {
 
 cudaError_t launch_labels_allpairs(const DbWork &w, int64_t n, int32_t *labels, int32_t *counts_out,
                                    uint8_t *core_out, cudaStream_t st) {
-    labels_allpairs_kernel<<<grid_for(n), 256, 0, st>>>((int)n, w.core, w.parent, w.border, w.count, labels,
+    launch_dependent(labels_allpairs_kernel, grid_for(n), 256, st, (int)n, w.core, w.parent, w.border, w.count, labels,
                                                         counts_out, core_out, w.ctr);
     w.marks->kernel("labels", st);
     return cudaGetLastError();
@@ -226,11 +238,11 @@ cudaError_t launch_labels_allpairs(const DbWork &w, int64_t n, int32_t *labels, 
 
 cudaError_t launch_compact(const DbWork &w, int64_t n, int32_t *labels, cudaStream_t st) {
     // The border array is free once labels exist; it holds the root flags.
-    root_flags_kernel<<<grid_for(n), 256, 0, st>>>((int)n, labels, w.border);
+    launch_dependent(root_flags_kernel, grid_for(n), 256, st, (int)n, labels, w.border);
     w.marks->kernel("root_flags", st);
     cudaError_t e = launch_exclusive_scan(w.border, w.scan, n, w.scan_part, w.scan_part_cap, st, w.marks);
     if (e) return e;
-    compact_kernel<<<grid_for(n), 256, 0, st>>>((int)n, labels, w.scan);
+    launch_dependent(compact_kernel, grid_for(n), 256, st, (int)n, labels, w.scan);
     w.marks->kernel("compact", st);
     return cudaGetLastError();
 }
