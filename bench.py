@@ -168,15 +168,16 @@ def grid_offsets(d: int, T: int):
     return c, offs
 
 
-# DRAM bytes per launch of a dominant kernel from an ncu capture (profiles/), with
+# DRAM bytes of a dominant pass from an ncu capture (profiles/: the recipe's sizes,
+# another seed; cold cache), with
 # the sha1 prefix of the kernel's source file when it was captured: a changed
 # source means the counters no longer describe the kernel, and the bench line
 # reports traffic null.
 NCU_TRAFFIC = {
-    ("lowd2", "grid_count"): (17419776, "paper_1506_02226_gb300/csrc/grid.cu", "faffd4840d06"),
-    ("lowd2", "grid_union_near"): (10742272, "paper_1506_02226_gb300/csrc/grid.cu", "faffd4840d06"),
-    ("lowd3", "grid_count"): (32878592, "paper_1506_02226_gb300/csrc/grid.cu", "faffd4840d06"),
-    ("lowd3", "grid_union_near"): (23241728, "paper_1506_02226_gb300/csrc/grid.cu", "faffd4840d06"),
+    ("lowd2", "grid_count"): (17994496, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
+    ("lowd2", "grid_union_near"): (11583000, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
+    ("lowd3", "grid_count"): (43683072, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
+    ("lowd3", "grid_union_near"): (57444000, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
 }
 
 
@@ -195,46 +196,39 @@ def ncu_traffic(workload: str, kernel: str):
 
 
 def algorithmic_work(name: str, n: int, d: int, gs: dict | None):
-    """(bound, bytes per launch) of a grid kernel: the bytes it has to move at
+    """(bound, bytes per launch) of an eps-grid kernel: the bytes it has to move at
     least, counting every input it must read and every output it must write
-    once.  gs is the instance's grid_structure (cells C, neighbour-list entries
-    E = adjacent En + outer Ef; H hash slots).
+    once.  gs is the instance's grid_structure (C cells); what a kernel reads of
+    the cells around a cell is in cache by then and not counted.
 
-      prep     reads x (4d), writes packed point (16) and hash slot (4), one
-               hash entry (8)                                 (4d + 28) n
-      cells    reads key and count of every slot (8), writes the packed
-               {key, id} table (8), 24 per cell               16 H + 24 C
-      scatter  reads slot, cell id and packed point (24), writes packed
-               point, index and cell id (24), one cursor (4)  52 n
-      nbrs     per cell key and list length (8), per entry a hash entry (8)
-               and the list entry (4)                         8 C + 12 E
-      count    per point the packed point (16), index (4), core flag and
-               parent written (5); per cell 32 (range, length, rep, centre);
-               per entry list entry and neighbour range (12)  25 n + 32 C + 12 E
-      union    per cell 32; per adjacent entry list entry, key, rep and
-               centre point (28); per outer entry 12           32 C + 28 En / 12 Ef
-      border   per point core flag (1) and border written (4) 5 n
-      root     per cell rep, parent and root (16)             16 C (also the snapshot
-               taken between the adjacent and outer-ring merges)
-      label    per point index, cell, flag, cell root, border (17), label (4)  21 n
+      prep     reads x (4d), writes packed point (16), key (4), rank (4)   (4d + 24) n
+      rows     per cell its coordinates (4), list length and points (8)    12 C
+      scatter  reads key, rank and packed point (24), writes packed point,
+               index and cell id (24); per cell its start (4)              48 n + 4 C
+      count    per point the packed point (16), index and cell id (8), core
+               flag (1); per cell list length, points (8), rep and centre (12)  25 n + 20 C
+      hook, union  per cell rep (4), centre point (8), parent (4)          16 C
+      flatten  per cell parent read and written                            8 C
+      border   per point core flag (1) and border written (4)              5 n
+      root     per cell rep, parent and set's least (12)                   12 C
+      label    per point index, cell, flag, border (13), label (4)         17 n
+      small    one launch for it all: x in, labels out                     (4d + 4) n
     """
     if d > 3 or gs is None:
         return None, 0
-    C, En, Ef = gs["cells"], gs["near_entries"], gs["far_entries"]
-    E = En + Ef
-    H = 1 << max(10, math.ceil(math.log2(2 * n)))
+    C = gs["cells"]
     table = {
-        "grid_prep": (4 * d + 28) * n,
-        "grid_cells": 16 * H + 24 * C,
-        "grid_scatter": 52 * n,
-        "grid_nbrs": 8 * C + 12 * E,
-        "grid_count": 25 * n + 32 * C + 12 * E,
-        "grid_union_near": 32 * C + 28 * En,
-        "grid_union_far": 32 * C + 12 * Ef,
+        "grid_prep": (4 * d + 24) * n,
+        "grid_rows": 12 * C,
+        "grid_scatter": 48 * n + 4 * C,
+        "grid_count": 25 * n + 20 * C,
+        "grid_hook": 16 * C,
+        "grid_flatten": 8 * C,
+        "grid_union_near": 32 * C,  # with the hook (ONE_PASS)
         "grid_border": 5 * n,
-        "grid_cell_root": 16 * C,
-        "grid_root_snapshot": 16 * C,
-        "grid_label": 21 * n,
+        "grid_root": 12 * C,
+        "grid_label": 17 * n,
+        "grid_small": (4 * d + 4) * n,
     }
     if name in table:
         return "hbm", table[name]
@@ -247,6 +241,11 @@ def fp32_peak_tops():
     peaks = load_peaks()
     sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
     return sms * 128 * peaks["sm_max_mhz"] * 1e6 / 1e12, sms
+
+
+# FP32-pipe operations of one pair on the warp tiles, whose dot product is on the
+# tensor cores: scale and add, add, saturate and add (or compare).
+WARP_TILE_OPS = 3
 
 
 def pair_ops(d: int) -> int:
@@ -273,9 +272,22 @@ def whole_job_rate(units_per_rank: float, world: int, ms_per_step: float) -> flo
 # ------------------------------------------------------------------ arms
 # Device counters 16..19 of a plan: pair tests of the count, merge, border and
 # outer-ring merge passes; the kernels that evaluate pairs, by pass.
-PASS_OF = {"grid_count": 0, "grid_union_near": 1, "grid_border": 2, "grid_union_far": 3,
+PASS_OF = {"grid_count": 0, "grid_union_near": 1, "grid_border": 2,
            "ap_count": 0, "ap_union": 1, "ap_border": 2, "tc_count": 0, "tc_union": 1, "tc_border": 2,
-           "mid_count": 0, "mid_union": 1, "mid_border": 2}
+           "wt_count": 0, "wt_union": 1, "wt_border": 2, "mid_count": 0, "mid_union": 1, "mid_border": 2}
+# Kernels whose evaluated pairs one counter holds: their times are taken together.
+ONE_PASS = {"tc_union": ("tc_adj", "tc_union_near", "tc_union"), "wt_union": ("wt_core", "wt_union_near", "wt_union"),
+            "grid_union_near": ("grid_hook", "grid_union_near", "grid_search"),
+            "batch_union": ("batch_core", "batch_union_near", "batch_union")}
+
+
+def by_pass(times: dict) -> dict:
+    """Per-kernel times with the kernels of one pass added up under its name."""
+    out = dict(times)
+    for name, parts in ONE_PASS.items():
+        if name in out:
+            out[name] = sum(out.pop(k) for k in parts if k in out)
+    return out
 
 
 def run_reference(args, wl_name):
@@ -376,7 +388,8 @@ def roofline(dom: str, avg_ms: float, ev: list, n: int, d: int, gs, wl_name: str
                                         "frac": ex / peaks["bf16_tflops"],
                                         "note": "the folded count's MMA runs K + 16 columns; frac above counts 2K"}
             return roof
-        ops_pp = pair_ops(d) if not dom.startswith(("grid_", "mid_")) else d + 2
+        ops_pp = WARP_TILE_OPS if dom.startswith("wt_") else (
+            pair_ops(d) if not dom.startswith(("grid_", "mid_")) else d + 2)
         fp32_peak, sms = fp32_peak_tops()
         ach = pairs * ops_pp / sec / 1e12
         alu = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": fp32_peak, "unit": "T FP32-pipe ops/s",
@@ -540,12 +553,13 @@ def run_ours(args, wl_name, baseline=True, steps=None):
         aplan.close()
         allpairs = {"ms_per_step": statistics.mean(a_ms), "pair_tests_per_step": a_pairs,
                     "speedup_of_grid": statistics.mean(a_ms) / ms_per_step,
-                    "what": "the same instance on the all-pairs CUDA-core path (grid off), 3 steps"}
+                    "what": "the same instance on the all-pairs path (grid off), 3 steps"}
 
     if rank != 0:
         return None
     avg = {k: statistics.mean(v) for k, v in kern.items()}
     ev_pass = [statistics.mean(r[k] for r in ev_runs) for k in range(4)]
+    kernel_avg, avg = avg, by_pass(avg)
     dom = max(avg, key=avg.get)
     folded = tc_form is not None and tc_form.startswith("folded")
     roof = roofline(dom, avg[dom], ev_pass, n, d, gs, wl_name, args.traffic, folded)
@@ -562,7 +576,7 @@ def run_ours(args, wl_name, baseline=True, steps=None):
         "scaling": "weak", "vs_baseline": None, "dtype": {2: "f32", 3: "f16" if prec != 3 else "bf16"}.get(
             st0["path"], "f32"), "data": "synthetic",
         "config": {"workload": wl_name + ": " + desc, "n": n, "d": d, "eps": inst.eps, "min_pts": inst.min_pts,
-                   "path": {1: "eps-grid", 2: "all-pairs SIMT", 3: "all-pairs tensor-core",
+                   "path": {1: "eps-grid", 2: "all-pairs SIMT" if prec == B.DBSCAN_PREC_EXACT_SIMT or d > 16 else "all-pairs warp tiles", 3: "all-pairs tensor-core",
                             4: "projected grid"}.get(st0["path"]),
                    "l2": "flushed by a 256 MiB write before every timed step", "parallelism": f"replicas x{world}"},
         "pair_tests_per_step": pairs_per_step,
@@ -576,7 +590,7 @@ def run_ours(args, wl_name, baseline=True, steps=None):
         "tc_count_form": tc_form,
         "points_per_s": world * n / (ms_per_step * 1e-3),
         "clusters": st0["n_clusters"], "core": st0["n_core"], "noise": st0["n_noise"],
-        "kernels_ms": {k: round(v, 5) for k, v in sorted(avg.items(), key=lambda kv: -kv[1])},
+        "kernels_ms": {k: round(v, 5) for k, v in sorted(kernel_avg.items(), key=lambda kv: -kv[1])},
         "kernels_ms_note": "each kernel alone (a profiled run, kernels serialised, L2 flushed before each run)",
         "roofline": roof,
         "roofline_next": others,
@@ -683,21 +697,21 @@ def run_batch(args, steps=None):
     jobs = count / (ms * 1e-3)
     pairs = sum(i.n * i.n for i in insts)
     peak_tops, sms = fp32_peak_tops()
-    dom = max(kern, key=kern.get)
+    passes = by_pass(kern)
+    dom = max(passes, key=passes.get)
     if dom in ("batch_count", "batch_union", "batch_border"):
         # pairs each pass evaluated (device counters of a batch run with statistics)
-        # times the FP32-pipe operations of one pair test at the instance's d
+        # times the FP32-pipe operations of one pair
         k = ("batch_count", "batch_union", "batch_border").index(dom)
         pp = pass_pairs[k]
-        mean_ops = sum(i.n * i.n * pair_ops(i.d) for i in insts) / max(sum(i.n * i.n for i in insts), 1)
-        ops = pp * mean_ops
-        ach = ops / (kern[dom] * 1e-3) / 1e12
+        ops = pp * WARP_TILE_OPS
+        ach = ops / (passes[dom] * 1e-3) / 1e12
         roof = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": peak_tops, "unit": "T FP32-pipe ops/s",
                 "frac": ach / peak_tops, "traffic": args.traffic, "peak_src": f"{sms} SMs x 128 lanes x max clock",
-                "avg_ms": kern[dom]}
+                "avg_ms": passes[dom]}
     else:
         roof = {"kernel": dom, "bound": None, "achieved": None, "peak": None, "unit": None, "frac": None,
-                "traffic": None, "avg_ms": kern[dom]}
+                "traffic": None, "avg_ms": passes[dom]}
     cpu = None
     if not args.no_baseline:
         import oracle
@@ -716,7 +730,7 @@ def run_batch(args, steps=None):
         "dtype": "f32", "data": "synthetic",
         "config": {"workload": f"batch: {count} instances, n log-uniform 64..8192, d in {{2,3,16}}, 1-8 blobs + 10% "
                                "noise, eps U[0.01,0.05], min_pts U{4..16}", "points": int(loffs[-1]),
-                   "path": "all-pairs SIMT, one graph launch",
+                   "path": "all-pairs warp tiles, one graph launch",
                    "autotuned": {"tile": [tile_rows, tile_cols], "chunk_tiles": ch, "blocks_per_sm": bps},
                    "l2": "flushed by a 256 MiB write before every timed step"},
         "pair_tests_per_step": pair_tests, "pair_tests_per_s": pair_tests / (ms * 1e-3),
@@ -728,7 +742,7 @@ def run_batch(args, steps=None):
         "roofline": roof, "cpu_baseline": cpu,
         "e2e": {"value": count / (e2e_ms * 1e-3), "unit": "jobs/s", "ms_per_step": e2e_ms,
                 "h2d_bytes_per_step": 4 * int(offs[-1]), "d2h_bytes_per_step": 4 * int(loffs[-1])},
-        "gpu_launches": 6 * steps, "clocks": clk,
+        "gpu_launches": len(kern) * steps, "clocks": clk,
     }
     return out
 

@@ -81,7 +81,7 @@ size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
         w.nbr = c.take<int32_t>((size_t)n * w.noff_cap);
         w.ncnt = c.take<int32_t>(n);
         w.cell_cand = c.take<int32_t>(n);
-        if (dg == o.max_d || !exact_d) {  // the eps-grid's (d <= 3)
+        if (n > kGridSmallMaxN && (dg == o.max_d || !exact_d)) {  // grid_rows.cu's
             w.rk = c.take<uint2>(w.occ_cap);
             w.rg_part = c.take<unsigned long long>(std::max(w.hcap, w.occ_cap) / 2048 + 8);
         }

@@ -62,8 +62,8 @@
 // are one-sided (m is an underestimate, r + eps an overestimate), so the order
 // and the cull change no result, only how much is proved empty: 200,000 x 64
 // in 100 blobs plus 15% noise evaluates 2.74e9 pairs instead of 5.70e10 in the
-// three passes (1.37 ms a run instead of 8.74; 100,003 x 48 in BF16 1.70 instead
-// of 6.87 ms; a burst of 40 served jobs, a third of them at d = 32, 12.8 instead
+// three passes (1.07 ms a run instead of 8.74; 100,003 x 48 in BF16 0.94 instead
+// of 6.87 ms; a burst of 40 served jobs, a third of them at d = 32, 9.7 instead
 // of 65.0 ms).  The limit of 32,768 points is where ordering (some 0.2 ms) and
 // testing all pairs cost about the same.  Three more rules skip
 // work whose outcome is known: the count leaves a row unit once all its rows
@@ -933,7 +933,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                 // all 256 columns in four groups of 64: the next group's TMEM load is
                 // in flight while this group is decided, and the accumulator goes
                 // back to the issuer before the last group is (groups of 32, given
-                // back at the end: 385 instead of COUNT64 us for the count of
+                // back at the end: 385 instead of 353 us for the count of
                 // 200,000 x 64, its warps waiting on tensor memory)
                 uint32_t ga[64], gb[64];
                 auto all_groups = [&](auto &&decide) {

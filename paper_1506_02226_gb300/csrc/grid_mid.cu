@@ -21,7 +21,7 @@
 //   scatter  rows grouped by cell: units padded to DP (4 or 8), -|u|^2, index
 //   nbrs     neighbour lists of the 27 offsets, own cell first (grid.cu)
 //   chunks   work items: 32-point chunks of every cell, so a dense cell is
-//            spread over many warps
+//            spread over many warps (one kernel)
 //   count    neighbour counts -> core flags (Section IV-B's fused pass); a
 //            chunk stops counting a point once it reaches min_pts unless exact
 //            counts are requested

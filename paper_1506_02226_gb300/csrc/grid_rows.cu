@@ -34,7 +34,7 @@
 //            pairs are skipped by one comparison;
 //   search   what is left, a list, a warp per cell pair (searched where they
 //            were found, a cell with a score of them held up its warp: the merge
-//            of 500,000 points in space took 141 us instead of MERGE_NOW).
+//            of 500,000 points in space took 141 us instead of 97).
 #include <algorithm>
 #include <climits>
 #include <type_traits>

@@ -101,13 +101,20 @@ __global__ void __launch_bounds__(256) wt_label_kernel(Rows R, int n, const int 
     if (threadIdx.x < 4 && red[threadIdx.x]) atomicAdd(ctr + 2 + threadIdx.x, (unsigned long long)red[threadIdx.x]);
 }
 
+// Bits of the counting sort's cells: about 2 n cells, at most 2^kWtMaxCellBits.
+int cell_bits(int64_t n) {
+    int lg = 1;
+    while ((int64_t(1) << lg) < n) ++lg;
+    return std::min(lg + 1, kWtMaxCellBits);
+}
+
 }  // namespace
 
 size_t wt_bytes(int64_t n) {
     const size_t nt = (size_t)((n + BT - 1) / BT), nr = nt * BT;
     auto al = [](size_t v) { return (v + 255) / 256 * 256; };
     return al(nt * sizeof(TileRec)) + al(nr * 32) + 8 * al(nr * 4) + al(nr) + al(nt * 128) + 2 * al(nt * 4) +
-           al((size_t)n * 4) + al(4 * ((size_t)1 << kWtMaxCellBits)) + 512;
+           al((size_t)n * 4) + al((size_t)4 << cell_bits(n)) + 512;
 }
 
 cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int32_t d, int64_t Tc, int32_t min_pts,
@@ -136,7 +143,7 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
     R.tag = static_cast<int *>(take((size_t)nt * 4));
     R.need = static_cast<int *>(take((size_t)nt * 4));
     o.inv = static_cast<int *>(take((size_t)n * 4));
-    int *hist = static_cast<int *>(take((size_t)4 << kWtMaxCellBits));
+    int *hist = static_cast<int *>(take((size_t)4 << cell_bits(n)));
     unsigned long long *work = static_cast<unsigned long long *>(take(64));
     Hdr *hdr = static_cast<Hdr *>(take(sizeof(Hdr)));
     o.cap_tiles = nt;
@@ -165,9 +172,7 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
 
     cudaError_t e;
     int *code = R.parent, *rank = R.border;  // free until the core kernel
-    int lg = 1;
-    while ((int64_t(1) << lg) < n) ++lg;
-    const int total = std::min({lg + 1, kWtMaxCellBits, 10 * d}), cells = 1 << total;
+    const int total = std::min(cell_bits(n), 10 * d), cells = 1 << total;
     if ((e = cudaMemsetAsync(hist, 0, sizeof(int) * (size_t)cells, st))) return e;
     const int nb = (n + 255) / 256;
     launch_dependent(wt_code_kernel, nb, 256, st, x, n, d, total, code, rank, hist);
