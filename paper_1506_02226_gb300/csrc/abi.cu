@@ -146,6 +146,12 @@ struct DeviceGuard {
 
 }  // namespace
 
+// Status of a run whose label kernel reported it (report_status).
+int plan_wait_reported(dbscan_plan *plan) {
+    if (cudaStreamSynchronize(plan->stream) != cudaSuccess) return DBSCAN_ERR_CUDA;
+    return plan_status_from_bits(*(volatile unsigned *)plan->h_status);
+}
+
 int plan_read_status(dbscan_plan *plan, bool clear) {
     cudaStream_t st = plan->stream;
     if (cudaMemcpyAsync(plan->h_status, plan->w.status, sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess)
@@ -186,6 +192,8 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     // these clear what they need themselves
     const bool small = eps_grid && n <= kGridSmallMaxN, rows = eps_grid && !small && grid_rows_serves(plan->w, g, n);
     const bool clears = small || rows;
+    const bool reported = o.synchronous && (!eps_grid || clears);  // by every path but grid.cu's
+    plan->w.status_out = reported ? plan->h_status : nullptr;
     if (!clears && o.synchronous && cudaMemsetAsync(plan->w.status, 0, sizeof(unsigned), st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
     if (!clears && cudaMemsetAsync(plan->w.ctr, 0, sizeof(unsigned long long) * DB_NCTR, st) != cudaSuccess)
@@ -250,7 +258,7 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     if (stats && cudaMemcpyAsync(plan->h_ctr, plan->w.ctr, sizeof(unsigned long long) * DB_NCTR,
                                  cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return DBSCAN_ERR_CUDA;
-    const int s = plan_read_status(plan, !o.synchronous);
+    const int s = reported ? plan_wait_reported(plan) : plan_read_status(plan, !o.synchronous);
     if (s) return s;
     if (stats) {
         const unsigned long long *c = plan->h_ctr;

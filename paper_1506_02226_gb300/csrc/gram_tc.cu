@@ -1784,9 +1784,11 @@ __global__ void __launch_bounds__(256) tc_label_kernel(int n, const uint8_t *__r
                                                        const int *__restrict__ parent, const int *__restrict__ border,
                                                        const int *__restrict__ least, const int *__restrict__ count,
                                                        int *__restrict__ labels, int *__restrict__ counts_out,
-                                                       uint8_t *__restrict__ core_out, unsigned long long *ctr) {
+                                                       uint8_t *__restrict__ core_out, unsigned long long *ctr,
+                                                       const unsigned *status, unsigned *status_out) {
     db::wait_prior_grid();  // started as a programmatic dependent
     db::allow_next_grid();
+    db::report_status(status, status_out);
     __shared__ int red[4];
     if (threadIdx.x < 4) red[threadIdx.x] = 0;
     __syncthreads();
@@ -2099,7 +2101,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     launch_dependent(tc_root_kernel, (n + 255) / 256, 256, st, n, w.core, perm, w.parent, least);
     w.marks->kernel("tc_root", st);
     launch_dependent(tc_label_kernel, (n + 255) / 256, 256, st, n, w.core, perm, inv, w.parent, w.border, least,
-                     w.count, labels, counts_out, core_out, w.ctr);
+                     w.count, labels, counts_out, core_out, w.ctr, w.status, w.status_out);
     w.marks->kernel("labels", st);
     return cudaGetLastError();
 }

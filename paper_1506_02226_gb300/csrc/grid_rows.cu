@@ -77,7 +77,7 @@ struct RowArgs {
     int *bord;
     int2 *pairs;              // merge: cell pairs left to a warp each, and their number
     int *npairs, pair_cap;
-    unsigned *status;
+    unsigned *status, *status_out;
     unsigned long long *ev;   // pair tests: [0] count, [1] merge, [2] border
 };
 
@@ -776,6 +776,7 @@ __global__ void __launch_bounds__(256) rows_root_kernel(RowArgs a) {
 __global__ void __launch_bounds__(256) rows_label_kernel(RowArgs a, int *__restrict__ labels, unsigned long long *ctr) {
     db::wait_prior_grid();
     db::allow_next_grid();
+    db::report_status(a.status, a.status_out);
     __shared__ int red[4];
     if (threadIdx.x < 4) red[threadIdx.x] = 0;
     __syncthreads();
@@ -886,6 +887,7 @@ cudaError_t run_rows(const DbWork &w, const RowGeom &g, const float *x, int n, i
     a.pair_cap = 2 * n;
     a.npairs = reinterpret_cast<int *>(w.ctr + DB_CTR_PAIRS);
     a.status = w.status;
+    a.status_out = w.status_out;
     a.ev = w.ctr + DB_CTR_EVAL;
     ScanArgs s{};
     s.part = w.rg_part;

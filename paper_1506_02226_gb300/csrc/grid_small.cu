@@ -4,8 +4,8 @@
 // The grid path (grid.cu) is a chain of some ten kernels; with a few thousand
 // points each of them works for a microsecond or two, and the launches, the
 // clears and the gaps between them are what a call takes (2,000 points in the
-// plane: 99 us a call, 70 with the merge on a forest in global memory, 60
-// as it is).  Here one thread block cluster runs the whole method: every block
+// plane: 99 us a call, 70 with the merge on a forest in global memory, 60 on
+// forests in shared memory, 50 with the status written to the host by the kernel).  Here one thread block cluster runs the whole method: every block
 // bins all points into its own shared memory (the binning is cheaper than
 // sharing it) and counts neighbours and finds border neighbours for its eighth
 // of the points.  The blocks meet when the core flags are known (each block
@@ -65,7 +65,7 @@ struct SmallArgs {
     GridGeom g;
     int *labels, *counts_out;
     uint8_t *core_out;
-    unsigned *status;
+    unsigned *status, *status_out;
     unsigned long long *ctr;
 };
 
@@ -566,6 +566,7 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
     __syncthreads();
     if (a.stats) db::block_sum_add(a.ctr + 1, cand);
     cluster_wait();
+    db::report_status(a.status, a.status_out);  // no block sets a bit after its arrival
 }
 
 }  // namespace
@@ -588,6 +589,7 @@ cudaError_t launch_grid_small(const DbWork &w, const GridGeom &g, const float *x
     a.counts_out = counts_out;
     a.core_out = core_out;
     a.status = w.status;
+    a.status_out = w.status_out;
     a.ctr = w.ctr;
     if ((1 << a.hbits) > kSlots || g.noff > 124) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(grid_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -144,6 +144,15 @@ __device__ __forceinline__ void block_sum_add(unsigned long long *dst, unsigned 
 __device__ __forceinline__ void wait_prior_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// The run's status word to the host, by the run's label kernel: every kernel that
+// can set a bit has completed by then.  (With a copy behind the
+// run instead, 2,000 points in the plane took 57.6 us a call, now 50.2; 6,007 x 32
+// 134, now 128.)
+__device__ __forceinline__ void report_status(const unsigned *status, unsigned *out) {
+    if (out && blockIdx.x == 0 && threadIdx.x == 0)
+        *(volatile unsigned *)out = (unsigned)ld_relaxed(reinterpret_cast<const int *>(status));
+}
+
 __device__ __forceinline__ unsigned lanemask_lt() {
     unsigned m;
     asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
@@ -218,6 +227,7 @@ struct DbWork {
     int64_t scan_part_cap;
     unsigned *status;       // device error bits
     unsigned long long *ctr;  // DB_NCTR counters (slots listed beside DB_NCTR)
+    unsigned *status_out;     // pinned host word for a run that is waited for (null: none), see report_status
     // grid path
     int64_t hcap;           // hash slots (power of two >= 2 cap_n)
     int32_t hbits;

@@ -28,9 +28,11 @@ __device__ __forceinline__ int block_sum(int v, int *red) {
 __global__ void labels_allpairs_kernel(int n, const uint8_t *__restrict__ core, int *parent,
                                        const int *__restrict__ border, const int *__restrict__ count,
                                        int *__restrict__ labels, int *__restrict__ counts_out,
-                                       uint8_t *__restrict__ core_out, unsigned long long *ctr) {
+                                       uint8_t *__restrict__ core_out, unsigned long long *ctr,
+                                       const unsigned *status, unsigned *status_out) {
     db::wait_prior_grid();
     db::allow_next_grid();
+    db::report_status(status, status_out);
     __shared__ int red[32];
     int nc = 0, nb = 0, nn = 0, nr = 0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
@@ -231,7 +233,7 @@ cudaError_t launch_bucket_scan(int32_t *v, int32_t n, cudaStream_t st) {
 cudaError_t launch_labels_allpairs(const DbWork &w, int64_t n, int32_t *labels, int32_t *counts_out,
                                    uint8_t *core_out, cudaStream_t st) {
     launch_dependent(labels_allpairs_kernel, grid_for(n), 256, st, (int)n, w.core, w.parent, w.border, w.count, labels,
-                                                        counts_out, core_out, w.ctr);
+                                                        counts_out, core_out, w.ctr, w.status, w.status_out);
     w.marks->kernel("labels", st);
     return cudaGetLastError();
 }

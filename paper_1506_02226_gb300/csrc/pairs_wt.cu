@@ -66,9 +66,10 @@ __global__ void __launch_bounds__(256) wt_pack_kernel(const float *__restrict__ 
 __global__ void __launch_bounds__(256) wt_label_kernel(Rows R, int n, const int *__restrict__ inv,
                                                        const int *__restrict__ least, int *__restrict__ labels,
                                                        int *__restrict__ counts_out, uint8_t *__restrict__ core_out,
-                                                       unsigned long long *ctr) {
+                                                       unsigned long long *ctr, unsigned *status_out) {
     db::wait_prior_grid();
     db::allow_next_grid();
+    db::report_status(R.status, status_out);
     __shared__ int red[4];
     if (threadIdx.x < 4) red[threadIdx.x] = 0;
     __syncthreads();
@@ -198,7 +199,8 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
     w.marks->kernel("wt_border", st);
     launch_dependent(root_kernel, std::min(nr / 64, 152 * 8), NT, st, R, hdr, o.least);
     w.marks->kernel("wt_root", st);
-    launch_dependent(wt_label_kernel, nb, 256, st, R, n, o.inv, o.least, labels, counts_out, core_out, w.ctr);
+    launch_dependent(wt_label_kernel, nb, 256, st, R, n, o.inv, o.least, labels, counts_out, core_out, w.ctr,
+                     w.status_out);
     w.marks->kernel("labels", st);
     return cudaGetLastError();
 }
