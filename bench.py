@@ -174,10 +174,10 @@ def grid_offsets(d: int, T: int):
 # source means the counters no longer describe the kernel, and the bench line
 # reports traffic null.
 NCU_TRAFFIC = {
-    ("lowd2", "grid_count"): (17994496, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
-    ("lowd2", "grid_union_near"): (11583000, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
-    ("lowd3", "grid_count"): (43683072, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
-    ("lowd3", "grid_union_near"): (57444000, "paper_1506_02226_gb300/csrc/grid_rows.cu", "8245be43dd18"),
+    ("lowd2", "grid_count"): (17999872, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
+    ("lowd2", "grid_union_near"): (11558656, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
+    ("lowd3", "grid_count"): (43691776, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
+    ("lowd3", "grid_union_near"): (57448704, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
 }
 
 

@@ -1,4 +1,4 @@
-// grid_small.cu — the eps-grid path for small point sets (d <= 3, up to 4,096
+// grid_small.cu — the eps-grid path for small point sets (d <= 3, up to 2,048
 // points), in one launch.
 //
 // The grid path (grid.cu) is a chain of some ten kernels; with a few thousand
@@ -15,6 +15,11 @@
 // a set and block.  One forest in global memory, with eight blocks linking the
 // same few roots, took 25 us of the call; all pairs in every block took 58.
 //
+// The limit: on eight SMs the time grows with n, on the whole chip it hardly does.
+// Calls on the field recipe, this kernel / the chain of grid_rows.cu: 1,000
+// points 50 / 84 us in the plane and 66 / 92 in space, 2,000 71 / 91 and 94 / 101,
+// 2,500 81 / 84 and 104 / 103, 4,096 108 / 90 and 130 / 106.
+//
 // The geometry, the exact test, the order of decisions and so the labels are
 // grid.cu's: cells are cliques, cell pairs within the kept offsets are
 // candidates, a cell's representative is its smallest core index, and only
@@ -29,10 +34,11 @@ namespace cg = cooperative_groups;
 
 namespace {
 
-constexpr int kMaxN = kGridSmallMaxN;  // 4,096
+constexpr int kMaxN = kGridSmallMaxN;  // 2,048
 constexpr int NB = 8, NT = 512;        // blocks of the cluster, threads of a block: at most one own point a thread
 constexpr int kSlots = 2 * kMaxN;      // cell hash
 constexpr int kList = 2048;            // merge: cell pairs in two sets, a warp each
+constexpr int kHookSteps = 4;          // merge: steps of 32 tests for a cell and one neighbour when it is hooked
 constexpr float kFar = -1e30f;         // near nothing
 constexpr unsigned FULL = 0xffffffffu;
 static_assert(kList * sizeof(unsigned) >= kMaxN * sizeof(uint16_t), "the list's place holds a forest");
@@ -163,23 +169,34 @@ __device__ __forceinline__ bool near(float cp, float px2, float py2, float pz2, 
     return fmaf(pz2, q.z, fmaf(py2, q.y, fmaf(px2, q.x, cp + q.w))) >= 1.f;
 }
 
-// Is a core point of cell a near one of cell b?  By GL lanes, a product of the
-// two cells' points each (a thread alone walks a chain of two dependent loads a
-// test); `mask` holds the group's lanes.
+// Is a core point of cell a near one of cell b?  By GL lanes (`mask`), each with a
+// point of the larger cell, against four points of the smaller a step; at most
+// max_steps steps, then false with `all` cleared.
 template <int GL>
 __device__ __forceinline__ bool cells_near(const SmallSmem &S, float Tp1, int sa, int sb, int sub, unsigned mask,
-                                           unsigned long long &tests) {
-    const unsigned ra = S.range[sa], rb = S.range[sb], nb = rb & 0xffffu, all = (ra & 0xffffu) * nb;
-    for (unsigned k0 = 0; k0 < all; k0 += GL) {
-        const unsigned k = k0 + (unsigned)sub;
-        bool hit = false;
-        if (k < all) {
-            const unsigned q = k / nb;
-            const float4 pa = S.pt[(ra >> 16) + q], pb = S.pt[(rb >> 16) + k - q * nb];
-            hit = near(Tp1 + pa.w, 2.f * pa.x, 2.f * pa.y, 2.f * pa.z, pb);
-            ++tests;
+                                           int max_steps, bool &all, unsigned long long &tests) {
+    unsigned ra = S.range[sa], rb = S.range[sb];
+    if ((ra & 0xffffu) < (rb & 0xffffu)) {
+        const unsigned t = ra;
+        ra = rb;
+        rb = t;
+    }
+    const int a0 = (int)(ra >> 16), a1 = a0 + (int)(ra & 0xffffu), b0 = (int)(rb >> 16), b1 = b0 + (int)(rb & 0xffffu);
+    int steps = 0;
+    for (int x0 = a0; x0 < a1; x0 += GL) {
+        const float4 pa = S.pt[min(x0 + sub, a1 - 1)];  // past the end: the last point again
+        const float cp = Tp1 + pa.w, px2 = 2.f * pa.x, py2 = 2.f * pa.y, pz2 = 2.f * pa.z;
+        for (int y0 = b0; y0 < b1; y0 += 4) {
+            if (steps++ == max_steps) {
+                all = false;
+                return false;
+            }
+            bool hit = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) hit |= near(cp, px2, py2, pz2, S.pt[min(y0 + u, b1 - 1)]);
+            if (x0 + sub < a1) tests += (unsigned)min(4, b1 - y0);
+            if (__ballot_sync(mask, hit) & mask) return true;
         }
-        if (__ballot_sync(mask, hit) & mask) return true;
     }
     return false;
 }
@@ -327,9 +344,13 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
                     const int q0 = (int)(r >> 16), q1 = q0 + (int)(r & 0xffffu);
                     cand += r & 0xffffu;
                     if (count + add >= lim) continue;
+                    int q = q0;
+                    while (q < q1 && count + add < lim) {  // (a tight blob's cell: not all of it)
+                        const int qe = min(q + 32, q1);
 #pragma unroll 4
-                    for (int q = q0; q < q1; ++q) add += near(cp, px2, py2, pz2, S.pt[q]);
-                    ev_count += r & 0xffffu;
+                        for (; q < qe; ++q) add += near(cp, px2, py2, pz2, S.pt[q]);
+                    }
+                    ev_count += (unsigned)(q - q0);
                 }
             }
             __syncwarp();
@@ -387,7 +408,8 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
                 if (mb >= 0 && S.rep[mb] == DB_NONE) mb = -1;
                 for (unsigned left = __ballot_sync(mask, mb >= 0) & mask; left && !hit; left &= left - 1) {
                     const int sb = __shfl_sync(mask, mb, __ffs(left) - 1);
-                    hit = cells_near<8>(S, Tp1, sa, sb, sub8, mask, ev_merge);
+                    bool all = true;
+                    hit = cells_near<8>(S, Tp1, sa, sb, sub8, mask, kHookSteps, all, ev_merge);
                     if (hit) cluster.map_shared_rank(par, sub8)[S.rep[sa]] = (uint16_t)S.rep[sb];
                 }
             }
@@ -432,7 +454,8 @@ __global__ void __cluster_dims__(NB, 1, 1) __launch_bounds__(NT, 1) grid_small_k
                 const int sa = (int)(S.list[e] >> 16), sb = (int)(S.list[e] & 0xffffu);
                 const int same = lane == 0 && find_root(par, S.rep[sa]) == find_root(par, S.rep[sb]);
                 if (__shfl_sync(FULL, same, 0)) continue;
-                if (cells_near<32>(S, Tp1, sa, sb, lane, FULL, ev_merge) && lane == 0)
+                bool all = true;
+                if (cells_near<32>(S, Tp1, sa, sb, lane, FULL, INT_MAX, all, ev_merge) && lane == 0)
                     unite(par, S.rep[sa], S.rep[sb], a.status);
                 __syncwarp();
             }

@@ -310,7 +310,7 @@ cudaError_t launch_grid_path(const DbWork &w, const GridGeom &g, const float *x,
 // The whole eps-grid run of up to kGridSmallMaxN points in one launch
 // (grid_small.cu), labels dense when `compact`; clears the run's counters, and
 // the status word when `reset` is set.
-constexpr int kGridSmallMaxN = 4096;
+constexpr int kGridSmallMaxN = 2048;
 cudaError_t launch_grid_small(const DbWork &w, const GridGeom &g, const float *x, int64_t n, int32_t min_pts, bool exact,
                               bool compact, bool stats, bool reset, int32_t *labels, int32_t *counts_out,
                               uint8_t *core_out, cudaStream_t st);

@@ -1,4 +1,4 @@
-"""The one-launch eps-grid run (d <= 3, up to 4,096 points) against the oracle, bit for bit.
+"""The one-launch eps-grid run (d <= 3, up to 2,048 points) against the oracle, bit for bit.
 
 Sizes around a block's share of the points and the limit, sparse points (one a
 cell), dense cells whose pairs go to whole warps, lattices whose cell pairs
@@ -36,7 +36,7 @@ def points(kind, n, d, rng):
 def test_small_grid_run(kind, d):
     from paper_1506_02226_gb300.api import Plan
     rng = np.random.default_rng(40 * d + len(kind))
-    for n in (1, 2, 7, 8, 9, 511, 513, 2000, 4095, 4096, 4097):
+    for n in (1, 2, 7, 8, 9, 511, 513, 2000, 2047, 2048, 2049, 4096):
         u, eps_units, min_pts = points(kind, n, d, rng)
         x = np.ascontiguousarray(np.clip(u, 0, 1023).astype(np.float32) / np.float32(1024))
         xt = torch.from_numpy(x).cuda()
@@ -49,7 +49,7 @@ def test_small_grid_run(kind, d):
                 np.testing.assert_array_equal(k.cpu().numpy().astype(bool), core)
                 np.testing.assert_array_equal(lab.cpu().numpy(), want, err_msg=f"n={n} mode={mode}")
                 assert st["path"] == B.DBSCAN_PATH_GRID
-                assert (st["kernels"] == 1) == (n <= 4096)
+                assert (st["kernels"] == 1) == (n <= 2048)
                 assert st["n_core"] == int(core.sum()) and st["n_core"] + st["n_border"] + st["n_noise"] == n
                 assert st["n_clusters"] == len(set(want[core].tolist()))
                 assert st["candidate_pairs"] >= int(cnt.sum()) and st["pair_tests"] == sum(p.pair_tests())
