@@ -110,6 +110,7 @@
 #include <type_traits>
 
 #include "internal.cuh"
+#include "tc_items.h"
 
 namespace {
 
@@ -490,10 +491,11 @@ __device__ __noinline__ int unite_sets(int *parent, int x, int y, unsigned *stat
 // come first: their neighbours settle most counts and unions, and the rules
 // below then drop later items.
 template <int PASS, int RTN>
-__device__ __forceinline__ unsigned item_mask(const TcArgs &a, int w, int units, int nct, int &u, int &c0) {
+__device__ __forceinline__ unsigned item_mask(const TcArgs &a, int64_t w, int units, int nct, int &u, int &c0) {
     const int nchunk = (nct + a.ct_chunk - 1) / a.ct_chunk;
-    const int rel = a.rel_lo + w / units;
-    u = w - (w / units) * units;
+    const tcitems::Item it = tcitems::item(w, units);
+    const int rel = a.rel_lo + it.rel;
+    u = it.unit;
     const int i = RTN == 2 ? u : u >> 1;  // the unit's tile
     int ch = rel;
     if (PASS == TC_UNION || PASS == TC_ADJ || a.rotate) ch += i / a.ct_chunk;
@@ -533,8 +535,9 @@ __global__ void __launch_bounds__(256) tc_items_kernel(TcArgs a) {
     db::wait_prior_grid();  // started as a programmatic dependent
     db::allow_next_grid();
     const int units = (a.nR + TM * RTN - 1) / (TM * RTN), nct = (a.nC + TN - 1) / TN;
-    const int nitems = units * (a.rel_hi - a.rel_lo), lane = threadIdx.x & 31;
-    const int w = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+    const int64_t nitems = tcitems::count(units, a.rel_hi - a.rel_lo);
+    const int lane = threadIdx.x & 31;
+    const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int u = 0, c0 = 0;
     const unsigned m = w < nitems ? item_mask<PASS, RTN>(a, w, units, nct, u, c0) : 0u;
     const unsigned on = __ballot_sync(FULL, m != 0);
@@ -563,7 +566,7 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
     Smem &S = *reinterpret_cast<Smem *>(smem_raw + pad);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int units = (a.nR + TMU - 1) / TMU, nct = (a.nC + TN - 1) / TN;
-    const int nitems = units * (a.rel_hi - a.rel_lo);
+    const int64_t nitems = tcitems::count(units, a.rel_hi - a.rel_lo);
 
     volatile int *abort_flag = &S.abort_flag;
     if (threadIdx.x == 0) {
@@ -705,11 +708,11 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                 e1 = e2;
             }
         } else {
-            for (int base = blockIdx.x; base < nitems && ok; base += (int)gridDim.x * 32) {
-                const int w = base + lane * (int)gridDim.x;
+            for (int64_t base = blockIdx.x; base < nitems && ok; base += tcitems::round((int)gridDim.x)) {
+                const int64_t w = tcitems::dealt(base, lane, (int)gridDim.x);
                 int u = 0, c0 = 0;
                 unsigned mask = 0;
-                if (w < nitems && w >= 0) mask = item_mask<PASS, RTN>(a, w, units, nct, u, c0);
+                if (w < nitems) mask = item_mask<PASS, RTN>(a, w, units, nct, u, c0);
                 unsigned live = __ballot_sync(FULL, mask != 0);
                 while (live && ok) {
                     const int l = __ffs(live) - 1;
@@ -1851,14 +1854,6 @@ int sm_count() {
     return sms;
 }
 
-// Column tiles per work item: about 8 items per SM, a power of two up to 16
-// (an item of 16 tiles keeps an SM busy for some 20 us, the longest tail).
-int chunk_tiles(int64_t units, int64_t nct, int sms) {
-    int c = 16;
-    while (c > 1 && units * ((nct + c - 1) / c) < (int64_t)8 * sms) c >>= 1;
-    return c;
-}
-
 // Merge: the tiles after a row unit's own that are taken first.
 constexpr int kNearTiles = 2;
 
@@ -1994,7 +1989,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
         c.tile_r = TN * K;
         c.tile_c = bf16 ? TN * K : tile;
         c.near = w.tc_pairs;
-        c.ct_chunk = chunk_tiles((2 * nt + 255) / 256, nt, sms);
+        c.ct_chunk = tcitems::chunk_tiles((2 * nt + 255) / 256, nt, sms);
         c.rel_lo = 0;
         c.rel_hi = (nt + c.ct_chunk - 1) / c.ct_chunk;
         if ((e = launch_pass_t<TC_CULL, false>(c, sms, st))) return e;
@@ -2020,7 +2015,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     a.stall = stall ? 1 : 0;
     if (stall) a.wait_ns = 50000000ull;
     const int units1 = (n + TM - 1) / TM;  // units of one row tile
-    a.ct_chunk = chunk_tiles(bf16 ? units1 : nt, nt, sms);
+    a.ct_chunk = tcitems::chunk_tiles(bf16 ? units1 : nt, nt, sms);
     a.rel_lo = 0;
     a.rel_hi = (nt + a.ct_chunk - 1) / a.ct_chunk;
     // opCore is free from here on: adjacency words, then the item list (when it fits)
@@ -2030,7 +2025,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     int next_list = 1;  // tc_lens[1..6]: length and ticket of up to three lists, cleared above
     auto use_list = [&](auto pass) -> cudaError_t {
         constexpr int PASS = decltype(pass)::value;
-        const int64_t units = bf16 || PASS == TC_UNION ? (n + TM - 1) / TM : nt, nit = units * (a.rel_hi - a.rel_lo);
+        const int64_t units = bf16 || PASS == TC_UNION ? (n + TM - 1) / TM : nt, nit = tcitems::count((int)units, a.rel_hi - a.rel_lo);
         a.items = nullptr;
         if (!sorted || nit > list_cap) return cudaSuccess;
         a.nlist = w.tc_lens + next_list++;
@@ -2059,7 +2054,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     // near tiles; then the rest, most of which the sets found so far skip.
     a.metaR = a.metaC = mcore;
     a.fold = 0;
-    const int ch_union = chunk_tiles(units1, nt, sms), nch = (nt + ch_union - 1) / ch_union;
+    const int ch_union = tcitems::chunk_tiles(units1, nt, sms), nch = (nt + ch_union - 1) / ch_union;
     a.ct_chunk = ch_union;
     a.rel_lo = 0;
     a.rel_hi = 1;
@@ -2091,7 +2086,7 @@ cudaError_t launch_allpairs_tc(const DbWork &w, const float *x, int64_t n64, int
     // pass 3: smallest core neighbour of the rows that need one
     a.metaR = mneed;
     a.metaC = mcore;
-    a.ct_chunk = chunk_tiles(bf16 ? units1 : nt, nt, sms);
+    a.ct_chunk = tcitems::chunk_tiles(bf16 ? units1 : nt, nt, sms);
     a.rel_lo = 0;
     a.rel_hi = (nt + a.ct_chunk - 1) / a.ct_chunk;
     if ((e = use_list(std::integral_constant<int, TC_BORDER>{}))) return e;
@@ -2139,7 +2134,7 @@ cudaError_t launch_tc_verify(const DbWork &w, const float *x, int64_t n64, int32
     a.opR = a.opC = w.opAll;
     a.metaR = a.metaC = reinterpret_cast<const MetaTile *>(w.metaAll);
     a.nR = a.nC = n;
-    a.ct_chunk = chunk_tiles((n + TM - 1) / TM, nt, sms);
+    a.ct_chunk = tcitems::chunk_tiles((n + TM - 1) / TM, nt, sms);
     a.rel_lo = 0;
     a.rel_hi = (nt + a.ct_chunk - 1) / a.ct_chunk;
     return launch_pass<TC_VERIFY>(a, bf16, sms, st);
