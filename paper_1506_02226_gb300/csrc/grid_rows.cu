@@ -541,7 +541,8 @@ __global__ void __launch_bounds__(256) rows_union_kernel(RowArgs a) {
                 ++ev;
                 bool hit = is_nbr<D>(a.g.Tp1 + m.w, 2.f * m.x, 2.f * m.y, 2.f * m.z, unpack_point(a.mid[id]));
                 const int sA = a.start[c], eA = a.start[c + 1], sB = a.start[id], eB = a.start[id + 1];
-                if (!hit && (eA - sA) * (eB - sB) <= kLaneTests) {  // few pairs: the lane tests them itself
+                // few pairs (64 bits: two hot spots make more than an int holds): the lane tests them itself
+                if (!hit && (long long)(eA - sA) * (eB - sB) <= kLaneTests) {
                     need = false;
                     for (int qa = sA; qa < eA && !hit; ++qa) {
                         if (!a.score[qa]) continue;
