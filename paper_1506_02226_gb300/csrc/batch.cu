@@ -29,12 +29,15 @@
 #include <cstring>
 #include <vector>
 
+#include "batch_items.h"
 #include "plan.h"
 #include "warp_tile.cuh"
 
 using namespace wtile;
 
 namespace {
+
+static_assert(BT == batchitems::kTileRows, "rows of a tile");
 
 struct BInst {
     const float *x;
@@ -556,13 +559,10 @@ extern "C" int dbscan_batch(dbscan_plan *plan, const dbscan_instance *inst, int3
         items += rows * ((cols + 3) / 4);
     }
     if (items > INT32_MAX) return DBSCAN_ERR_UNSUPPORTED;
-    // Rows are counted in int32 (64 per tile): a batch of more tiles (tens of
-    // millions of tiny instances) runs in parts.
+    // Rows are counted in int32: a batch of very many tiles runs in parts.
     unsigned long long tot[4] = {0, 0, 0, 0};
     for (int32_t i = 0; i < count;) {
-        int64_t tiles = 0;
-        int32_t end = i;
-        while (end < count && tiles + (inst[end].n + BT - 1) / BT <= INT32_MAX / BT) tiles += (inst[end++].n + BT - 1) / BT;
+        const int32_t end = batchitems::part_end(i, count, [&](int32_t k) { return inst[k].n; });
         const int s = batch_run(plan, inst + i, end - i, per_inst ? per_inst + i : nullptr, tot);
         if (s) return s;
         i = end;

@@ -1,0 +1,44 @@
+"""A batch of more tiles than one part takes (2^20): every instance of every part
+gets its labels and statistics."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1506_02226_gb300 import binding as B
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+INSTANCE = np.dtype({"names": ["points", "n", "d", "eps", "min_pts", "labels"],
+                     "formats": ["<u8", "<i8", "<i4", "<f4", "<i4", "<u8"],
+                     "offsets": [0, 8, 16, 20, 24, 32], "itemsize": 40})
+
+
+def test_more_than_a_part():
+    from paper_1506_02226_gb300.api import Plan
+    rng = np.random.default_rng(5)
+    sizes = np.array([3, 1, 0, 5, 2], dtype=np.int64)
+    pool = [(rng.integers(0, 60, size=(s, 2)) / 1024).astype(np.float32) for s in sizes]
+    eps, min_pts, count = 25 / 1024, 2, 1_400_003
+    want = [oracle.dbscan(p, eps, min_pts)[0] if len(p) else np.zeros(0, np.int32) for p in pool]
+    kind = np.arange(count) % len(pool)
+    n = sizes[kind]
+    first = np.concatenate([[0], np.cumsum(n)[:-1]])
+    x = torch.from_numpy(np.concatenate(pool)).cuda()
+    at = np.concatenate([[0], np.cumsum(sizes)[:-1]])[kind]
+    labels = torch.full((int(n.sum()),), -9, dtype=torch.int32, device="cuda")
+    assert (n > 0).sum() > 1 << 20
+    t = np.zeros(count, INSTANCE)
+    t["points"], t["n"], t["d"], t["eps"] = x.data_ptr() + 8 * at, n, 2, eps
+    t["min_pts"], t["labels"] = min_pts, labels.data_ptr() + 4 * first
+    insts = (B.dbscan_instance * count).from_buffer(t)
+    st = (B.dbscan_stats * count)()
+    with Plan(max_n=16, max_d=2) as p:
+        assert B.dbscan_batch(p.handle, insts, st) == B.DBSCAN_OK
+    whole = np.concatenate(want)
+    reps = -(-count // len(pool))
+    np.testing.assert_array_equal(labels.cpu().numpy(), np.tile(whole, reps)[:len(labels)])
+    got = np.frombuffer(st, dtype=np.dtype({"names": ["n_core"], "formats": ["<i8"],
+                                            "offsets": [B.dbscan_stats.n_core.offset], "itemsize": 96}))["n_core"]
+    cores = np.array([oracle.dbscan(p, eps, min_pts)[2].sum() if len(p) else 0 for p in pool])
+    np.testing.assert_array_equal(got, cores[kind])
