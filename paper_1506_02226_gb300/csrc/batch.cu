@@ -39,6 +39,11 @@ namespace {
 
 static_assert(BT == batchitems::kTileRows, "rows of a tile");
 
+struct BHdr {  // the sizes of a run, and the tiles before each step of its passes
+    Hdr h;
+    unsigned first[batchitems::kMaxSteps + 1];
+};
+
 struct BInst {
     const float *x;
     int32_t *labels;
@@ -165,6 +170,7 @@ __global__ void batch_compact_kernel(Rows R, const Hdr *__restrict__ hdr, const 
 
 constexpr int kCH[] = {64, 256};
 constexpr int kBPS[] = {4, 8};
+static_assert(kCH[0] == batchitems::kMinChunk && kCH[1] % kCH[0] == 0, "the tiles' order holds for every chunk");
 constexpr int kSortMax = 16384;  // largest instance reordered (160 KiB of shared memory, 16-bit starts)
 constexpr size_t sort_bytes(int cap) { return (size_t)cap * (2 * sizeof(unsigned) + sizeof(uint16_t)); }
 
@@ -176,19 +182,20 @@ struct BatchState {
     void *dev = nullptr;
     size_t dev_bytes = 0;
     BInst *d_table = nullptr;
-    Hdr *d_hdr = nullptr;
+    Hdr *d_hdr = nullptr;      // the head of a BHdr
+    const unsigned *d_first = nullptr;  // and its table
     Rows rows{};               // by row and tile (ev set per launch)
     PackOut pack{};            // the same arrays, writable
     int *d_flags = nullptr, *d_scan = nullptr, *d_part = nullptr;  // by point
     int64_t part_cap = 0;
     int sort_cap = 0;          // instances up to this many points are reordered (a power of two)
-    unsigned long long *d_work = nullptr;
+    unsigned *d_work = nullptr;
     unsigned *d_status = nullptr;
     int *d_istats = nullptr;
     unsigned long long *d_ev = nullptr;  // pair tests evaluated per instance and pass [count][3]
     unsigned long long *h_ev = nullptr;
     BInst *h_table = nullptr;
-    Hdr *h_hdr = nullptr;
+    BHdr *h_hdr = nullptr;
     int *h_istats = nullptr;
     unsigned *h_status = nullptr;
     cudaGraphExec_t graph = nullptr;
@@ -227,12 +234,12 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
         off = al256(off + bytes);
         return o;
     };
-    const size_t o_table = take(sizeof(BInst) * nc), o_hdr = take(sizeof(Hdr)), o_tiles = take(sizeof(TileRec) * nt),
+    const size_t o_table = take(sizeof(BInst) * nc), o_hdr = take(sizeof(BHdr)), o_tiles = take(sizeof(TileRec) * nt),
                  o_P16 = take(32 * nr), o_nb = take(4 * nr), o_nbc = take(4 * nr), o_box = take(128 * nt),
                  o_count = take(4 * nr), o_core = take(nr), o_parent = take(4 * nr), o_border = take(4 * nr),
                  o_perm = take(4 * nr), o_least = take(4 * nr), o_tag = take(4 * nt), o_need = take(4 * nt),
                  o_inv = take(4 * np), o_flags = take(4 * np), o_scan = take(4 * (np + 1)), o_part = take(4 * part),
-                 o_work = take(8 * 8), o_status = take(16), o_istats = take(16 * nc), o_ev = take(24 * (size_t)nc);
+                 o_work = take(4 * 8), o_status = take(16), o_istats = take(16 * nc), o_ev = take(24 * (size_t)nc);
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
@@ -255,13 +262,14 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
         cudaMallocHost(&b->h_istats, 16 * (size_t)nc) != cudaSuccess ||
         cudaMallocHost(&b->h_ev, 24 * (size_t)nc) != cudaSuccess)
         return DBSCAN_ERR_OOM;
-    if (!b->h_hdr && cudaMallocHost(&b->h_hdr, sizeof(Hdr)) != cudaSuccess) return DBSCAN_ERR_OOM;
+    if (!b->h_hdr && cudaMallocHost(&b->h_hdr, sizeof(BHdr)) != cudaSuccess) return DBSCAN_ERR_OOM;
     if (!b->h_status && cudaMallocHost(&b->h_status, 16) != cudaSuccess) return DBSCAN_ERR_OOM;
     char *base = static_cast<char *>(b->dev);
     auto at = [&](size_t o) { return static_cast<void *>(base + o); };
     b->dev_bytes = off;
     b->d_table = static_cast<BInst *>(at(o_table));
     b->d_hdr = static_cast<Hdr *>(at(o_hdr));
+    b->d_first = reinterpret_cast<const BHdr *>(b->d_hdr)->first;
     PackOut &w = b->pack;
     w.tiles = static_cast<TileRec *>(at(o_tiles));
     w.perm = static_cast<int *>(at(o_perm));
@@ -290,7 +298,7 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
     b->d_scan = static_cast<int *>(at(o_scan));
     b->d_part = static_cast<int *>(at(o_part));
     b->part_cap = part;
-    b->d_work = static_cast<unsigned long long *>(at(o_work));
+    b->d_work = static_cast<unsigned *>(at(o_work));
     b->d_status = r.status = static_cast<unsigned *>(at(o_status));
     b->d_istats = static_cast<int *>(at(o_istats));
     b->d_ev = static_cast<unsigned long long *>(at(o_ev));
@@ -301,11 +309,12 @@ int batch_reserve(BatchState *b, int count, int64_t points, int64_t tiles) {
     return DBSCAN_OK;
 }
 
-// Host table; returns the tiles of the largest instance.
-int64_t build_table(const dbscan_instance *inst, int count, BInst *t, int64_t *points, int64_t *tiles,
-                    int64_t *max_n) {
+// Host table, rows and tiles given out in the order of the passes' queue.
+void build_table(const dbscan_instance *inst, int count, const batchitems::Queue &q, BInst *t, int64_t *points,
+                 int64_t *tiles, int64_t *max_n) {
     int64_t base = 0, nt = 0, mx = 0;
-    for (int i = 0; i < count; ++i) {
+    for (int k = 0; k < count; ++k) {
+        const int i = q.order.empty() ? k : q.order[k];
         const dbscan_instance &in = inst[i];
         BInst &B = t[i];
         B = BInst{};
@@ -332,7 +341,6 @@ int64_t build_table(const dbscan_instance *inst, int count, BInst *t, int64_t *p
     *points = base;
     *tiles = nt;
     *max_n = mx;
-    return (mx + BT - 1) / BT;
 }
 
 cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int bps, cudaStream_t st,
@@ -346,8 +354,8 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
     cudaError_t e;
     if ((e = cudaMemcpyAsync(b->d_table, b->h_table, sizeof(BInst) * b->cap_count, cudaMemcpyHostToDevice, st)))
         return e;
-    if ((e = cudaMemcpyAsync(b->d_hdr, b->h_hdr, sizeof(Hdr), cudaMemcpyHostToDevice, st))) return e;
-    if ((e = cudaMemsetAsync(b->d_work, 0, 8 * 8, st))) return e;
+    if ((e = cudaMemcpyAsync(b->d_hdr, b->h_hdr, sizeof(BHdr), cudaMemcpyHostToDevice, st))) return e;
+    if ((e = cudaMemsetAsync(b->d_work, 0, 4 * 8, st))) return e;
     if (stats && (e = cudaMemsetAsync(b->d_istats, 0, 16 * (size_t)b->cap_count, st))) return e;
     if (stats && (e = cudaMemsetAsync(b->d_ev, 0, 24 * (size_t)b->cap_count, st))) return e;
     Rows R = b->rows;
@@ -355,17 +363,17 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
     batch_sortpack_kernel<<<sms * 3, 512, sort_bytes(b->sort_cap), st>>>(b->d_table, b->d_hdr, b->sort_cap, b->pack,
                                                                         b->d_status);
     pm->kernel("batch_prep", st);
-    pass_kernel<WT_COUNT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 0);
+    pass_kernel<WT_COUNT, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 0);
     pm->kernel("batch_count", st);
     core_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
     pm->kernel("batch_core", st);
-    pass_kernel<WT_NEAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 1);
+    pass_kernel<WT_NEAR, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 1);
     pm->kernel("batch_union_near", st);
     flatten_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
     pm->kernel("batch_flatten", st);
-    pass_kernel<WT_FAR><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 2);
+    pass_kernel<WT_FAR, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 2);
     pm->kernel("batch_union", st);
-    pass_kernel<WT_BORDER><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_work + 3);
+    pass_kernel<WT_BORDER, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 3);
     pm->kernel("batch_border", st);
     root_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->pack.least);
     pm->kernel("batch_root", st);
@@ -443,7 +451,9 @@ int batch_run(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, dbs
 
     std::vector<BInst> tmp(count);
     int64_t points = 0, tiles = 0, max_n = 0;
-    const int64_t max_tiles = build_table(inst, count, tmp.data(), &points, &tiles, &max_n);
+    const batchitems::Queue queue = batchitems::make_queue(count, [&](int32_t k) { return inst[k].n; });
+    if (!queue.fits) return DBSCAN_ERR_UNSUPPORTED;
+    build_table(inst, count, queue, tmp.data(), &points, &tiles, &max_n);
     int s = batch_reserve(b, count, points, tiles);
     if (s) return s;
     // Instances up to kSortMax points are put in Z-order; the sort's shared
@@ -463,10 +473,8 @@ int batch_run(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, dbs
     std::memcpy(b->h_table, tmp.data(), sizeof(BInst) * count);
     if (b->cap_count > count) std::memset(b->h_table + count, 0, sizeof(BInst) * (b->cap_count - count));
     auto prepare = [&](int ch) {
-        b->h_hdr->count = count;
-        b->h_hdr->total_points = (int)points;
-        b->h_hdr->total_tiles = (int)tiles;
-        b->h_hdr->max_chunks = (int)((max_tiles + ch - 1) / ch);
+        b->h_hdr->h = Hdr{count, (int)points, (int)tiles,
+                          batchitems::step_table(queue, ch / batchitems::kMinChunk, b->h_hdr->first)};
     };
 
     if (!b->tuned) {

@@ -50,11 +50,11 @@ __global__ void __launch_bounds__(256) wt_scatter_kernel(int n, const int *__res
 
 __global__ void __launch_bounds__(256) wt_pack_kernel(const float *__restrict__ x, TileRec I,
                                                       const int *__restrict__ order, PackOut w, Hdr h, Hdr *hdr,
-                                                      unsigned long long *work, unsigned *status) {
+                                                      unsigned *work, unsigned *status) {
     db::wait_prior_grid();
     db::allow_next_grid();
     const int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-    if (blockIdx.x == 0 && threadIdx.x < 4) work[threadIdx.x] = 0ull;
+    if (blockIdx.x == 0 && threadIdx.x < 4) work[threadIdx.x] = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) *hdr = h;
     if (T >= I.ntiles) return;
     if (pack_tile_d(x, I, T, order, w)) atomicOr(status, DB_EBIT_NOT_QUANTISED);
@@ -145,7 +145,7 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
     R.need = static_cast<int *>(take((size_t)nt * 4));
     o.inv = static_cast<int *>(take((size_t)n * 4));
     int *hist = static_cast<int *>(take((size_t)4 << cell_bits(n)));
-    unsigned long long *work = static_cast<unsigned long long *>(take(64));
+    unsigned *work = static_cast<unsigned *>(take(64));
     Hdr *hdr = static_cast<Hdr *>(take(sizeof(Hdr)));
     o.cap_tiles = nt;
     R.tiles = o.tiles;
@@ -165,7 +165,8 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
     I.Tp1 = (float)(Tc + 1);
     I.min_pts = min_pts;
     I.leave = exact ? INT_MAX : min_pts;
-    // column tiles per work item: enough items (two a tile and chunk) to fill the
+    // column tiles per work item (2^19 tiles of 2,048 chunks at most: 32 bits hold
+    // two items each): enough items (two a tile and chunk) to fill the
     // chip some four times over, 8 to 256 tiles each
     int ch = 256;
     while (ch > 8 && 2 * (int64_t)nt * ((nt + ch - 1) / ch) < 16384) ch >>= 1;
@@ -185,17 +186,17 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
     launch_dependent(wt_pack_kernel, (nt + 7) / 8, 256, st, x, I, order, o, h, hdr, work, w.status);
     w.marks->kernel("wt_pack", st);
     const int grid = 152 * 3, tgrid = std::min((nt + 7) / 8, 152 * 8);
-    launch_dependent(pass_kernel<WT_COUNT>, grid, NT, st, R, hdr, ch, work);
+    launch_dependent(pass_kernel<WT_COUNT, false>, grid, NT, st, R, hdr, ch, nullptr, work);
     w.marks->kernel("wt_count", st);
     launch_dependent(core_kernel, std::min(tgrid, 152 * 3), NT, st, R, hdr);
     w.marks->kernel("wt_core", st);
-    launch_dependent(pass_kernel<WT_NEAR>, std::min((2 * nt + 7) / 8, grid), NT, st, R, hdr, ch, work + 1);
+    launch_dependent(pass_kernel<WT_NEAR, false>, std::min((2 * nt + 7) / 8, grid), NT, st, R, hdr, ch, nullptr, work + 1);
     w.marks->kernel("wt_union_near", st);
     launch_dependent(flatten_kernel, tgrid, NT, st, R, hdr);
     w.marks->kernel("wt_flatten", st);
-    launch_dependent(pass_kernel<WT_FAR>, grid, NT, st, R, hdr, ch, work + 2);
+    launch_dependent(pass_kernel<WT_FAR, false>, grid, NT, st, R, hdr, ch, nullptr, work + 2);
     w.marks->kernel("wt_union", st);
-    launch_dependent(pass_kernel<WT_BORDER>, grid, NT, st, R, hdr, ch, work + 3);
+    launch_dependent(pass_kernel<WT_BORDER, false>, grid, NT, st, R, hdr, ch, nullptr, work + 3);
     w.marks->kernel("wt_border", st);
     launch_dependent(root_kernel, std::min(nr / 64, 152 * 8), NT, st, R, hdr, o.least);
     w.marks->kernel("wt_root", st);

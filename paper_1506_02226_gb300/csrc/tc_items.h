@@ -5,10 +5,12 @@
 
 #include <cstdint>
 
+#ifndef DB_HD
 #ifdef __CUDACC__
 #define DB_HD __host__ __device__ __forceinline__
 #else
 #define DB_HD inline
+#endif
 #endif
 
 namespace tcitems {

@@ -37,6 +37,7 @@
 
 #include <climits>
 
+#include "batch_items.h"
 #include "internal.cuh"
 
 namespace wtile {
@@ -504,25 +505,28 @@ __device__ __forceinline__ void root_row(int *parent, int *least, bool is, int r
 
 // ---- the passes, as kernels ----
 
-// Work item w: half w mod 2 of tile (w / 2) mod total, the chunk (w / 2) / total
-// steps after the tile's own (wrapping around its instance), for one warp; the
-// next item is claimed while the current one runs.
-template <int PASS>
+// Work item w: half w mod 2 of tile T of some step, with the chunk `step` after
+// the tile's own (wrapping around its instance), for one warp; the next item is
+// claimed while the current one runs.  TABLE: first holds the tiles before each
+// step (batch_items.h); else all tiles have max_chunks chunks.
+template <int PASS, bool TABLE>
 static __global__ void __launch_bounds__(NT, 3) pass_kernel(Rows R, const Hdr *__restrict__ hdr, int ch_tiles,
-                                                     unsigned long long *work) {
+                                                     const unsigned *__restrict__ first, unsigned *work) {
     db::wait_prior_grid();  // returns at once when launched the plain way
     db::allow_next_grid();
-    const int total = hdr->total_tiles, lane = threadIdx.x & 31;
-    const unsigned long long nitems =
-        2ull * (unsigned long long)total * (PASS == WT_NEAR ? 1 : hdr->max_chunks);
-    unsigned long long next = 0;
-    if (lane == 0) next = atomicAdd(work, 1ull);
+    const int lane = threadIdx.x & 31;
+    const unsigned total = (unsigned)hdr->total_tiles, steps = PASS == WT_NEAR ? 1u : (unsigned)hdr->max_chunks;
+    const unsigned nitems = 2u * (TABLE && PASS != WT_NEAR ? first[steps] : total * steps);
+    int step = 0;
+    unsigned next = 0;
+    if (lane == 0) next = atomicAdd(work, 1u);
     while (true) {
-        const unsigned long long item = __shfl_sync(FULL, next, 0);
+        const unsigned item = __shfl_sync(FULL, next, 0);
         if (item >= nitems) return;
-        if (lane == 0) next = atomicAdd(work, 1ull);
-        const unsigned long long two = item >> 1;
-        const int step = (int)(two / (unsigned)total), T = (int)(two - (unsigned long long)step * total);
+        if (lane == 0) next = atomicAdd(work, 1u);
+        if (TABLE && PASS != WT_NEAR) step = batchitems::step_at(item >> 1, step, first);
+        else step = (int)((item >> 1) / total);
+        const int T = (int)((item >> 1) - (TABLE && PASS != WT_NEAR ? first[step] : (unsigned)step * total));
         const TileRec I = R.tiles[T];
         const int end = I.tile0 + I.ntiles;
         int ct0, ct1;
@@ -531,7 +535,6 @@ static __global__ void __launch_bounds__(NT, 3) pass_kernel(Rows R, const Hdr *_
             ct1 = min(end, T + 1 + kNear);
         } else {
             const int nchunk = (I.ntiles + ch_tiles - 1) / ch_tiles;
-            if (step >= nchunk) continue;
             int chunk = (T - I.tile0) / ch_tiles + step;
             if (chunk >= nchunk) chunk -= nchunk;
             ct0 = I.tile0 + chunk * ch_tiles;
