@@ -254,7 +254,9 @@ typedef struct dbscan_instance {
 /* Clusters `count` independent instances, each by Section I's three steps as
  * dbscan_run would (with the plan's label mode; the exact all-pairs
  * test of Sections IV-A/IV-B on ordered rows, 1 <= d <= 16, larger d gives
- * DBSCAN_ERR_UNSUPPORTED).  Batching many instances into one launch sequence
+ * DBSCAN_ERR_UNSUPPORTED).  A plan of DBSCAN_PREC_EXACT_SIMT takes the dot
+ * products in FP32 on the CUDA cores, any other in exact FP16 products on
+ * mma.sync; the labels are the same.  Batching many instances into one launch sequence
  * is this library's addition: the paper clusters one point set.  All instances run in one graph-captured launch
  * sequence of persistent kernels that share a work queue of (instance, row
  * tile, column chunk) items.  The first call autotunes the chunk size and grid

@@ -20,6 +20,8 @@
 // 46.6 / 4.5 ms a batch.  All passes are bound by the latency of an item's
 // first loads (record, rows, boxes) and then by the scores' FP32 operations, two
 // a pair; the matrix instructions are a few percent of the issue slots.
+// On a plan of DBSCAN_PREC_EXACT_SIMT the passes take their dot products on the
+// CUDA cores: 16.1 ms for the same batch (46.6 as 64 x 64 FP32 tiles).
 //
 // Autotuning: the column chunk per work item (CH) and the number of resident
 // blocks per SM are picked on the first call by timing every candidate on the
@@ -343,7 +345,25 @@ void build_table(const dbscan_instance *inst, int count, const batchitems::Queue
     *max_n = mx;
 }
 
-cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int bps, cudaStream_t st,
+// The pair passes and what lies between them.  SIMT: dot products on the CUDA
+// cores (DBSCAN_PREC_EXACT_SIMT).
+template <bool SIMT>
+void enqueue_passes(BatchState *b, const Rows &R, int ch, int pgrid, int egrid, cudaStream_t st, PhaseMarks &pm) {
+    pass_kernel<WT_COUNT, true, SIMT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 0);
+    pm.kernel(SIMT ? "batch_count_simt" : "batch_count", st);
+    core_kernel<SIMT><<<egrid, NT, 0, st>>>(R, b->d_hdr);
+    pm.kernel(SIMT ? "batch_core_simt" : "batch_core", st);
+    pass_kernel<WT_NEAR, true, SIMT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 1);
+    pm.kernel(SIMT ? "batch_union_near_simt" : "batch_union_near", st);
+    flatten_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
+    pm.kernel("batch_flatten", st);
+    pass_kernel<WT_FAR, true, SIMT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 2);
+    pm.kernel(SIMT ? "batch_union_simt" : "batch_union", st);
+    pass_kernel<WT_BORDER, true, SIMT><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 3);
+    pm.kernel(SIMT ? "batch_border_simt" : "batch_border", st);
+}
+
+cudaError_t enqueue_batch(BatchState *b, int label_mode, bool simt, bool stats, int ch, int bps, cudaStream_t st,
                           PhaseMarks *pm = nullptr) {
     PhaseMarks off;
     if (!pm) pm = &off;
@@ -363,18 +383,8 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
     batch_sortpack_kernel<<<sms * 3, 512, sort_bytes(b->sort_cap), st>>>(b->d_table, b->d_hdr, b->sort_cap, b->pack,
                                                                         b->d_status);
     pm->kernel("batch_prep", st);
-    pass_kernel<WT_COUNT, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 0);
-    pm->kernel("batch_count", st);
-    core_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
-    pm->kernel("batch_core", st);
-    pass_kernel<WT_NEAR, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 1);
-    pm->kernel("batch_union_near", st);
-    flatten_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr);
-    pm->kernel("batch_flatten", st);
-    pass_kernel<WT_FAR, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 2);
-    pm->kernel("batch_union", st);
-    pass_kernel<WT_BORDER, true><<<pgrid, NT, 0, st>>>(R, b->d_hdr, ch, b->d_first, b->d_work + 3);
-    pm->kernel("batch_border", st);
+    if (simt) enqueue_passes<true>(b, R, ch, pgrid, egrid, st, *pm);
+    else enqueue_passes<false>(b, R, ch, pgrid, egrid, st, *pm);
     root_kernel<<<egrid, NT, 0, st>>>(R, b->d_hdr, b->pack.least);
     pm->kernel("batch_root", st);
     const bool compact = label_mode == DBSCAN_LABEL_COMPACT;
@@ -400,7 +410,7 @@ cudaError_t enqueue_batch(BatchState *b, int label_mode, bool stats, int ch, int
 
 // The whole sequence as one CUDA graph (rebuilt when capacities or the tuned
 // configuration change).
-int batch_graph_launch(BatchState *b, int label_mode, bool stats, cudaStream_t st) {
+int batch_graph_launch(BatchState *b, int label_mode, bool simt, bool stats, cudaStream_t st) {
     if (!b->graph || b->graph_ch != b->ch || b->graph_bps != b->bps ||
         b->graph_stats != (int)stats || b->graph_ch < 0) {
         if (b->graph) {
@@ -411,7 +421,7 @@ int batch_graph_launch(BatchState *b, int label_mode, bool stats, cudaStream_t s
         if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return DBSCAN_ERR_CUDA;
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        if (!e) e = enqueue_batch(b, label_mode, stats, b->ch, b->bps, cs);
+        if (!e) e = enqueue_batch(b, label_mode, simt, stats, b->ch, b->bps, cs);
         cudaError_t e2 = cudaStreamEndCapture(cs, &g);
         cudaStreamDestroy(cs);
         if (e || e2 || !g) {
@@ -446,7 +456,7 @@ int batch_run(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, dbs
     if (!plan->batch) plan->batch = new BatchState();
     BatchState *b = plan->batch;
     const int label_mode = plan->opts.label_mode;
-    const bool stats = per_inst != nullptr;
+    const bool stats = per_inst != nullptr, simt = plan->opts.precision == DBSCAN_PREC_EXACT_SIMT;
     cudaStream_t st = plan->stream;
 
     std::vector<BInst> tmp(count);
@@ -489,7 +499,7 @@ int batch_run(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, dbs
                 float tbest = 1e30f;
                 for (int rep = 0; rep < 2; ++rep) {
                     cudaEventRecord(e0, st);
-                    if (enqueue_batch(b, label_mode, false, ch, bps, st)) {
+                    if (enqueue_batch(b, label_mode, simt, false, ch, bps, st)) {
                         cudaEventDestroy(e0);
                         cudaEventDestroy(e1);
                         return DBSCAN_ERR_CUDA;
@@ -513,9 +523,9 @@ int batch_run(dbscan_plan *plan, const dbscan_instance *inst, int32_t count, dbs
     prepare(b->ch);
     if (plan->opts.profile) {  // per-kernel events: run the sequence uncaptured
         plan->marks.begin(st);
-        if (enqueue_batch(b, label_mode, stats, b->ch, b->bps, st, &plan->marks)) return DBSCAN_ERR_CUDA;
+        if (enqueue_batch(b, label_mode, simt, stats, b->ch, b->bps, st, &plan->marks)) return DBSCAN_ERR_CUDA;
     } else {
-        s = batch_graph_launch(b, label_mode, stats, st);
+        s = batch_graph_launch(b, label_mode, simt, stats, st);
         if (s) return s;
     }
     if (cudaStreamSynchronize(st) != cudaSuccess) return DBSCAN_ERR_CUDA;

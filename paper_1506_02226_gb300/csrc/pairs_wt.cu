@@ -186,17 +186,17 @@ cudaError_t launch_allpairs_wt(const DbWork &w, const float *x, int64_t n64, int
     launch_dependent(wt_pack_kernel, (nt + 7) / 8, 256, st, x, I, order, o, h, hdr, work, w.status);
     w.marks->kernel("wt_pack", st);
     const int grid = 152 * 3, tgrid = std::min((nt + 7) / 8, 152 * 8);
-    launch_dependent(pass_kernel<WT_COUNT, false>, grid, NT, st, R, hdr, ch, nullptr, work);
+    launch_dependent(pass_kernel<WT_COUNT, false, false>, grid, NT, st, R, hdr, ch, nullptr, work);
     w.marks->kernel("wt_count", st);
-    launch_dependent(core_kernel, std::min(tgrid, 152 * 3), NT, st, R, hdr);
+    launch_dependent(core_kernel<false>, std::min(tgrid, 152 * 3), NT, st, R, hdr);
     w.marks->kernel("wt_core", st);
-    launch_dependent(pass_kernel<WT_NEAR, false>, std::min((2 * nt + 7) / 8, grid), NT, st, R, hdr, ch, nullptr, work + 1);
+    launch_dependent(pass_kernel<WT_NEAR, false, false>, std::min((2 * nt + 7) / 8, grid), NT, st, R, hdr, ch, nullptr, work + 1);
     w.marks->kernel("wt_union_near", st);
     launch_dependent(flatten_kernel, tgrid, NT, st, R, hdr);
     w.marks->kernel("wt_flatten", st);
-    launch_dependent(pass_kernel<WT_FAR, false>, grid, NT, st, R, hdr, ch, nullptr, work + 2);
+    launch_dependent(pass_kernel<WT_FAR, false, false>, grid, NT, st, R, hdr, ch, nullptr, work + 2);
     w.marks->kernel("wt_union", st);
-    launch_dependent(pass_kernel<WT_BORDER, false>, grid, NT, st, R, hdr, ch, nullptr, work + 3);
+    launch_dependent(pass_kernel<WT_BORDER, false, false>, grid, NT, st, R, hdr, ch, nullptr, work + 3);
     w.marks->kernel("wt_border", st);
     launch_dependent(root_kernel, std::min(nr / 64, 152 * 8), NT, st, R, hdr, o.least);
     w.marks->kernel("wt_root", st);

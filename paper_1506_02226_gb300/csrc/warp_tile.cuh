@@ -12,6 +12,7 @@
 // is exact, as in the scalar form (ap_tile.cuh).  (mma.sync and not tcgen05: a
 // work item here is a few 32 x 64 pair blocks of one small instance, and a
 // fragment in registers needs no staging, no barrier and no tensor memory.)
+// SIMT forms of the kernels take the same sums on the CUDA cores in FP32.
 //
 // Work.  A tile is 64 consecutive rows of one instance, in an order that puts
 // close rows next to each other; a work item is half a tile (32 rows, its
@@ -91,6 +92,40 @@ __device__ __forceinline__ void mma16(float (&c)[4], const unsigned (&a)[4], uin
         : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y), "f"(0.f), "f"(0.f), "f"(0.f), "f"(0.f));
 }
+// The same products on the CUDA cores, in FP32 (a batch whose plan asks for
+// DBSCAN_PREC_EXACT_SIMT): the fragments' units are fetched from the lanes that
+// hold them, four at a time for each of the lane's two rows and two columns.
+__device__ __forceinline__ void fma16(float (&c)[4], const unsigned (&a)[4], uint2 b) {
+    const int lane = threadIdx.x & 31;
+    auto f2 = [](unsigned v) { return __half22float2(*reinterpret_cast<const __half2 *>(&v)); };
+    c[0] = c[1] = c[2] = c[3] = 0.f;
+#pragma unroll 1  // unrolled, the rows' units of a whole tile are held at once and spill (a kilobyte in the count)
+    for (int k = 0; k < 4; ++k) {
+        float2 p[4], q[4];  // units 2k, 2k+1 of the rows, then 2k+8, 2k+9; the same of the columns
+#pragma unroll
+        for (int i = 0; i < 4; ++i) p[i] = f2(__shfl_sync(FULL, a[i], (lane & 28) + k));
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            q[e] = f2(__shfl_sync(FULL, b.x, 8 * (lane & 3) + 4 * e + k));
+            q[2 + e] = f2(__shfl_sync(FULL, b.y, 8 * (lane & 3) + 4 * e + k));
+        }
+#pragma unroll
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float &s = c[2 * r + e];
+                s = fmaf(p[r].x, q[e].x, s);
+                s = fmaf(p[r].y, q[e].y, s);
+                s = fmaf(p[2 + r].x, q[2 + e].x, s);
+                s = fmaf(p[2 + r].y, q[2 + e].y, s);
+            }
+    }
+}
+template <bool SIMT>
+__device__ __forceinline__ void dot16(float (&c)[4], const unsigned (&a)[4], uint2 b) {
+    if constexpr (SIMT) fma16(c, a, b);
+    else mma16(c, a, b);
+}
 // Operand fragment of the 16 rows from `row`.
 __device__ __forceinline__ void load_rows16(const uint2 *P16, int row, unsigned (&a)[4]) {
     const int lane = threadIdx.x & 31;
@@ -134,7 +169,7 @@ static __device__ __noinline__ int unite_sets(int *parent, int x, int y, unsigne
 
 // The state of one work item's 32 rows.  Lane l holds rows l/4 + 8 i, i < 4,
 // of columns 2 (l mod 4) and the next in every group of 8.
-template <int PASS>
+template <int PASS, bool SIMT>
 struct Item {
     unsigned a[2][4];             // operand fragments
     float an[4];                  // T + 1 - |p|^2, or -1e30 for a row the pass has no use for
@@ -166,7 +201,7 @@ struct Item {
 #pragma unroll
                 for (int m = 0; m < 2; ++m) {
                     float c[4];
-                    mma16(c, a[m], b[g]);
+                    dot16<SIMT>(c, a[m], b[g]);
 #pragma unroll
                     for (int k = 0; k < 2; ++k) {
                         const int i = 2 * m + k;
@@ -256,7 +291,7 @@ __device__ __forceinline__ float box_gap2(const Rows &R, int s, int t, int d) {
 
 // One work item: rows [64 T + 32 half, + 32) against column tiles [ct0, ct1) of
 // the batch.  Called by whole warps.
-template <int PASS>
+template <int PASS, bool SIMT>
 __device__ __forceinline__ void run_item(const Rows &R, const TileRec &I, int T, int half, int ct0, int ct1) {
     const int lane = threadIdx.x & 31;
     const int mytag = PASS == WT_COUNT ? kMixed : R.tag[T];
@@ -264,7 +299,7 @@ __device__ __forceinline__ void run_item(const Rows &R, const TileRec &I, int T,
     if (PASS == WT_BORDER && !R.need[T]) return;
     const int left = I.n - ((T - I.tile0) * BT + 32 * half);  // rows of the instance from this half on
     if (left <= 0) return;
-    Item<PASS> it;
+    Item<PASS, SIMT> it;
     it.row0 = T * BT + 32 * half;
     load_rows16(R.P16, it.row0, it.a[0]);
     load_rows16(R.P16, it.row0 + 16, it.a[1]);
@@ -353,6 +388,7 @@ __device__ __forceinline__ void run_item(const Rows &R, const TileRec &I, int T,
 // shared memory: no global atomics), and what follows: the masked norms, the
 // tile's tag and whether some row needs the border pass.  A warp per tile, two
 // rows a lane; adj and lab are the warp's own.
+template <bool SIMT>
 __device__ __forceinline__ void core_tile(const Rows &R, const TileRec &I, int T, unsigned long long *adj, int *lab) {
     const int lane = threadIdx.x & 31, r0 = (T - I.tile0) * BT;
     bool is[2], need[2];
@@ -395,7 +431,7 @@ __device__ __forceinline__ void core_tile(const Rows &R, const TileRec &I, int T
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 float c[4];
-                mma16(c, a[m], b);
+                dot16<SIMT>(c, a[m], b);
 #pragma unroll
                 for (int k = 0; k < 2; ++k) {
                     const unsigned e0 = fmaf(2.f, c[2 * k], b0) + an[2 * m + k] >= 1.f;
@@ -509,7 +545,7 @@ __device__ __forceinline__ void root_row(int *parent, int *least, bool is, int r
 // the tile's own (wrapping around its instance), for one warp; the next item is
 // claimed while the current one runs.  TABLE: first holds the tiles before each
 // step (batch_items.h); else all tiles have max_chunks chunks.
-template <int PASS, bool TABLE>
+template <int PASS, bool TABLE, bool SIMT>
 static __global__ void __launch_bounds__(NT, 3) pass_kernel(Rows R, const Hdr *__restrict__ hdr, int ch_tiles,
                                                      const unsigned *__restrict__ first, unsigned *work) {
     db::wait_prior_grid();  // returns at once when launched the plain way
@@ -541,10 +577,11 @@ static __global__ void __launch_bounds__(NT, 3) pass_kernel(Rows R, const Hdr *_
             ct1 = min(end, ct0 + ch_tiles);
             if (PASS == WT_FAR) ct0 = max(ct0, T + 1 + kNear);
         }
-        if (ct0 < ct1) run_item<PASS>(R, I, T, (int)(item & 1), ct0, ct1);
+        if (ct0 < ct1) run_item<PASS, SIMT>(R, I, T, (int)(item & 1), ct0, ct1);
     }
 }
 
+template <bool SIMT>
 static __global__ void __launch_bounds__(NT, 3) core_kernel(Rows R, const Hdr *__restrict__ hdr) {
     db::wait_prior_grid();
     db::allow_next_grid();
@@ -552,7 +589,7 @@ static __global__ void __launch_bounds__(NT, 3) core_kernel(Rows R, const Hdr *_
     __shared__ int lab[NT / 32][BT];
     const int total = hdr->total_tiles, nwarps = (int)((gridDim.x * blockDim.x) >> 5), wib = threadIdx.x >> 5;
     for (int T = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); T < total; T += nwarps)
-        core_tile(R, R.tiles[T], T, adj[wib], lab[wib]);
+        core_tile<SIMT>(R, R.tiles[T], T, adj[wib], lab[wib]);
 }
 
 static __global__ void __launch_bounds__(NT) flatten_kernel(Rows R, const Hdr *__restrict__ hdr) {
