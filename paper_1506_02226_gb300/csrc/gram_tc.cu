@@ -1243,10 +1243,8 @@ __global__ void __launch_bounds__(Shape<PASS, BF16>::THREADS, 1) tc_pass_kernel(
                             if (j >= 0 && lane == leader) {
                                 const int q = ct * TN + j;
                                 rt = unite_sets(a.parent, rootp, hq, a.status);
-                                if (rt >= 0) {
-                                    if (q != rt) db::st_relaxed(a.parent + q, rt);
-                                    if (p != rt && rt != rootp) db::st_relaxed(a.parent + p, rt);
-                                }
+                                if (q != rt) db::st_relaxed(a.parent + q, rt);
+                                if (p != rt && rt != rootp) db::st_relaxed(a.parent + p, rt);
                             }
                             rt = __shfl_sync(FULL, rt, leader);
                             if (j >= 0) {

@@ -441,10 +441,9 @@ __global__ void __launch_bounds__(256) mid_union_kernel(MidArgs a, const uint8_t
                         int r = 0;
                         if (lane == src) {
                             r = db::uf_unite_root(parent, h, hq, status);
-                            if (r >= 0) db::st_relaxed(hint + q, r);
+                            db::st_relaxed(hint + q, r);
                         }
                         r = __shfl_sync(FULL, r, src);
-                        if (r < 0) r = hq;
                         if (hm == h || hm == hq) hm = r;
 #pragma unroll
                         for (int u = 0; u < 4; ++u) {

@@ -48,60 +48,11 @@ __device__ __forceinline__ void st_relaxed(int *p, int v) {
     asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// ---------------------------------------------------------------------------
-// Lock-free union-find over point indices (replaces the paper's per-target
-// merge kernel of Section IV-C).  Invariant: parent[x] <= x, and a root is the
-// smallest index of its set, because union always links the larger root under
-// the smaller one.  Path halving writes only ancestors, so concurrent halving
-// and linking keep the invariant.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ int uf_find(int *parent, int x) {
-    while (true) {
-        int p = ld_relaxed(parent + x);
-        if (p == x) return x;
-        int gp = ld_relaxed(parent + p);
-        if (gp == p) return p;
-        st_relaxed(parent + x, gp);
-        x = gp;
-    }
-}
+}  // namespace db
 
-// Union of the sets of a and b.  Each failed CAS means another thread linked
-// the root first, so the loop makes global progress; the cap only guards
-// against a corrupted forest and reports it.
-__device__ __forceinline__ void uf_unite(int *parent, int a, int b, unsigned *status) {
-    for (int it = 0; it < (1 << 24); ++it) {
-        a = uf_find(parent, a);
-        b = uf_find(parent, b);
-        if (a == b) return;
-        if (a > b) {
-            int t = a;
-            a = b;
-            b = t;
-        }
-        if (atomicCAS(parent + b, b, a) == b) return;
-    }
-    atomicOr(status, DB_EBIT_TIMEOUT);
-}
+#include "union_find.cuh"
 
-// Union that also returns a root of the merged set (a hint for callers that
-// cache it: the value is the set's root at some moment, so any point whose
-// parent equals it is in the set).
-__device__ __forceinline__ int uf_unite_root(int *parent, int a, int b, unsigned *status) {
-    for (int it = 0; it < (1 << 24); ++it) {
-        a = uf_find(parent, a);
-        b = uf_find(parent, b);
-        if (a == b) return a;
-        if (a > b) {
-            int t = a;
-            a = b;
-            b = t;
-        }
-        if (atomicCAS(parent + b, b, a) == b) return a;
-    }
-    atomicOr(status, DB_EBIT_TIMEOUT);
-    return -1;
-}
+namespace db {
 
 // Cell hash slot of the grid paths: four consecutive keys (four cells in a
 // row along x) share one 32-byte bucket of the packed table, so the lookups of
