@@ -1764,11 +1764,7 @@ __global__ void __launch_bounds__(256) tc_root_kernel(int n, const uint8_t *__re
     db::allow_next_grid();
     const int p = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31;
     const bool is = p < n && core[p];
-    int root = -1 - lane;
-    if (is) {
-        root = db::uf_find(parent, p);
-        if (root != p) db::st_relaxed(parent + p, root);
-    }
+    const int root = is ? db::uf_settle(parent, p) : -1 - lane;
     // one atomic per distinct root of the warp, and none that cannot lower the value
     const unsigned peers = __match_any_sync(FULL, root);
     if (is) {

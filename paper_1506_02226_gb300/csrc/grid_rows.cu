@@ -757,11 +757,7 @@ __global__ void __launch_bounds__(256) rows_root_kernel(RowArgs a) {
     const int ncells = (int)(*a.ctr0 >> 32), step = (int)(gridDim.x * blockDim.x), lane = threadIdx.x & 31;
     for (int c0 = (int)(blockIdx.x * blockDim.x); c0 < ncells; c0 += step) {
         const int c = c0 + (int)threadIdx.x, rep = c < ncells ? a.rep[c] : DB_NONE;
-        int root = -1 - lane;
-        if (rep != DB_NONE) {
-            root = db::uf_find(a.par, c);
-            if (root != c) db::st_relaxed(a.par + c, root);
-        }
+        const int root = rep != DB_NONE ? db::uf_settle(a.par, c) : -1 - lane;
         // one atomic per distinct root of the warp, and none that cannot lower the value
         const unsigned peers = __match_any_sync(FULL, root);
         if (rep != DB_NONE) {

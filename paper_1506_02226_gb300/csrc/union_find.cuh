@@ -27,6 +27,20 @@ __device__ __forceinline__ int uf_find(int *parent, int x) {
     }
 }
 
+// Root of x, and x straight under it, for the kernels that leave the forest flat
+// (each node settled by a thread of its own, no set joined meanwhile): behind
+// such a kernel every settled node's parent is its root, and labels are read
+// through it.  Nothing else is written on the way: another thread's uf_find that
+// read x's old ancestors would halve the path at x after x has its root, and
+// leave an ancestor there that is not one (its points' label is then that of no
+// set; 500,000 points in the plane were seen with four such).
+__device__ __forceinline__ int uf_settle(int *parent, int x) {
+    int r = x;
+    for (int p = ld_relaxed(parent + r); p != r; p = ld_relaxed(parent + r)) r = p;
+    if (r != x) st_relaxed(parent + x, r);
+    return r;
+}
+
 // Union of the sets of a and b.  Each failed CAS means another thread linked
 // the root first, so the loop makes global progress; the cap only guards
 // against a corrupted forest and reports it.

@@ -527,11 +527,7 @@ __device__ __forceinline__ void flatten_tile(const Rows &R, int T) {
 // of the warp calls it.
 __device__ __forceinline__ void root_row(int *parent, int *least, bool is, int row, int point) {
     const int lane = threadIdx.x & 31;
-    int root = -1 - lane;
-    if (is) {
-        root = db::uf_find(parent, row);
-        if (root != row) db::st_relaxed(parent + row, root);
-    }
+    const int root = is ? db::uf_settle(parent, row) : -1 - lane;
     const unsigned peers = __match_any_sync(FULL, root);
     if (is) {
         const int m = __reduce_min_sync(peers, point);

@@ -61,11 +61,66 @@ int main() {
 """
 
 
-def test_union_find(tmp_path):
+SETTLE = r"""
+#include <cstdio>
+#include <vector>
+#define __device__
+#define __forceinline__ inline
+#define DB_EBIT_TIMEOUT 2u
+static void step();  // before every access of the forest
+namespace db {
+inline int ld_relaxed(const int *p) { step(); return *p; }
+inline void st_relaxed(int *p, int v) { step(); *p = v; }
+}
+inline int atomicCAS(int *p, int, int v) { const int old = *p; *p = v; return old; }
+inline void atomicOr(unsigned *p, unsigned v) { *p |= v; }
+#include "union_find.cuh"
+static std::vector<int> parent, others;  // others: settled, whole, in one thread's way
+static int countdown = -1;
+static void step() {
+    if (countdown < 0 || countdown-- > 0) return;
+    for (int v : others) db::uf_settle(parent.data(), v);
+    others.clear();
+}
+int main() {
+    const int n = 9;
+    for (int fan = 0; fan < 2; ++fan)               // a chain, or a binary tree
+        for (int x = 0; x < n; ++x)                 // the thread that is held up,
+            for (int at = 0; at < 2 * n; ++at)      // before which of its accesses,
+                for (int mask = 0; mask < (1 << n); ++mask) {  // while which others run
+                    parent.assign(n, 0);
+                    for (int i = 1; i < n; ++i) parent[i] = fan ? (i - 1) / 2 : i - 1;
+                    others.clear();
+                    for (int v = 0; v < n; ++v)
+                        if (v != x && (mask >> v & 1)) others.push_back(v);
+                    countdown = at;
+                    if (db::uf_settle(parent.data(), x) != 0) return 1;
+                    countdown = -1;
+                    for (int v : others) db::uf_settle(parent.data(), v);  // (x was done before)
+                    for (int v = 0; v < n; ++v)
+                        if (v != x && !(mask >> v & 1)) db::uf_settle(parent.data(), v);
+                    for (int v = 0; v < n; ++v)
+                        if (parent[v] != 0) return 2;
+                }
+    return 0;
+}
+"""
+
+def run(tmp_path, text):
     if shutil.which("g++") is None:
         pytest.skip("no C++ compiler")
-    (tmp_path / "uf.cpp").write_text(PROGRAM)
+    (tmp_path / "uf.cpp").write_text(text)
     r = subprocess.run(["g++", "-std=c++17", "-O1", "-Wall", "-Werror", "-I", CSRC, str(tmp_path / "uf.cpp"), "-o",
                         str(tmp_path / "uf")], capture_output=True, text=True)
     assert r.returncode == 0, r.stderr
-    assert subprocess.run([str(tmp_path / "uf")]).returncode == 0
+    return subprocess.run([str(tmp_path / "uf")]).returncode
+
+
+def test_union_find(tmp_path):
+    assert run(tmp_path, PROGRAM) == 0
+
+
+def test_settled_nodes_stay_under_their_root(tmp_path):
+    """Whatever settles in a thread's way, every node is straight under its root
+    once its own thread is done: labels are read through the parents."""
+    assert run(tmp_path, SETTLE) == 0
