@@ -34,25 +34,44 @@ struct Carver {
     }
 };
 
+// The most points an all-pairs run takes: its work items (row tiles x column
+// chunks) are counted in int32.
+constexpr int64_t kAllPairsMaxN = int64_t(1) << 25;
+
 // Lays the workspace out (base == nullptr: just measures it).  exact_d: o.max_d
 // is the only dimension served (a plan's is an upper bound).
+// A run takes one path, and no path reads what another run left, so arrays of
+// different paths share memory: the warp tiles' with the grids' and the tensor
+// cores' (where there are none, with the CUDA-core path's rows), the key-ordered
+// cells' ranks with what only grid.cu and the projected grid use.
 size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
     Carver c{base};
     const int64_t n = std::max<int64_t>(o.max_n, 1);
     w.cap_n = n;
     w.cap_d = o.max_d;
     w.dp_cap = dp_for(std::min(o.max_d, 64));
-    w.P = c.take<float>((size_t)n * w.dp_cap);
-    w.count = c.take<int32_t>(n);
-    w.core = c.take<uint8_t>(n);
-    w.parent = c.take<int32_t>(n);
+    const bool grid = o.grid != DBSCAN_GRID_OFF && o.max_d >= 1;
+    auto take_rows = [&] {
+        w.P = c.take<float>((size_t)n * w.dp_cap);
+        w.count = c.take<int32_t>(n);
+        w.core = c.take<uint8_t>(n);
+        w.parent = c.take<int32_t>(n);
+    };
+    const bool rows_last = !grid && o.max_d < 16;
+    if (!rows_last) take_rows();
     w.border = c.take<int32_t>(n);
     w.scan = c.take<int32_t>(n + 1);
     w.scan_part_cap = n / 2048 + 4;
     w.scan_part = c.take<int32_t>(w.scan_part_cap);
     w.status = c.take<unsigned>(4);
     w.ctr = c.take<unsigned long long>(DB_NCTR);
-    const bool grid = o.grid != DBSCAN_GRID_OFF && o.max_d >= 1;
+    // warp tiles: all-pairs runs of d <= 16, none at d <= 3 with a grid (the eps-grid always applies there)
+    const bool wt = o.precision == DBSCAN_PREC_AUTO && (!grid || o.max_d > 3) && !(exact_d && o.max_d > 16);
+    const size_t shared_from = c.off;
+    w.wt = wt ? c.take<char>(wt_bytes(std::min(n, kAllPairsMaxN))) : nullptr;
+    const size_t wt_end = c.off;
+    c.off = shared_from;
+    if (rows_last) take_rows();
     w.rk = nullptr;
     if (grid) {
         int bits = 10;
@@ -61,8 +80,18 @@ size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
         w.hbits = bits;
         w.hcount = c.take<int32_t>(w.hcap);  // right behind status and ctr: one clear covers all three
         w.hkey = c.take<uint32_t>(w.hcap);
+        const int dg = std::min(o.max_d, 3);
+        const size_t rk_from = c.off;
         w.hpack = c.take<int2>(w.hcap);
+        w.cell_count = c.take<int32_t>(n);
         w.occ_cap = std::max<int64_t>(int64_t(1) << 15, 4 * n);
+        if (n > kGridSmallMaxN && (dg == o.max_d || !exact_d)) {  // grid_rows.cu's
+            const size_t others_end = c.off;
+            c.off = rk_from;
+            w.rk = c.take<uint2>(w.occ_cap);
+            c.off = std::max(c.off, others_end);
+            w.rg_part = c.take<unsigned long long>(std::max(w.hcap, w.occ_cap) / 2048 + 8);
+        }
         w.occ = c.take<uint32_t>(w.occ_cap);
         w.hcursor = c.take<int32_t>(w.hcap);
         w.slot_of = c.take<int32_t>(n);
@@ -72,19 +101,13 @@ size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
         w.scell = c.take<int32_t>(n);
         w.score = c.take<uint8_t>(n);
         w.cell_start = c.take<int32_t>(n);
-        w.cell_count = c.take<int32_t>(n);
         w.cell_rep = c.take<int32_t>(n);
         w.cell_mid = c.take<float4>(n);
         w.cell_key = c.take<uint32_t>(n);
-        const int dg = std::min(o.max_d, 3);
         w.noff_cap = dg == 1 ? 8 : (dg == 2 ? 24 : 124);
         w.nbr = c.take<int32_t>((size_t)n * w.noff_cap);
         w.ncnt = c.take<int32_t>(n);
         w.cell_cand = c.take<int32_t>(n);
-        if (n > kGridSmallMaxN && (dg == o.max_d || !exact_d)) {  // grid_rows.cu's
-            w.rk = c.take<uint2>(w.occ_cap);
-            w.rg_part = c.take<unsigned long long>(std::max(w.hcap, w.occ_cap) / 2048 + 8);
-        }
     } else {
         w.hcap = 0;
         w.noff_cap = 0;
@@ -109,15 +132,12 @@ size_t layout(DbWork &w, const dbscan_opts &o, bool exact_d, char *base) {
         w.tc_udone = c.take<int32_t>(2 * nt);
         w.tc_cbeta = c.take<float>(2 * nt);
         w.tc_crad = c.take<float>(2 * nt);
-        const int64_t ntp = std::min<int64_t>(nt, (int64_t(1) << 17) + 1);  // all-pairs runs take up to 2^25 points
+        const int64_t ntp = std::min<int64_t>(nt, kAllPairsMaxN / 256 + 1);
         w.tc_pairs = c.take<uint32_t>((size_t)ntp * ((ntp + 31) / 32));
     } else {
         w.tc_cap_pad = 0;
     }
-    // warp tiles: all-pairs runs of d <= 16, none at d <= 3 with a grid (the eps-grid always applies there)
-    const bool wt = o.precision == DBSCAN_PREC_AUTO && (!grid || o.max_d > 3) && !(exact_d && o.max_d > 16);
-    w.wt = wt ? c.take<char>(wt_bytes(n)) : nullptr;
-    return align_up(c.off, 256);
+    return align_up(std::max(c.off, wt_end), 256);
 }
 
 }  // namespace
@@ -175,9 +195,8 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     const int64_t T = (int64_t)std::floor(e * e * 1048576.0);  // exact: 48-bit square, power-of-two scale
     if (stats) stats->threshold = T;
     if (n == 0) return DBSCAN_OK;
-    // Index ranges counted in int32: the eps-grid's hash (at least 2n slots)
-    // and the all-pairs work items (row tiles x column chunks).
-    constexpr int64_t kGridMaxN = int64_t(1) << 29, kAllPairsMaxN = int64_t(1) << 25;
+    // the eps-grid's hash (at least 2n slots) is counted in int32
+    constexpr int64_t kGridMaxN = int64_t(1) << 29;
     const bool grid_path = d <= 8 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0;
     if (grid_path ? n > kGridMaxN : n > kAllPairsMaxN) return DBSCAN_ERR_UNSUPPORTED;
     const int64_t Dmax = (int64_t)d * 1023 * 1023;
