@@ -228,16 +228,20 @@ int dbscan_plan_counters(dbscan_plan *plan, uint64_t *out, int32_t n);
 /* Device bytes the plan's workspace holds. */
 int64_t dbscan_plan_workspace_bytes(const dbscan_plan *plan);
 
-/* Failure-detection test hook (the paper has none).  DBSCAN_HOOK_TC_STALL
+/* Test hooks (the paper has none), consumed by the plan's next run that each
+ * applies to.  DBSCAN_HOOK_GRID_GENERAL makes an eps-grid run (d <= 3) take the
+ * kernels that serve any size, which otherwise only very large inputs and cells
+ * far smaller than the data's extent reach; the results are the same.
+ * DBSCAN_HOOK_TC_STALL
  * makes the plan's next run that takes the tensor-core path issue no MMA in
  * its counting pass: every bounded device-side wait of that pass then expires
  * (50 ms budget instead of about 2 s), the CTAs take their abort path (wait
  * for their own copies, free tensor memory, return), and the run returns
- * DBSCAN_ERR_TIMEOUT with unspecified labels.  The hook is consumed by that
- * run; the plan stays usable.  No GPU fault, trap or hang is involved.
+ * DBSCAN_ERR_TIMEOUT with unspecified labels; the plan stays usable.  No GPU fault, trap or hang is involved.
  * Returns DBSCAN_ERR_ARG for a null plan or an unknown hook. */
 #define DBSCAN_HOOK_NONE 0
 #define DBSCAN_HOOK_TC_STALL 1
+#define DBSCAN_HOOK_GRID_GENERAL 2
 int dbscan_plan_test_hook(dbscan_plan *plan, int32_t hook);
 
 /* ---- Batched form: many independent instances in one graph-captured launch sequence ---- */

@@ -32,7 +32,7 @@ DBSCAN_LABEL_ROOT_INDEX, DBSCAN_LABEL_COMPACT = 0, 1
 DBSCAN_PATH_NONE, DBSCAN_PATH_GRID, DBSCAN_PATH_ALLPAIRS_SIMT, DBSCAN_PATH_ALLPAIRS_TC = 0, 1, 2, 3
 DBSCAN_PATH_GRID_PROJECTED, DBSCAN_PATH_PAPER = 4, 5
 DBSCAN_PAPER_MAX_N = 65536
-DBSCAN_HOOK_NONE, DBSCAN_HOOK_TC_STALL = 0, 1
+DBSCAN_HOOK_NONE, DBSCAN_HOOK_TC_STALL, DBSCAN_HOOK_GRID_GENERAL = 0, 1, 2
 
 c_i32, c_i64, c_f32, c_p = ctypes.c_int32, ctypes.c_int64, ctypes.c_float, ctypes.c_void_p
 

@@ -208,8 +208,11 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
     const bool want_grid = d <= 3 && o.grid != DBSCAN_GRID_OFF && plan->w.hcap > 0;
     GridGeom g;
     const bool eps_grid = want_grid && grid_geometry(d, Tc, n, &g);
+    const bool general = eps_grid && plan->test_hook == DBSCAN_HOOK_GRID_GENERAL;
+    if (general) plan->test_hook = DBSCAN_HOOK_NONE;  // consumed by this run
     // these clear what they need themselves
-    const bool small = eps_grid && n <= kGridSmallMaxN, rows = eps_grid && !small && grid_rows_serves(plan->w, g, n);
+    const bool small = eps_grid && !general && n <= kGridSmallMaxN;
+    const bool rows = eps_grid && !general && !small && grid_rows_serves(plan->w, g, n);
     const bool clears = small || rows;
     const bool reported = o.synchronous && (!eps_grid || clears);  // by every path but grid.cu's
     plan->w.status_out = reported ? plan->h_status : nullptr;
@@ -249,7 +252,7 @@ int plan_run(dbscan_plan *plan, const float *points, int64_t n, int32_t d, float
         if (want_tc && tc_ok) {
             path = DBSCAN_PATH_ALLPAIRS_TC;
             const bool stall = plan->test_hook == DBSCAN_HOOK_TC_STALL;
-            plan->test_hook = DBSCAN_HOOK_NONE;  // consumed by this run
+            if (stall) plan->test_hook = DBSCAN_HOOK_NONE;  // consumed by this run
             err = launch_allpairs_tc(plan->w, points, n, d, Tc, min_pts, exact, o.precision == DBSCAN_PREC_BF16_GRAM,
                                      stall, labels, counts_out, core_out, st);
         } else if (d <= 16 && o.precision == DBSCAN_PREC_AUTO && plan->w.wt) {
@@ -543,7 +546,7 @@ int dbscan_plan_counters(dbscan_plan *plan, uint64_t *out, int32_t n) {
 }
 
 int dbscan_plan_test_hook(dbscan_plan *plan, int32_t hook) {
-    if (!plan || hook < DBSCAN_HOOK_NONE || hook > DBSCAN_HOOK_TC_STALL) return DBSCAN_ERR_ARG;
+    if (!plan || hook < DBSCAN_HOOK_NONE || hook > DBSCAN_HOOK_GRID_GENERAL) return DBSCAN_ERR_ARG;
     plan->test_hook = hook;
     return DBSCAN_OK;
 }
