@@ -144,7 +144,7 @@ __global__ void mid_scatter_kernel(const float *__restrict__ x, int n, int d, co
 // Work items (cell, first point of the chunk), in no particular order beyond the
 // 32 cells of a warp, which take their places at one go; *nitems counts them.
 // (One launch where a count, a scan of three and a fill were five; with the
-// path's other launches made dependent, 50,021 x 5: 337 us a call, now 310.)
+// path's other launches made dependent, 50,001 x 5: 337 us a call, now 310.)
 __global__ void mid_chunk_table_kernel(const unsigned long long *ctr0, const int *__restrict__ cell_count,
                                        int2 *__restrict__ items, int *nitems) {
     db::wait_prior_grid();  // started as a programmatic dependent

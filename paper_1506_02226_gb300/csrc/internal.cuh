@@ -201,7 +201,7 @@ struct DbWork {
     int32_t *ncnt;          // (adjacent count << 16) | count [cap_n]
     int32_t *cell_cand;     // points in the cells of each neighbour list [cap_n]
     int32_t noff_cap;
-    uint2 *rk;              // cells in key order: per 32 cells {occupied cells before, bits} [occ_cap]
+    uint2 *rk;              // cells in key order: per 32 cells {occupied cells before, bits} [occ_cap] (over hpack and on)
     unsigned long long *rg_part;  // block totals of its scans
     // tensor-core path (max_d >= 16)
     int64_t tc_cap_pad;     // rows of each packed operand (cap_n rounded up to 256, plus 256)
@@ -215,7 +215,7 @@ struct DbWork {
     int32_t *tc_tag, *tc_rowneed, *tc_udone;  // per tile: common root of its core points, border rows; per unit
     float *tc_cbeta, *tc_crad;  // per ball (two a tile): |c|^2 of its centre, largest squared distance to it
     uint32_t *tc_pairs;     // tile pairs that may hold neighbours (bits) [tiles][ceil(tiles / 32)]
-    void *wt;               // warp-tile path (d <= 16 all pairs): its arrays, wt_bytes(cap_n) (null: not served)
+    void *wt;               // warp-tile path (d <= 16 all pairs): its arrays, over other paths' (null: not served)
     PhaseMarks *marks;      // host-side timing marks of the owning plan
     // second stream of the grid path: independent kernels run beside each
     // other (fork/join by events); unused while per-kernel marks are taken
