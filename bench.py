@@ -174,10 +174,10 @@ def grid_offsets(d: int, T: int):
 # source means the counters no longer describe the kernel, and the bench line
 # reports traffic null.
 NCU_TRAFFIC = {
-    ("lowd2", "grid_count"): (17999872, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
-    ("lowd2", "grid_union_near"): (11558656, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
-    ("lowd3", "grid_count"): (43691776, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
-    ("lowd3", "grid_union_near"): (57448704, "paper_1506_02226_gb300/csrc/grid_rows.cu", "2247da0a3cf1"),
+    ("lowd2", "grid_count"): (17992960, "paper_1506_02226_gb300/csrc/grid_rows.cu", "d885e835e521"),
+    ("lowd2", "grid_union_near"): (11562240, "paper_1506_02226_gb300/csrc/grid_rows.cu", "d885e835e521"),
+    ("lowd3", "grid_count"): (43673856, "paper_1506_02226_gb300/csrc/grid_rows.cu", "d885e835e521"),
+    ("lowd3", "grid_union_near"): (57534208, "paper_1506_02226_gb300/csrc/grid_rows.cu", "d885e835e521"),
 }
 
 

@@ -12,12 +12,12 @@
 // compaction) is captured once into a CUDA graph; a batch is then one table
 // upload and one graph launch.
 //
-// Measured, 4,096 instances of 64 to 8,192 points, d in {2, 3, 16} (us; with
-// 64 x 64 FP32 tiles a block, before / after): prep 1,874 / 630 (scattered row
-// reads, the counting sort), count 10,030 / 785, core flags and the merge inside
-// tiles - / 341, the merge across tiles 30,161 / 1,450 (pairs of tiles that hold
-// several sets or none of whose pairs are neighbours), border 4,556 / 890;
-// 46.6 / 4.5 ms a batch.  All passes are bound by the latency of an item's
+// Measured, 4,096 instances of 64 to 8,192 points, d in {2, 3, 16} (us, kernels
+// one by one; with 64 x 64 FP32 tiles a block, before / after): prep 1,874 / 604
+// (scattered row reads, the counting sort), count 10,030 / 912, core flags and
+// the merge inside tiles - / 349, the merge across tiles 30,161 / 1,344 (pairs of
+// tiles that hold several sets or none of whose pairs are neighbours), border
+// 4,556 / 852; 46.6 / 4.1 ms a batch.  All passes are bound by the latency of an item's
 // first loads (record, rows, boxes) and then by the scores' FP32 operations, two
 // a pair; the matrix instructions are a few percent of the issue slots.
 // On a plan of DBSCAN_PREC_EXACT_SIMT the passes take their dot products on the
