@@ -577,14 +577,18 @@ extern "C" int dbscan_batch(dbscan_plan *plan, const dbscan_instance *inst, int3
         items += rows * ((cols + 3) / 4);
     }
     if (items > INT32_MAX) return DBSCAN_ERR_UNSUPPORTED;
-    // Rows are counted in int32: a batch of very many tiles runs in parts.
+    // Rows are counted in int32: a batch of very many tiles runs in parts.  An
+    // off-grid instance fails the call, not the instances of the other parts.
+    int status = DBSCAN_OK;
     unsigned long long tot[4] = {0, 0, 0, 0};
     for (int32_t i = 0; i < count;) {
         const int32_t end = batchitems::part_end(i, count, [&](int32_t k) { return inst[k].n; });
         const int s = batch_run(plan, inst + i, end - i, per_inst ? per_inst + i : nullptr, tot);
-        if (s) return s;
+        if (s && s != DBSCAN_ERR_NOT_QUANTISED) return s;
+        if (!status) status = s;
         i = end;
     }
+    if (status) return status;
     // the batch's pair tests per pass, also left in the plan's counters 16..18
     if (per_inst && cudaMemcpy(plan->w.ctr + DB_CTR_EVAL, tot, sizeof(tot), cudaMemcpyHostToDevice) != cudaSuccess)
         return DBSCAN_ERR_CUDA;

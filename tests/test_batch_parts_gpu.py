@@ -35,6 +35,16 @@ def test_more_than_a_part():
     st = (B.dbscan_stats * count)()
     with Plan(max_n=16, max_d=2) as p:
         assert B.dbscan_batch(p.handle, insts, st) == B.DBSCAN_OK
+        # an off-grid instance in the first part: the call fails, the other parts' labels are as before
+        good = labels.clone()
+        bad = torch.full((3, 2), 0.3, device="cuda")
+        t["points"][0] = bad.data_ptr()
+        labels.fill_(-9)
+        assert B.dbscan_batch(p.handle, insts) == B.DBSCAN_ERR_NOT_QUANTISED
+        assert torch.equal(labels[-1000:], good[-1000:])
+        t["points"][0] = x.data_ptr() + 8 * at[0]
+        labels.fill_(-9)
+        assert B.dbscan_batch(p.handle, insts) == B.DBSCAN_OK and torch.equal(labels, good)
     whole = np.concatenate(want)
     reps = -(-count // len(pool))
     np.testing.assert_array_equal(labels.cpu().numpy(), np.tile(whole, reps)[:len(labels)])
